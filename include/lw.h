@@ -136,38 +136,28 @@ lw_status lw_wait(lw_ctx *ctx);
 /*
  * lw_get_stats -- counters of the last completed run, written to the host
  * array `stats` (first `count` entries; entries past the last counter are 0):
- *   [0] rounds (each certifies one or more consecutive merges between two
- *       grid barriers),
- *   [1] rounds that certified no merge (waiting for a row refill),
+ *   [0] rounds (each takes one or more consecutive merges),
+ *   [1] rounds that took no merge (waiting for a row refill),
  *   [2] cells rewritten by the update formula (sum over merges of m_t - 2),
  *   [3] CTAs of the persistent grid,
  *   [4] row refills served by all CTAs together,
  *   [5] live cells read by those refills,
  *   [6] refills installed by the rows' owners,
- *   [7] published entries the walks visited (all rounds),
+ *   [7] entries that the rounds selected their members from,
  *   [8..13] with LW_OPT_PHASE_TIMES on: wall-clock nanoseconds summed over
- *       the CTAs of the grid, per phase of a round: [8] barrier waits,
- *       [9] exchange, walk, refill installs and scans, [10] pass 1 (new cells, read
- *       only), [11] the cells after two merges, computed in the window of
- *       the second barrier, [12] certification and bookkeeping, [13] pass 2
- *       (writes, cache upkeep) and publish;
+ *       the CTAs of the grid, per phase of a round: [8] waits at the main
+ *       barrier, [9] from the records to the round's merges, [10] the
+ *       step from there to the new cells, [11] the wait for every CTA's
+ *       gather, [12] 0, [13] new cells, cache upkeep and publish;
  *   [14] rows rescanned at once by their owner (cache emptied),
  *   [15] live cells read by those rescans,
- *   [16..25] with LW_OPT_PHASE_TIMES on, a finer split of [9], [11], [12]
- *       and [13] (same units): [16] reading the CTAs' records, [17] the
- *       walk with the refill installs and scans beside it, [18] the
- *       chain's sizes, stamps and member
- *       cells, [19] the cross-CTA minima of the new cells, [20] the
- *       certification, [21] bookkeeping and survivor caches, [22] pass 2,
- *       [23] owner rescans; refill scans in the row-log layout: [24] the
- *       log part, [25] the matrix part; [26] the walk alone (part of [17]);
- *   [27..32] with LW_OPT_PHASE_TIMES on, the barriers' own cost: [27] the
- *       waits (ns) of the CTA that arrived last, summed over the barriers
- *       of the loop, [28] those barriers (as counted by the CTAs that
- *       completed them), [29] of them the second barrier of a round, [30]
- *       second barriers completed by a CTA serving a refill that round,
- *       [31] first barriers completed by such a CTA, [32] barriers
- *       completed by CTA 0.
+ *   [16..25] with LW_OPT_PHASE_TIMES on, a finer split of [9] and [13] (same
+ *       units): [16] survivors' lists and installs, [17] the selection, [18]
+ *       the cells between members, [19] the round's merges, [20] the new
+ *       cells, [21] reading the CTAs' records, [22] logs, lists and caches,
+ *       [23] owner rescans; refill scans in the row-log layout: [25] all of
+ *       the scan ([24], [26]: 0);
+ *   [27..32] 0.
  */
 lw_status lw_get_stats(lw_ctx *ctx, int64_t *stats, int count);
 

@@ -192,31 +192,14 @@ struct BusyGuard {
     }
 };
 
-int choose_grid(lw_ctx *ctx, long long n)
+int choose_grid(lw_ctx *ctx, long long n, int linkage)
 {
-    int G = ctx->grid_opt > 0 ? ctx->grid_opt : 0;
-    if (G == 0) {
-        // small matrices: one CTA (no grid barrier); larger: every SM
-        G = n <= 4096 ? 1 : ctx->num_sms;
-    }
+    int G = ctx->grid_opt > 0 ? ctx->grid_opt : lw::default_grid(n, linkage, ctx->num_sms);
     if (G > ctx->num_sms)
         G = ctx->num_sms;
     const long long nb = (n + lw::kRowBlock - 1) / lw::kRowBlock;
     if (G > nb)
         G = (int)nb;
-    if (ctx->grid_opt <= 0 && G > 1) {
-        // as few CTAs as give the same most row blocks per CTA, when that
-        // saves a tenth of them or more: the walk, the exchange and the
-        // barriers cost less while the slowest CTA's share of the rows stays
-        // the same (n = 16384: 128 CTAs of 4 blocks instead of 152 of 3 or
-        // 4, 2.4 % faster).  A smaller saving is not taken: CTAs with a block
-        // fewer take the refill scans (n = 65536: 147 CTAs of 14 blocks ran
-        // 0.3 % slower than 152 of 13 or 14).
-        const long long per = (nb + G - 1) / G;
-        const int G2 = (int)((nb + per - 1) / per);
-        if (10LL * G2 <= 9LL * G)
-            G = G2;
-    }
     const int nt = ctx->cta_threads;
     while (G < ctx->num_sms && !lw::merge_config_ok(n, G, ctx->num_sms, nt))
         ++G;  // too much shared memory per CTA: spread the rows wider
@@ -233,7 +216,7 @@ int choose_grid(lw_ctx *ctx, long long n)
 lw_status enqueue(lw_ctx *ctx, float *ddist, long long n, int linkage, int32_t *dmerges,
                   float *dheights, bool host_src = false, bool *declined = nullptr)
 {
-    const int G = choose_grid(ctx, n);
+    const int G = choose_grid(ctx, n, linkage);
     if (G <= 0) {
         set_err(ctx, "n=%lld does not fit a co-resident grid on this device", n);
         return LW_ERR_INVALID_ARG;
@@ -852,7 +835,7 @@ lw_status lw_batch_create(lw_ctx *ctx, const lw_job *jobs, int32_t njobs, lw_bat
     }
     if (st == LW_OK && !b->big_idx.empty()) {
         // size the context's workspace now so that runs never allocate
-        const int G = choose_grid(ctx, big_n);
+        const int G = choose_grid(ctx, big_n, LW_COMPLETE);
         if (G <= 0) {
             set_err(ctx, "n=%lld does not fit a co-resident grid on this device", big_n);
             st = LW_ERR_INVALID_ARG;

@@ -12,11 +12,24 @@ namespace lw {
 constexpr int kThreads = 512;            // default threads per CTA of the merge kernel
 constexpr int kRowBlock = 32;            // rows per ownership block (one warp)
 constexpr int kCacheKeys = 4;            // smallest keys cached per row
-constexpr int kPub = 4;                  // entries a CTA of a multi-CTA grid publishes per round
-constexpr int kPubOne = 16;              // entries a job's only CTA publishes per round
-constexpr int kRound = 32;               // most merges one round of a multi-CTA grid certifies
-constexpr int kRoundOne = 16;            // the same for a job's only CTA
-constexpr int kRefillAt = 0;             // ask for a refill when the cache holds this many keys or fewer
+constexpr int kPub = 8;                  // entries a CTA of a multi-CTA grid publishes per round
+constexpr int kTeam = 64;                // most members (clusters) of a round
+constexpr int kSurv = 32;                // most merged clusters a round leaves
+constexpr int kEntries = 64;             // most entries a round selects its members from
+constexpr int kCand = 512;               // most entries up to a round's pivot
+constexpr int kHeadsHi = 64;             // most lists whose heads the pivot takes in
+constexpr int kPieces = 4;               // most pieces a refill row is scanned in
+constexpr int kPartWords = 8;            // words of a piece: its smallest keys, the bound of the others
+constexpr int kSvList = 64;             // listed new cells per survivor
+constexpr int kRankBits = 4;             // an entry's rank in its row
+constexpr unsigned kRankMask = 15u;
+constexpr int kBar2 = 32;                // words of the second and third barrier counter and of
+constexpr int kBar3 = 48;                // the first conditional merge that must wait (two, by
+constexpr int kViol = 8;                 // round parity; kSurv less it, 0: none)
+constexpr int kRedoBelow = 16;           // a chain cut below this many merges, and below half its
+constexpr int kRedoGap = 4;              // length (and a bit), is walked step by step instead
+constexpr int kTieGain = 3;              // merges a round must gain to take them on condition
+constexpr long long kRefillEarlyN = 24576;  // up to this n a row asks for a refill at one key left, above it at none
 constexpr int kSurvivorRefillAt = 1;     // the same for a survivor row right after its merge
 constexpr int kMaxReq = 256;             // refill requests served per round
 constexpr int kReqPerCta = 8;            // refill requests one CTA may make per round
@@ -41,18 +54,20 @@ struct CheckRange {
     unsigned long long bytes;
 };
 
-// One CTA's record at the start of a round, 240 bytes: its smallest cache
-// entries (kPub of them, kPubOne for a one-CTA job; key = (bits(value) << 32)
-// | (row << 3) | rank, column word beside it) and the rows (at most
-// kReqPerCta) that ask for a refill.
+// One CTA's record at the start of a round: its kPub smallest cache entries
+// (key = (bits(value) << 32) | (row << kRankBits) | rank, column word beside
+// it), the rows (at most kReqPerCta) that ask for a refill and, in the first
+// round, the largest value of its rows.  Two sets, by round parity: a CTA may
+// write the next round's while another still reads this one's.
 struct __align__(16) RecA {
-    unsigned long long key[kPubOne];
-    unsigned int col[kPubOne];
+    unsigned long long key[kPub];
+    unsigned int col[kPub];
     int nreq;
     int req[kReqPerCta];
-    int pad[3];
+    unsigned dmax;
+    int pad[2];
 };
-static_assert(sizeof(RecA) == 240, "record layout");
+static_assert(sizeof(RecA) == kPub * 12 + 48, "record layout");
 
 struct MergeParams {
     float *D;                      // working matrix, rewritten in place: the packed
@@ -75,10 +90,13 @@ struct MergeParams {
     int32_t *merges;               // [2(n-1)] device
     float *heights;                // [n-1]    device
     int *size_g;                   // [n] cluster sizes
-    RecA *recA;                    // [G] published entries and refill requests
-    unsigned long long *recB;      // [G][2][kRound] per-pair minima of the new cells
-    unsigned long long *parts;     // [2][kMaxReq][kCacheKeys] refill lists (top-K of a row)
-    unsigned int *bar;             // grid barrier counter (zero at launch)
+    int chunk;                     // rows per chunk of the apply pass (set at launch)
+    RecA *recA;                    // [2][G] published entries and refill requests
+    int *svcnt;                    // [2][kSurv] new cells of a survivor below the limit,
+    unsigned long long *svovf;     // the least of them that is not listed [2][kSurv],
+    unsigned long long *svlist;    // and the listed ones [2][kSurv][kSvList], by round parity
+    unsigned long long *parts;     // [2][kMaxReq][kPieces][kPartWords] refill lists (top-K of a row's pieces)
+    unsigned int *bar;             // grid barrier counters, words 0 and kBar2 (zero at launch)
     int *status;                   // [4] status word [0]; barrier that gave up [1]
     long long *stats;              // [kStats] counters, see lw_get_stats
     unsigned long long timeout_ns; // bound of every device wait
@@ -110,7 +128,7 @@ __host__ __device__ inline void check_range(MergeParams &p, const void *base, un
 // block (every part 256-byte aligned).  The words from `zero` to `total`
 // (barrier, status, stats) must be zero at launch.
 struct WorkspaceLayout {
-    size_t size, recA, recB, parts, zero, bar, status, stats, total;
+    size_t size, recA, sv, parts, zero, bar, status, stats, total;
 };
 
 __host__ __device__ inline WorkspaceLayout workspace_layout(long long n, int G)
@@ -119,9 +137,9 @@ __host__ __device__ inline WorkspaceLayout workspace_layout(long long n, int G)
     WorkspaceLayout L;
     size_t off = 0;
     L.size = off;   off = up(off + sizeof(int) * (size_t)n);
-    L.recA = off;   off = up(off + sizeof(RecA) * (size_t)G);
-    L.recB = off;   off = up(off + 8 * 2 * kRound * (size_t)G);
-    L.parts = off;  off = up(off + 8 * kCacheKeys * (size_t)kMaxReq * 2);
+    L.recA = off;   off = up(off + sizeof(RecA) * 2 * (size_t)G);
+    L.sv = off;     off = up(off + 2 * kSurv * (size_t)(16 + 8 * kSvList));
+    L.parts = off;  off = up(off + 8 * kPartWords * (size_t)kMaxReq * kPieces * 2);
     L.zero = off;
     L.bar = off;    off = up(off + 256);
     L.status = off; off = up(off + 4 * sizeof(int));
@@ -135,7 +153,9 @@ __host__ __device__ inline void bind_workspace(MergeParams &p, char *ws, const W
 {
     p.size_g = reinterpret_cast<int *>(ws + L.size);
     p.recA = reinterpret_cast<RecA *>(ws + L.recA);
-    p.recB = reinterpret_cast<unsigned long long *>(ws + L.recB);
+    p.svlist = reinterpret_cast<unsigned long long *>(ws + L.sv);
+    p.svovf = p.svlist + 2 * kSurv * kSvList;
+    p.svcnt = reinterpret_cast<int *>(p.svovf + 2 * kSurv);
     p.parts = reinterpret_cast<unsigned long long *>(ws + L.parts);
     p.bar = reinterpret_cast<unsigned int *>(ws + L.bar);
     p.status = reinterpret_cast<int *>(ws + L.status);
@@ -164,6 +184,7 @@ struct BatchParams {
     int *job_status;               // [njobs] lw_status of each job
     long long *merges_done;        // total merges performed (optional)
     unsigned long long timeout_ns;
+    int chunk;                     // rows per chunk of the apply pass (set at launch)
 };
 
 // Writes the symmetric n x n matrix `full` (row-major, rows `pitch` words
@@ -177,7 +198,10 @@ inline long long log_pitch(long long n) { return (n + 3) & ~3LL; }
 
 // Bytes of dynamic shared memory the merge kernel needs for (n, G) with CTAs
 // of nt threads.
+int default_grid(long long n, int linkage, int num_sms);
 size_t merge_smem_bytes(long long n, int G, int nt);
+// Rows per chunk of the apply pass (its new cells are kept in shared memory).
+int merge_chunk_rows(long long n, int G, int nt);
 // CTA sizes the kernels are built for: 128, 256 or 512 threads (4, 2 or 1
 // CTAs per SM by registers).
 // True if a grid of G CTAs of nt threads for n objects fits co-resident on

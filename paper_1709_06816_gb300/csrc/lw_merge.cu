@@ -16,42 +16,64 @@
 // every live cell of the row outside the cache has a key above B (B = "none"
 // when the cache holds every live cell of the row).
 //
-// Rounds.  A grid barrier costs about a microsecond on GB300, more than the
-// arithmetic of one merge, so the kernel certifies several consecutive merges
-// of the sequential iteration per pair of barriers (up to 32 for a grid, 16
-// for a job's only CTA).  The merges are exactly those of the step-by-step
-// algorithm (same pairs, same order, same rounded values); only the
-// bookkeeping differs.  One round:
+// Rounds.  A grid barrier costs about a microsecond on GB300, and a merge by
+// itself less, so a round takes as many consecutive merges of the sequential
+// iteration as it can prove from one exchange (up to 32).  The merges are
+// exactly those of the step-by-step algorithm (same pairs, same order, same
+// rounded values); only the bookkeeping differs.  One round:
 //
-//   A  every CTA publishes its smallest cache entries (kPub of them, kPubOne
-//      for a job's only CTA), each row's entries followed by a stop mark at
-//      its bound B.  After the barrier every CTA walks the union of all
-//      published entries in (value, row, column) order and proposes a chain
-//      of disjoint pairs P_1..P_s: an entry whose row or column already
-//      belongs to a proposed pair is skipped, a stop mark of an untouched row
-//      (or the last entry of a CTA that had more) ends the walk.  P_{p+1} is
-//      then the smallest cell among those no earlier proposal touches.
-//   pass 1 (reads only): for every live k outside the chain and every pair a,
-//      the new distance D(k, i_a + j_a) of Section 4 step 3; each CTA
-//      publishes, per pair, its smallest new cell over all k and over k > i_a.
-//      The cells between members of two proposed pairs are computed by every
-//      CTA, in the order the sequential algorithm would write them.
-//   B  after the barrier, every CTA finds the longest prefix P_1..P_L such
-//      that each P_{p+1} is smaller than every cell the merges P_1..P_p have
-//      rewritten: then P_{p+1} is the global minimum after merge p, so the
-//      prefix is what the sequential algorithm does.  P_1 always qualifies.
-//   pass 2: the L merges are emitted and applied: D(k, i_a) rewritten, caches
-//      kept (column j_a leaves, the new cell (k, i_a) enters when <= B), the
-//      survivor rows get their new caches from the published minima.
+//   publish  every CTA publishes its kPub smallest entries: cached keys of its
+//      rows, and at the end of a row's list a mark at its bound B.  (A job's
+//      only CTA uses its caches directly.)  Barrier 1.
+//   selection  every CTA reads all entries, takes the smallest in (value, row,
+//      column) order, and makes the rows and columns they name the round's
+//      members (at most kTeam): until the next entry would be one member too
+//      many, or is a mark of a row without a member, or the last one of a CTA
+//      that may have more.  Every cell between live slots that is not among the
+//      entries taken is at or above the first entry not taken, TH, or, in a
+//      member's row that ended in a mark, at or above that mark.
+//   gather  every CTA reads all cells between members; an arrival at barrier 2
+//      says that it has.
+//   merges  every CTA works out the same merges from those cells: while the
+//      smallest cell between members lies below TH, below the marks and below
+//      every cell that a merged cluster can have to a slot outside (a lower
+//      bound from the operands' bounds), it is the smallest of all, so it is
+//      the sequential algorithm's next merge.  Complete, average, weighted and
+//      Ward linkage mostly merge disjoint entries: those are taken in one go
+//      and the limits checked side by side (the chain); where cells made by the
+//      round's own merges cut it short, and for single and centroid linkage,
+//      one warp takes the merges step by step.
+//   on condition  the bounds for outside cells may end a chain that the cells
+//      themselves would not (many equal values).  When that costs kTieGain
+//      merges or more, the merges are taken on condition: the new cells are
+//      computed and kept back, every CTA looks whether one of its own comes
+//      before a merge of the round, and barrier 3 tells which merges stand.
+//   apply  behind barrier 2 (no CTA still reads the members' old cells): the new
+//      cells D(k, survivor) for every live k, a warp per 32 rows and up to 8
+//      survivors, all loads of an item in flight at once; then logs, caches
+//      (merged columns leave, new cells at or below B enter) and the
+//      survivors' lists: their new cells below a limit go to lists in global
+//      memory that every CTA reads after the next barrier 1.
 //
-// Refills.  A row whose cache empties (a survivor row: right after its merge)
-// asks for a refill; in the window of the next round's barrier B (after a CTA
-// has arrived and before it waits) one CTA scans the whole row, all threads,
-// and publishes its top-K; at the start of the round after that the owner
-// takes the list and replays the merges of the round in between.  A row that
-// empties while its bound sits at the front of the merges is rescanned at
-// once by its owner.  A job's only CTA sees every write after pass 2 and
-// refreshes survivor and emptied rows itself, a warp per row.
+// Refills.  A row whose cache is down to one key (n <= kRefillEarlyN: rows are
+// short and rounds are what costs) or empty asks for a refill.  In the next
+// round the upper half of the warps of each CTA (team B) scans the rows, cut
+// in pieces, beside the lower half's (team A's) gather and merges, and then
+// joins the apply; for longer rows it starts before the selection.  At the
+// start of the round after that the owner takes the list, dropping the columns
+// merged meanwhile and replaying the new cells.  A row that empties while its
+// bound sits at the front of the merges is rescanned at once by its owner.  A
+// job's only CTA refreshes emptied rows itself, a warp per row.
+//
+// What bounds it.  A round is a chain of latencies: about 40 us at n = 16384 of
+// which 3 are barrier 1, 6 the selection, 7 the gather and the chain's operands,
+// 5 the merges, 7 the new cells, 6 caches and lists; the memory traffic of a
+// round (some 10 MB) would take under 2 us.  So what counts is merges per
+// round.  Certifying a walk of disjoint entries after the new cells' minima
+// were exchanged (two full barriers and about 13 merges per round) took 46.1 ms for
+// n = 16384 average linkage, 162.8 ms for single and 16.8 ms for n = 1968
+// (complete, one CTA then); selecting up to 64 members by a threshold and
+// merging inside them takes 28.8, 62.4 and 2.7 ms.
 //
 // Exact arithmetic: every product and sum of the update uses __fmul_rn /
 // __fadd_rn / __fsub_rn (never contracted into FMA), the coefficient
@@ -68,6 +90,7 @@
 // with acquire loads.  Each spin is bounded by a wall-clock limit after which
 // the kernel records LW_ERR_TIMEOUT and returns.
 
+#include "../../include/lw.h"
 #include "lw_internal.h"
 
 #include <cstdint>
@@ -108,13 +131,13 @@ __device__ __forceinline__ void st_checked(const MergeParams &p, T *a, typename 
     if (check_ok(p, a, sizeof(T), line))
         __stcg(a, v);
 }
+#define CHECK_PREFETCH(a) check_ok(p, (a), 4, __LINE__)
 #define LDCG(a) ld_checked(p, (a), __LINE__)
 #define STCG(a, v) st_checked(p, (a), (v), __LINE__)
-#define CHECKED_16(a) check_ok(p, (a), 16, __LINE__)
 #else
+#define CHECK_PREFETCH(a) true
 #define LDCG(a) __ldcg(a)
 #define STCG(a, v) __stcg((a), (v))
-#define CHECKED_16(a) true
 #endif
 
 __device__ __forceinline__ long long tri_off(long long r, long long n)
@@ -169,26 +192,10 @@ __device__ __forceinline__ void red_release_add(unsigned *p, unsigned v)
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ unsigned atom_release_add(unsigned *p, unsigned v)
+// Brings the line of an address into L2.
+__device__ __forceinline__ void prefetch_l2(const void *a)
 {
-    unsigned old;
-    asm volatile("atom.release.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
-}
-
-// 16 bytes global -> shared, cached in L2 only (the words read are written by
-// other CTAs between grid barriers, so L1 must not hold them).  The copy
-// writes no register: a warp that issues one per step does not wait for the
-// previous one.
-__device__ __forceinline__ void copy16_async(void *dst_smem, const void *src_gmem)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src_gmem) : "memory");
-}
-
-__device__ __forceinline__ void copy_async_wait_all()
-{
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
 }
 
 __device__ __forceinline__ u64 global_ns()
@@ -209,24 +216,14 @@ __device__ __forceinline__ void cswap(u64 &a, u64 &b)
     a = lo;
 }
 
-// Insert x into the K smallest: a compare-swap pass; the largest falls off.
-__device__ __forceinline__ void list_insert(u64 (&L)[K], u64 x)
+// Insert x into the K smallest: a compare-swap pass; the largest falls off
+// (and is returned).
+__device__ __forceinline__ u64 list_insert(u64 (&L)[K], u64 x)
 {
 #pragma unroll
     for (int q = 0; q < K; ++q)
         cswap(L[q], x);
-}
-
-// Re-sort a sorted list in which at most two entries were replaced by kNoKey:
-// two bubble passes carry both holes to the end.
-__device__ __forceinline__ void close_holes(u64 (&L)[K])
-{
-#pragma unroll
-    for (int pass = 0; pass < 2; ++pass) {
-#pragma unroll
-        for (int q = 0; q + 1 < K; ++q)
-            cswap(L[q], L[q + 1]);
-    }
+    return x;
 }
 
 __device__ __forceinline__ int list_count(const u64 *L)
@@ -265,6 +262,16 @@ __device__ __forceinline__ void warp_topk(u64 (&L)[KK], u64 (&out)[KK])
     }
 }
 
+// warp_topk over lists that may have dropped keys above their last one, and
+// `next`, a lower bound of every key not in out: the next listed one, or just
+// above the last key of a full list whose keys are all in out.
+__device__ __forceinline__ void warp_topk_next(u64 (&L)[K], u64 (&out)[K], u64 &next)
+{
+    const u64 end = L[K - 1] == kNoKey ? kNoKey : L[K - 1] + 1;
+    warp_topk(L, out);
+    next = warp_u64_min(L[0] != kNoKey ? L[0] : end);
+}
+
 // Insert x into a sorted list of KK keys; the largest falls off.
 template <int KK>
 __device__ __forceinline__ void list_insert_n(u64 (&L)[KK], u64 x)
@@ -274,27 +281,11 @@ __device__ __forceinline__ void list_insert_n(u64 (&L)[KK], u64 x)
         cswap(L[q], x);
 }
 
-// Candidate of the global minimum: (value, row) and column.
-struct Cand {
-    u64 A;       // (bits(v) << 32) | row
-    unsigned c;  // column
-};
-
-__device__ __forceinline__ void cand_min(Cand &x, const Cand &y)
-{
-    if (y.A < x.A || (y.A == x.A && y.c < x.c))
-        x = y;
-}
-
-// Most merges one round certifies: a one-CTA job publishes kPubOne entries
-// and walks at most kRoundOne pairs; a grid walks up to kRound.
-__host__ __device__ constexpr int round_of(int pub) { return pub == kPubOne ? kRoundOne : kRound; }
 constexpr unsigned kFull = 0xffffffffu;
 constexpr u64 kHi = 0xffffffff00000000ull;
-static_assert(kPub <= kPubOne && kPub % 4 == 0 && kPubOne % 4 == 0, "record layout");
 static_assert(K == 4, "sort_list is a 4-input network");
-static_assert(kRound <= 32 && (32 % kRound) == 0 && (32 % kRoundOne) == 0,
-              "certification and pair minima use lane groups of the round size");
+static_assert(kPub % 4 == 0 && kPub >= K, "record layout");
+static_assert(kTeam == 64, "a warp's lanes hold two members each; masks of 64 bits");
 
 // Sort a K-list in which any entries were replaced by kNoKey.
 __device__ __forceinline__ void sort_list(u64 (&L)[K])
@@ -306,91 +297,127 @@ __device__ __forceinline__ void sort_list(u64 (&L)[K])
     cswap(L[1], L[2]);
 }
 
-// The update of Section 4 step 3 with the Table 1 coefficients for clusters
-// of sizes ni, nj (merged) and nk (the other one); terms added in printed
-// order, every operation rounded once.
-__device__ __forceinline__ float lw_cell(int linkage, float dki, float dkj, float dij, int ni, int nj,
-                                         int nk)
+// The update of Section 4 step 3 from coefficients: the four terms (bh is the
+// third) added in printed order, every operation rounded once.
+__device__ __forceinline__ float lw_sum(float ai, float aj, float bh, float ga, float dki, float dkj)
 {
-    float ai = 0.5f, aj = 0.5f, be = 0.0f, ga = 0.0f;
-    if (linkage == 0) {
-        ga = -0.5f;
-    } else if (linkage == 1) {
-        ga = 0.5f;
-    } else if (linkage == 2 || linkage == 5) {
-        // group average; centroid adds beta = -n_i n_j / (n_i + n_j)^2 (exact
-        // integers, each converted to float once, one division)
-        const float sum = (float)(ni + nj);
-        ai = __fdiv_rn((float)ni, sum);
-        aj = __fdiv_rn((float)nj, sum);
-        if (linkage == 5)
-            be = -__fdiv_rn(__ll2float_rn((long long)ni * nj),
-                            __ll2float_rn((long long)(ni + nj) * (ni + nj)));
-    } else if (linkage == 3) {
-        const float T = (float)(ni + nj + nk);
-        ai = __fdiv_rn((float)(ni + nk), T);
-        aj = __fdiv_rn((float)(nj + nk), T);
-        be = -__fdiv_rn((float)nk, T);
-    }
-    // linkage 4, weighted average: 1/2, 1/2, 0, 0
     float s = __fmul_rn(ai, dki);
     s = __fadd_rn(s, __fmul_rn(aj, dkj));
-    s = __fadd_rn(s, __fmul_rn(be, dij));
-    s = __fadd_rn(s, __fmul_rn(ga, fabsf(__fsub_rn(dki, dkj))));
-    return s;
+    s = __fadd_rn(s, bh);
+    return __fadd_rn(s, __fmul_rn(ga, fabsf(__fsub_rn(dki, dkj))));
 }
 
-// Order key of the cell between clusters x and y holding value bits vb.
-__device__ __forceinline__ Cand cell_cand(unsigned vb, unsigned x, unsigned y)
-{
-    Cand c;
-    c.A = ((u64)vb << 32) | (x < y ? x : y);
-    c.c = x < y ? y : x;
-    return c;
-}
+// A round's members and merges (static shared memory).
+struct Team {
+    // the members (slots in ascending order), size and bound of the cells
+    // outside (value bits), stamp, row base; every cell not between two members
+    // is above (thA, thC) = (value << 32 | row, column), or above the member's
+    // own bound (lbA, lbC) where a row's cached keys end below that
+    int m;
+    unsigned thC, thv;
+    u64 thA;
+    unsigned dmax;               // largest input value (bits)
+    int mem[kTeam], mst[kTeam];
+    int2 sl[kTeam];
+    long long mbase[kTeam];      // cell (slot, c) at mbase + c
+    u64 lbA[kTeam];
+    unsigned lbC[kTeam];
+    float S[kTeam][kTeam + 1];   // cells between members
+    unsigned nnv[kTeam], nnc[kTeam];
+    u64 mask[kTeam];
+    // the entries in key order: members i | j << 8 (0xffff: a bound mark) and
+    // value bits; per member the entries it takes part in
+    uint2 ent[kEntries];
+    u64 em[kTeam];
+    int ne;
+    int sz0[kTeam];              // sizes before the round
+    // the chain: per entry the entries that share a member with it, per member
+    // its merge (0xff: none), the cells merge q makes with every member, those
+    // between survivors after the round, and the least cell before each merge
+    uint2 enm[kEntries];
+    unsigned char step[kEntries];
+    unsigned char ce[kSurv];     // entry of merge q
+    unsigned char ex[kTeam];     // entry that ends a member's row (0xff: none)
+    int tie;                     // the merges wait for a look at the cells outside
+    int redo;                    // the chain broke off early: step by step instead
+    float X[kSurv][kTeam + 1];
+    float C[kSurv][kSurv + 1];
+    unsigned lim[kSurv];
+    // the round's merges in order: members i | j << 8 and, in the upper half,
+    // the merge that made each operand (q + 1; 0: a cell in memory), height
+    // bits, sizes; coefficients (a_i, a_j, b times the height, g; not Ward)
+    int L;
+    int4 rec[kTeam];
+    float4 co[kTeam];
+    int res[kTeam];
+    // the merged clusters still live after the round: the merges that lead to
+    // each in order (prog[sfirst[s] .. sfirst[s + 1])), the last of them, slot
+    int ns;
+    int prog[kTeam], root[kTeam], sfirst[kSurv + 1], sq[kSurv], sslot[kSurv];
+    u64 tT[kSurv][K], tB[kSurv]; // smallest keys of the survivor's cells to other survivors
+    __device__ int mi(int q) const { return rec[q].x & 0xff; }
+    __device__ int mj(int q) const { return (rec[q].x >> 8) & 0xff; }
+};
 
-template <int NT, int S>
+// Static shared memory of a CTA.  ONE: the CTA is its job's only one (no
+// records, no refill requests).
+template <int NT, bool ONE>
 struct Shared {
     static constexpr int W = NT / 32;
-    u64 tk[W][kPubOne];
-    u64 tko[kPubOne];
+    u64 tk[W][kPub];
+    u64 tko[kPub], tnext, tnx[W];
     int wcnt[W];
+    u64 wmin[W][2];
     int flag;
     int nexec;                   // refill rows served this round
     int exec_row[kMaxReq];
     int nmyreq[2];               // this CTA's requests, by round parity
     int myreq_l[2][kReqPerCta];
-    int ninst;                   // refills to install at the start of the next round
+    int npieces;                 // pieces per row of the refills served last
+    int ninst;                   // refills to install in this round
     int inst_slot[kReqPerCta];
-    // the round's chain of proposed merges and the cells between its members
-    int np, nacc;
-    unsigned front;              // value bits where this round's walk stopped
-    int okp[S];
-    int pi[S], pj[S];
-    float ph[S];
-    int szi[S], szj[S];
-    long long bi[S], bj[S];      // row bases of the members: cell (x, c) at b + c
-    int si[S], sj[S];            // row-log layout: the members' stamps before the round
-    // the 16-byte words holding size_g[i_a], size_g[j_a], stamp[i_a], stamp[j_a]
-    alignas(16) int qw[S][16];
-    u64 wam[W][S], whm[W][S];    // per warp: smallest new cell per pair (all k, k > i)
-    u64 gamin[S], ghmin[S];      // the same over all CTAs
-    // (rows padded by one word: the certification reads a column of these
-    // per warp, one row per lane, which would otherwise hit a single bank)
-    alignas(16) float Dm[2 * S][2 * S + 1];  // D between members (2a = i_a, 2a + 1 = j_a)
-    float X[S][S + 1];           // cell (i_a, i_b) after merge a alone
-    float Y[S][S + 1];           // cell (i_a, j_b) after merge a alone
-    float C[S][S + 1];           // cell (i_a, i_b) after merges a then b (a < b)
-    // the previous round's merges, replayed on installed refills
-    int ppi[S], ppj[S];
-    int nprev;
+    // candidate entries of the round (unordered), the first kEntries of them in
+    // key order, and which of those bring a new row (1) or column (2) or end
+    // the selection (4)
+    int ncand;
+    u64 ckey[kCand];
+    unsigned ccol[kCand];
+    u64 ekey[kEntries + 1];
+    uint2 erc[kEntries + 1];     // row, column word
+    unsigned char enew[kEntries];
+    int umem[kTeam];
+    Team tm;
+    // the previous round's survivors and their caches
+    int nps;
+    int pslot[kSurv];
+    u64 svk[kSurv][K], svB[kSurv];
+    int svc[kSurv];
+    int nptouch;                 // slots the previous round touched
+    int ptouch[kTeam];
+    unsigned okm[NT / 32];       // rows of the chunk that take the round's merges
     int nresc;                   // rows to rescan at once this round
+    int item, viol;              // apply pass: next item, first merge that must wait
+    unsigned limit, width;       // see the selection
+    int svsum;                   // entries of the previous round's survivors' lists
+    u64 ppivot;                  // the last round's pivot of the published entries
+    u64 pivot;                   // the last round's pivot of the entry selection
+    // the job's arrays in dynamic shared memory (see merge_job) and its row split,
+    // for the functions kept out of line (the round loop holds as many registers
+    // as a CTA may have: inline, they would spill)
+    struct {
+        unsigned *bitmap, *touched, *wcol;
+        u64 *wkey, *ck, *cB;
+        float *kvs;
+        int *rsize, *rlist, *pend_t, *pend_s, *rstamp;
+        unsigned char *ccnt;
+        long long Rmax;
+        int R, b, G;
+    } cx;
     // phase timers and the counters one thread keeps (thread 0, thread 32 for
     // the refill team): here rather than in registers of the round loop
     struct {
-        u64 ph[6], xs[8], xscan[2], xwalk, xlast, tmark;
+        u64 ph[6], xs[8], xscan[2], tmark;
         long long fills, installs, rounds, idle, walk, rescans;
-        long long nlast, nlast_b, nlast_b_scan, nlast_a_scan;
     } ty;
 };
 
@@ -399,8 +426,8 @@ struct Shared {
 // kMaxReq.  Thread t holds CTA t's request count and rows.  Sets
 // sh.exec_row and sh.nexec; thread b gives this CTA's own requests (list
 // pq) their list positions.
-template <int NT, int S>
-__device__ void exchange_requests(int cnt, const int (&rq)[kReqPerCta], int b, Shared<NT, S> &sh, int pq,
+template <int NT, bool ONE>
+__device__ void exchange_requests(int cnt, const int (&rq)[kReqPerCta], int b, Shared<NT, ONE> &sh, int pq,
                                   int *pend_t, int *pend_s)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -458,18 +485,22 @@ __device__ __forceinline__ void team_sync()
 }
 
 // KK smallest keys over every thread's sorted list, for a team of the CTA's
-// last TB threads (default: all of them); result in sh.tko (team threads).
-template <int NT, int S, int KK, int TB = NT>
-__device__ void block_topk(u64 (&L)[KK], Shared<NT, S> &sh)
+// last TB threads (default: all of them); result in sh.tko, and in sh.tnext a
+// lower bound of every other key (team threads).
+template <int NT, bool ONE, int KK, int TB = NT>
+__device__ void block_topk(u64 (&L)[KK], Shared<NT, ONE> &sh)
 {
     constexpr int W0 = (NT - TB) / 32;  // first warp of the team
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     u64 w[KK];
+    u64 end = L[KK - 1] == kNoKey ? kNoKey : L[KK - 1] + 1;
     warp_topk(L, w);
+    u64 nx = warp_u64_min(L[0] != kNoKey ? L[0] : end);
     if (lane == 0) {
 #pragma unroll
         for (int q = 0; q < KK; ++q)
             sh.tk[warp][q] = w[q];
+        sh.tnx[warp] = nx;
     }
     team_sync<NT, TB>();
     if (warp == W0) {
@@ -477,11 +508,14 @@ __device__ void block_topk(u64 (&L)[KK], Shared<NT, S> &sh)
 #pragma unroll
         for (int q = 0; q < KK; ++q)
             M[q] = lane < TB / 32 ? sh.tk[W0 + lane][q] : kNoKey;
+        end = lane < TB / 32 ? sh.tnx[W0 + lane] : kNoKey;
         warp_topk(M, w);
+        nx = warp_u64_min(M[0] != kNoKey ? M[0] : end);
         if (lane == 0) {
 #pragma unroll
             for (int q = 0; q < KK; ++q)
                 sh.tko[q] = w[q];
+            sh.tnext = nx;
         }
     }
     team_sync<NT, TB>();
@@ -493,24 +527,20 @@ __device__ void block_topk(u64 (&L)[KK], Shared<NT, S> &sh)
 // are published).  wait: that thread spins with acquire loads until every
 // CTA has arrived, bounded by a wall-clock limit; returns false when the run
 // must stop (this CTA gave up, or another CTA flagged an error).
-// With `last` given (phase timing), thread 0 also learns whether its CTA
-// was the last to arrive.
-__device__ __forceinline__ void grid_arrive(const MergeParams &p, unsigned &epoch, bool *last = nullptr)
+// Two counters: one for the start of a round, one for "every CTA holds the
+// members' cells" (see merge_job).
+__device__ __forceinline__ void grid_arrive(const MergeParams &p, unsigned *bar, unsigned &epoch)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         epoch += 1;
-        if (p.G > 1) {
-            if (last)
-                *last = atom_release_add(p.bar, 1u) + 1u == epoch * (unsigned)p.G;
-            else
-                red_release_add(p.bar, 1u);
-        }
+        if (p.G > 1)
+            red_release_add(bar, 1u);
     }
 }
 
-template <int NT, int S>
-__device__ bool grid_wait(const MergeParams &p, unsigned epoch, Shared<NT, S> &sh)
+template <int NT, bool ONE, class F>
+__device__ bool grid_wait(const MergeParams &p, const unsigned *bar, unsigned epoch, Shared<NT, ONE> &sh, F &&sync)
 {
     if (threadIdx.x == 0) {
         int st = 0;
@@ -518,7 +548,7 @@ __device__ bool grid_wait(const MergeParams &p, unsigned epoch, Shared<NT, S> &s
             const unsigned target = epoch * (unsigned)p.G;
             const u64 t0 = global_ns();
             unsigned spins = 0;
-            while (ld_acquire_u32(p.bar) < target) {
+            while (ld_acquire_u32(bar) < target) {
                 if ((++spins & 255u) == 0) {
                     st = ld_relaxed_s32(p.status);
                     if (st != 0)
@@ -534,8 +564,14 @@ __device__ bool grid_wait(const MergeParams &p, unsigned epoch, Shared<NT, S> &s
         }
         sh.flag = st;
     }
-    __syncthreads();
+    sync();
     return sh.flag == 0;
+}
+
+template <int NT, bool ONE>
+__device__ bool grid_wait(const MergeParams &p, const unsigned *bar, unsigned epoch, Shared<NT, ONE> &sh)
+{
+    return grid_wait(p, bar, epoch, sh, [] { __syncthreads(); });
 }
 
 // Live-column test against the CTA's copy of the liveness bitmap.
@@ -547,7 +583,7 @@ __device__ __forceinline__ bool live(const unsigned *bitmap, long long c)
 // Adds one input cell to a per-lane list during the initial scan: checks it
 // (finite and >= 0), rewrites -0 as +0 in memory, and keeps the K smallest.
 __device__ __forceinline__ void init_cell(float v, long long q, unsigned c, const MergeParams &p,
-                                          u64 (&L)[K], int &bad)
+                                          u64 (&L)[K], int &bad, unsigned &mx)
 {
     unsigned u = __float_as_uint(v);
     if (u > 0x7f7fffffu) {
@@ -559,6 +595,7 @@ __device__ __forceinline__ void init_cell(float v, long long q, unsigned c, cons
             return;
         }
     }
+    mx = u > mx ? u : mx;
     // a key not below the list's largest cannot enter it (an exact test of
     // the whole key: cells tying on the value are common and go no further)
     const u64 key = ((u64)u << 32) | (u64)c;
@@ -569,7 +606,7 @@ __device__ __forceinline__ void init_cell(float v, long long q, unsigned c, cons
 
 // K smallest keys of row r (all columns are live at launch), computed by one
 // warp that also validates every cell of the row.
-__device__ void warp_row_topk(const MergeParams &p, long long r, u64 (&out)[K], int &bad)
+__device__ void warp_row_topk(const MergeParams &p, long long r, u64 (&out)[K], u64 &next, int &bad, unsigned &mx)
 {
     const long long n = p.n;
     const int lane = threadIdx.x & 31;
@@ -585,9 +622,9 @@ __device__ void warp_row_topk(const MergeParams &p, long long r, u64 (&out)[K], 
         a0 = end;
     const long long a1 = a0 + ((end - a0) & ~3LL);
     for (long long q = start + lane; q < a0; q += 32)
-        init_cell(LDCG(p.D + q), q, (unsigned)(q + base_c), p, L, bad);
+        init_cell(LDCG(p.D + q), q, (unsigned)(q + base_c), p, L, bad, mx);
     for (long long q = a1 + lane; q < end; q += 32)
-        init_cell(LDCG(p.D + q), q, (unsigned)(q + base_c), p, L, bad);
+        init_cell(LDCG(p.D + q), q, (unsigned)(q + base_c), p, L, bad, mx);
     // 128-bit body, four loads in flight per lane
     long long q = a0 + 4 * lane;
     for (; q + 3 * 128 < a1; q += 4 * 128) {
@@ -599,21 +636,21 @@ __device__ void warp_row_topk(const MergeParams &p, long long r, u64 (&out)[K], 
         for (int u = 0; u < 4; ++u) {
             const long long qq = q + 128 * u;
             const unsigned c = (unsigned)(qq + base_c);
-            init_cell(x[u].x, qq, c, p, L, bad);
-            init_cell(x[u].y, qq + 1, c + 1, p, L, bad);
-            init_cell(x[u].z, qq + 2, c + 2, p, L, bad);
-            init_cell(x[u].w, qq + 3, c + 3, p, L, bad);
+            init_cell(x[u].x, qq, c, p, L, bad, mx);
+            init_cell(x[u].y, qq + 1, c + 1, p, L, bad, mx);
+            init_cell(x[u].z, qq + 2, c + 2, p, L, bad, mx);
+            init_cell(x[u].w, qq + 3, c + 3, p, L, bad, mx);
         }
     }
     for (; q < a1; q += 128) {
         const float4 x = LDCG(reinterpret_cast<const float4 *>(p.D + q));
         const unsigned c = (unsigned)(q + base_c);
-        init_cell(x.x, q, c, p, L, bad);
-        init_cell(x.y, q + 1, c + 1, p, L, bad);
-        init_cell(x.z, q + 2, c + 2, p, L, bad);
-        init_cell(x.w, q + 3, c + 3, p, L, bad);
+        init_cell(x.x, q, c, p, L, bad, mx);
+        init_cell(x.y, q + 1, c + 1, p, L, bad, mx);
+        init_cell(x.z, q + 2, c + 2, p, L, bad, mx);
+        init_cell(x.w, q + 3, c + 3, p, L, bad, mx);
     }
-    warp_topk(L, out);
+    warp_topk_next(L, out, next);
 }
 
 // K smallest keys of row r over live columns, computed by the whole CTA (a
@@ -621,9 +658,9 @@ __device__ void warp_row_topk(const MergeParams &p, long long r, u64 (&out)[K], 
 // `live_cells`.  Result in sh.tko.
 // (Row scans are kept out of line: inside the round loop's register
 // allocation their loads in flight would be spilled.)
-template <int NT, int S, int TB = NT>
-__device__ __noinline__ void block_row_topk(const MergeParams &p, long long r, const unsigned *bitmap,
-                                            Shared<NT, S> &sh, long long &live_cells)
+template <int NT, bool ONE, int TB = NT>
+__device__ __noinline__ void block_row_topk(const MergeParams &p, long long r, int piece, int np,
+                                            const unsigned *bitmap, Shared<NT, ONE> &sh, long long &live_cells)
 {
     const int ts = threadIdx.x - (NT - TB);  // thread of the team
     const long long n = p.n;
@@ -651,13 +688,17 @@ __device__ __noinline__ void block_row_topk(const MergeParams &p, long long r, c
     if (a0 > end)
         a0 = end;
     const long long a1 = a0 + ((end - a0) & ~3LL);
-    for (long long q = start + ts; q < a0; q += TB)
-        take(LDCG(p.D + q), q);
-    for (long long q = a1 + ts; q < end; q += TB)
-        take(LDCG(p.D + q), q);
+    if (piece == 0)
+        for (long long q = start + ts; q < a0; q += TB)
+            take(LDCG(p.D + q), q);
+    if (piece == np - 1)
+        for (long long q = a1 + ts; q < end; q += TB)
+            take(LDCG(p.D + q), q);
     const float4 *D4 = reinterpret_cast<const float4 *>(p.D);
-    const long long j1 = a1 >> 2;
-    for (long long j0 = (a0 >> 2) + ts; j0 < j1; j0 += 8 * TB) {
+    const long long part = ((a1 - a0) >> 2) / np;
+    const long long jb = (a0 >> 2) + part * piece;
+    const long long j1 = piece == np - 1 ? a1 >> 2 : jb + part;
+    for (long long j0 = jb + ts; j0 < j1; j0 += 8 * TB) {
         float4 v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -676,158 +717,8 @@ __device__ __noinline__ void block_row_topk(const MergeParams &p, long long r, c
         }
     }
     live_cells += cnt;
-    block_topk<NT, S, K, TB>(L, sh);
+    block_topk<NT, ONE, K, TB>(L, sh);
 }
-
-// block_row_topk in the row-log layout.  Row r's current cells are (a) r's
-// log at every merge q after r's stamp whose survivor c is still live and
-// has not merged again (vpos: this CTA's bitmap of such "latest" merges),
-// and (b) row r of M at every other live column.  Part (a) marks its columns
-// in the scratch bitmap `newer`, part (b) skips them; only c > r count.
-// Merges t0 .. t0 + L0 - 1 (the current round, L0 > 0 only after this CTA's
-// own pass 2) take their survivors from the round's chain in shared memory,
-// older ones from the merge list.  Used by the owner's immediate rescans,
-// which run in the round they are needed (refill scans, which read the state
-// a whole round left, go column by column: block_row_topk_cols).  Result in
-// sh.tko.
-template <int NT, int S, int TB = NT>
-__device__ __noinline__ void block_row_topk_log(const MergeParams &p, long long r, const unsigned *bitmap,
-                                   const unsigned *vpos, unsigned *newer, Shared<NT, S> &sh, long long t0,
-                                   int L0, long long &live_cells, u64 *tlog = nullptr)
-{
-    const int ts = threadIdx.x - (NT - TB);  // thread of the team
-    // with phase timing on, the team's first thread adds the time of the log
-    // part to tlog[0] and of the matrix part (and the top-K) to tlog[1]
-    u64 tm0 = tlog && ts == 0 ? global_ns() : 0;
-    const long long n = p.n;
-    const long long nwords = (n + 31) / 32;
-    const int sr = LDCG(p.stamp + r);
-    u64 L[K];
-#pragma unroll
-    for (int q = 0; q < K; ++q)
-        L[q] = kNoKey;
-    long long cnt = 0;
-    auto take = [&](float v, long long c) {
-        ++cnt;
-        const u64 key = make_key(v, (unsigned)c);
-        if (key < L[K - 1])  // the whole key: ties on the value stop here
-            list_insert(L, key);
-    };
-    for (long long w = ts; w < nwords; w += TB)
-        newer[w] = 0u;
-    team_sync<NT, TB>();
-    // (a) the log: latest merges after r's stamp, eight positions in flight
-    const float *log = p.TL + r * p.pitch;
-    const long long t1 = t0 + L0;
-    {
-        constexpr int U = 8;
-        for (long long q0 = (long long)sr + 1 + ts; q0 < t1; q0 += U * TB) {
-            float v[U];
-            int c[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const long long q = q0 + (long long)u * TB;
-                c[u] = -1;
-                if (q < t1 && ((vpos[q >> 5] >> (q & 31)) & 1u)) {
-                    c[u] = q < t0 ? LDCG(p.merges + 2 * q) : sh.pi[q - t0];
-                    v[u] = LDCG(log + q);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (c[u] >= 0) {
-                    atomicOr(&newer[c[u] >> 5], 1u << (c[u] & 31));
-                    if (c[u] > r)
-                        take(v[u], c[u]);
-                }
-            }
-        }
-    }
-    team_sync<NT, TB>();
-    if (tlog && ts == 0) {
-        const u64 now = global_ns();
-        tlog[0] += now - tm0;
-        tm0 = now;
-    }
-    // (b) row r of M at live columns c > r not found in the log: 16-byte
-    // pieces (rows start 16-byte aligned), eight in flight per thread.  The
-    // first batch also gives a bound: the 4th smallest of the team's
-    // per-thread minima is the key of a real cell with at least three real
-    // cells below it, so no cell above it can be among the row's four
-    // smallest; after it only cells at or below it reach the lists.
-    const float *row = p.D + r * p.pitch;
-    auto cur = [&](long long c) { return ((bitmap[c >> 5] & ~newer[c >> 5]) >> (c & 31)) & 1u; };
-    long long c_a = (r + 4) & ~3LL;  // first multiple of 4 above r
-    if (c_a > n)
-        c_a = n;
-    const long long c_b = c_a + ((n - c_a) & ~3LL);
-    for (long long c = r + 1 + ts; c < c_a; c += TB)
-        if (cur(c))
-            take(LDCG(row + c), c);
-    for (long long c = c_b + ts; c < n; c += TB)
-        if (cur(c))
-            take(LDCG(row + c), c);
-    {
-        constexpr int U = 8;
-        const float4 *R4 = reinterpret_cast<const float4 *>(row);
-        const long long j1 = c_b >> 2;
-        u64 thr = kNoKey;
-        bool first = true;
-        for (long long j0 = (c_a >> 2) + ts;; j0 += U * TB) {
-            if (!first && j0 >= j1)
-                break;  // (every thread of the team runs the first batch: it holds a barrier)
-            float4 v[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const long long j = j0 + (long long)u * TB;
-                v[u] = j < j1 ? LDCG(R4 + j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
-            if (first) {
-                u64 mn = kNoKey;
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const long long j = j0 + (long long)u * TB;
-                    if (j < j1) {
-                        const long long c = j << 2;
-                        const unsigned m4 = ((bitmap[c >> 5] & ~newer[c >> 5]) >> (c & 31)) & 15u;
-                        const float vv[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const u64 k = make_key(vv[e], (unsigned)(c + e));
-                            if (((m4 >> e) & 1u) && k < mn)
-                                mn = k;
-                        }
-                    }
-                }
-                u64 M4[K] = {mn, kNoKey, kNoKey, kNoKey};
-                block_topk<NT, S, K, TB>(M4, sh);
-                thr = sh.tko[K - 1];
-                first = false;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const long long j = j0 + (long long)u * TB;
-                if (j < j1) {
-                    const long long c = j << 2;
-                    const unsigned m4 = ((bitmap[c >> 5] & ~newer[c >> 5]) >> (c & 31)) & 15u;
-                    cnt += __popc(m4);
-                    const float vv[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const u64 k = make_key(vv[e], (unsigned)(c + e));
-                        if (((m4 >> e) & 1u) && k <= thr && k < L[K - 1])
-                            list_insert(L, k);
-                    }
-                }
-            }
-        }
-    }
-    live_cells += cnt;
-    block_topk<NT, S, K, TB>(L, sh);
-    if (tlog && ts == 0)
-        tlog[1] += global_ns() - tm0;
-}
-
 // block_row_topk in the row-log layout, column by column: live column c > r
 // holds its current cell in row r of M when c's stamp is not after r's, and
 // otherwise in r's log at c's stamp (written by that merge).  The stamps are
@@ -835,13 +726,20 @@ __device__ __noinline__ void block_row_topk_log(const MergeParams &p, long long 
 // batch), then the log cells of the columns stamped after r: two dependent
 // reads per batch and no pass over the merge list.  (A deeper batch holds
 // more registers across the call, and the caller, the round loop, then
-// spills: two pieces measured fastest.)  Needs p.D and p.stamp 16-byte
-// aligned (rows are, the pitch being a multiple of 4).  The first batch
-// gives a bound when the row has more than one batch (see
-// block_row_topk_log).  Result in sh.tko.
-template <int NT, int S, int TB = NT>
-__device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long r, const unsigned *bitmap,
-                                                 Shared<NT, S> &sh, long long &live_cells, u64 *tlog = nullptr)
+// spills: two pieces measured fastest.)  p.D and p.stamp are 16-byte aligned
+// (rows are, the pitch being a multiple of 4).  Columns stamped tskip or
+// later are left out: a scan that runs while other CTAs apply the round's
+// merges skips the columns they rewrite, whose log cells may not be there
+// yet.  The first batch gives a bound when the row has more than one: the 5th
+// smallest of the team's per-thread minima is the key of a real cell with at
+// least four real cells below it, so no cell above it can be among the row's
+// five smallest (the lists and the bound of the rest); after it only cells at
+// or below it reach the lists.  Piece
+// `piece` of np equal pieces of the row.  Result in sh.tko.
+template <int NT, bool ONE, int TB = NT>
+__device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long r, int piece, int np,
+                                                 int tskip, const unsigned *bitmap, Shared<NT, ONE> &sh,
+                                                 long long &live_cells, u64 *tlog = nullptr)
 {
     const int ts = threadIdx.x - (NT - TB);  // thread of the team
     const u64 tm0 = tlog && ts == 0 ? global_ns() : 0;
@@ -856,8 +754,10 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
     long long cnt = 0;
     auto one = [&](long long c) {
         if (live(bitmap, c)) {
-            ++cnt;
             const int sc = LDCG(p.stamp + c);
+            if (sc >= tskip)
+                return;
+            ++cnt;
             const float v = sc > sr ? LDCG(log + sc) : LDCG(row + c);
             const u64 key = make_key(v, (unsigned)c);
             if (key < L[K - 1])
@@ -868,15 +768,36 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
     if (c_a > n)
         c_a = n;
     const long long c_b = c_a + ((n - c_a) & ~3LL);
-    for (long long c = r + 1 + ts; c < c_a; c += TB)
-        one(c);
-    for (long long c = c_b + ts; c < n; c += TB)
-        one(c);
+    if (piece == 0)
+        for (long long c = r + 1 + ts; c < c_a; c += TB)
+            one(c);
+    if (piece == np - 1)
+        for (long long c = c_b + ts; c < n; c += TB)
+            one(c);
     {
         constexpr int U = 2;
         const float4 *R4 = reinterpret_cast<const float4 *>(row);
         const int4 *S4 = reinterpret_cast<const int4 *>(p.stamp);
-        const long long j0a = c_a >> 2, j1 = c_b >> 2;
+        const long long part = ((c_b - c_a) >> 2) / np;
+        const long long j0a = (c_a >> 2) + part * piece;
+        const long long j1 = piece == np - 1 ? c_b >> 2 : j0a + part;
+        if (tskip < 0x7fffffff && n > kRefillEarlyN) {
+            // the piece's lines of the row, and an equal part of the log's words
+            // that live columns may need unless those are few: read at the
+            // memory's rate now instead of a sector per column later (n = 65536
+            // complete: 22.0 us of scans per round without, 18.5 with; nothing
+            // gained where a piece is a batch or two)
+            for (long long j = (j0a & ~7LL) + 8LL * ts; j < j1; j += 8LL * TB)
+                if (CHECK_PREFETCH(R4 + j))
+                    prefetch_l2(R4 + j);
+            const long long words = tskip - sr;
+            if (words <= 4 * (n - tskip)) {
+                const long long w0 = sr + words * piece / np, w1 = sr + words * (piece + 1) / np;
+                for (long long j = (w0 & ~31LL) + 32LL * ts; j < w1; j += 32LL * TB)
+                    if (j >= 0 && CHECK_PREFETCH(log + j))
+                        prefetch_l2(log + j);
+            }
+        }
         // a bound from the first batch only pays when more batches follow
         bool first = j1 - j0a > (long long)U * TB;
         u64 thr = kNoKey;
@@ -903,8 +824,12 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
             for (int u = 0; u < U; ++u) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (((m4[u] >> e) & 1u) && sc[u][e] > sr)
-                        v[u][e] = LDCG(log + sc[u][e]);
+                    if (((m4[u] >> e) & 1u) && sc[u][e] > sr) {
+                        if (sc[u][e] < tskip)
+                            v[u][e] = LDCG(log + sc[u][e]);
+                        else
+                            m4[u] &= ~(1u << e);
+                    }
             }
             if (first) {
                 u64 mn = kNoKey;
@@ -919,8 +844,8 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
                     }
                 }
                 u64 M4[K] = {mn, kNoKey, kNoKey, kNoKey};
-                block_topk<NT, S, K, TB>(M4, sh);
-                thr = sh.tko[K - 1];
+                block_topk<NT, ONE, K, TB>(M4, sh);
+                thr = sh.tnext;
                 first = false;
             }
 #pragma unroll
@@ -937,7 +862,7 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
         }
     }
     live_cells += cnt;
-    block_topk<NT, S, K, TB>(L, sh);
+    block_topk<NT, ONE, K, TB>(L, sh);
     if (tlog && ts == 0)
         tlog[1] += global_ns() - tm0;
 }
@@ -946,8 +871,7 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
 // rows of a one-CTA job are refreshed this way, several warps side by side).
 // Adds the live cells read to `live_cells`.  Result in out (all lanes).
 __device__ __noinline__ void warp_row_refresh(const MergeParams &p, long long r, const unsigned *bitmap,
-                                              u64 (&out)[K],
-                                 long long &live_cells)
+                                              u64 (&out)[K], u64 &next, long long &live_cells)
 {
     const int lane = threadIdx.x & 31;
     const long long start = row_base(p, r) + r + 1;
@@ -996,20 +920,985 @@ __device__ __noinline__ void warp_row_refresh(const MergeParams &p, long long r,
         }
     }
     live_cells += cnt;
-    warp_topk(L, out);
+    warp_topk_next(L, out, next);
+}
+// Ward's cell (coefficients depend on the third cluster's size fk).
+__device__ __forceinline__ float ward_cell(float fi, float fj, float fs, float fk, float h, float a, float b)
+{
+    const float T = __fadd_rn(fs, fk);  // (integers below 2^24: exact)
+    const float x = __fdiv_rn(__fadd_rn(fi, fk), T), y = __fdiv_rn(__fadd_rn(fj, fk), T);
+    const float z = -__fdiv_rn(fk, T);
+    return lw_sum(x, y, __fmul_rn(z, h), 0.0f, a, b);
+}
+
+// Table 1 coefficients of a merge of sizes ni, nj at height h: a_i, a_j, b
+// times h, g (LK 3, Ward: per cell, see ward_cell).  Centroid: exact integers,
+// each converted to float once, one division.
+template <int LK>
+__device__ __forceinline__ float4 merge_coefs(int ni, int nj, float h)
+{
+    float4 co = make_float4(0.5f, 0.5f, __fmul_rn(0.0f, h), 0.0f);
+    if (LK == 0)
+        co.w = -0.5f;
+    if (LK == 1)
+        co.w = 0.5f;
+    if (LK == 2 || LK == 5) {
+        const float fs = (float)(ni + nj);
+        co.x = __fdiv_rn((float)ni, fs);
+        co.y = __fdiv_rn((float)nj, fs);
+    }
+    if (LK == 5)
+        co.z = __fmul_rn(-__fdiv_rn(__ll2float_rn((long long)ni * nj), __ll2float_rn((long long)(ni + nj) * (ni + nj))),
+                         h);
+    return co;
+}
+
+// Merge q for a row of size nk: the new cell from its two cells.
+__device__ __forceinline__ float merge_cell(const Team &tm, int linkage, int q, float a, float b, float nk)
+{
+    if (linkage == 3) {
+        const int4 rec = tm.rec[q];
+        return ward_cell((float)rec.z, (float)rec.w, (float)(rec.z + rec.w), nk, __int_as_float(rec.y), a, b);
+    }
+    const float4 co = tm.co[q];
+    return lw_sum(co.x, co.y, co.z, co.w, a, b);
+}
+
+// A lower bound (value bits) of the cells between a merged cluster and others,
+// from the bounds la, lb of its two parts' cells (both above the height h): the
+// update formula is monotone in both distances, so it is evaluated at the
+// bounds, less a margin for its roundings.  Per linkage, rounding errors in
+// units of 2^-24: complete: s + |d|/2 >= max(a, b) up to 3 relative, and >=
+// min(a, b) without error (rounding is monotone, and so for weighted); single:
+// the terms reach the larger distance, 2.5 of the largest value in the matrix;
+// weighted: 1 relative; average, centroid: 4 relative; Ward: the weighted mean
+// of a and b is a bound for every size of the third cluster (the formula rises
+// from it with that size while a, b >= h), at most 12 relative.  The margins
+// taken (2e-6 = 33, 8e-6 = 134 units) leave room for the bound's own roundings.
+// Values too small for a relative margin, or not finite, give bound 0: the
+// round then ends where it would need it.
+template <int LK>
+__device__ __forceinline__ unsigned merged_bound(int lab, int lbb, float fi, float fs, float h, unsigned dmax)
+{
+    const float la = __int_as_float(lab), lb = __int_as_float(lbb);
+    float r;
+    if (LK == 0)
+        r = fminf(la, lb) - 2.0e-6f * __uint_as_float(dmax);
+    else if (LK == 1)
+        r = fmaxf(fminf(la, lb), fmaxf(la, lb) * (1.0f - 2.0e-6f));
+    else if (LK == 4)
+        r = fmaxf(fminf(la, lb), (0.5f * la + 0.5f * lb) * (1.0f - 2.0e-6f));
+    else {
+        const float w = __fdividef(fi, fs);
+        r = w * la + (1.0f - w) * lb;
+        if (LK == 5)
+            r = r - w * (1.0f - w) * h;
+        r = r * (1.0f - 8.0e-6f);
+    }
+    if ((lab & lbb) == -1)
+        return 0xffffffffu;  // no such cells
+    // (a NaN fails both comparisons)
+    return r > 1.0e-30f && r < 3.0e38f ? __float_as_uint(r) : 0u;
+}
+
+// The step-by-step iteration among a round's members, as far as no other cell
+// can come first; run by one warp, lane l holding members l and l + 32.  Only
+// cells at or below the bound matter: per member row a mask of them (columns
+// above the row) and the smallest one are kept in registers.
+//
+// One warp issues a step's instructions one after another, so their number is
+// its time: everything is computed for all 64 members without branches, and
+// what rarely happens (a lost minimum with other cells below the bound, a new
+// cell below it, equal values at a bound) sits behind votes.
+template <int LK>
+__device__ __noinline__ void simulate_steps(Team &tm, int &L_out, bool &dep_out)
+{
+    const int lane = threadIdx.x & 31;
+    const int m = tm.m;
+    const unsigned thv = tm.thv;
+    constexpr unsigned kNone = 0xffffffffu;
+    unsigned nv[2], nc[2], lbv[2];
+    u64 mk[2];
+    bool lv[2];
+    float fk[2];
+    float *row[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int a = lane + 32 * h;
+        lv[h] = a < m;
+        nv[h] = lv[h] ? tm.nnv[a] : kNone;
+        nc[h] = lv[h] ? tm.nnc[a] : kNone;
+        mk[h] = lv[h] ? tm.mask[a] : 0ull;
+        lbv[h] = lv[h] ? (unsigned)tm.sl[a].y : kNone;
+        fk[h] = lv[h] ? (float)tm.sl[a].x : 1.0f;
+        row[h] = tm.S[a];
+        tm.res[a] = 0;
+    }
+    u64 merged = 0ull;
+    bool dep = false;
+    int L = 0;
+    __syncwarp();
+    while (L < kTeam - 1) {
+        const bool sec = nv[1] < nv[0] || (nv[1] == nv[0] && nc[1] < nc[0]);
+        const unsigned v1 = sec ? nv[1] : nv[0], c1 = sec ? nc[1] : nc[0];
+        const unsigned hb = __reduce_min_sync(kFull, v1);
+        const unsigned lbmin = __reduce_min_sync(kFull, lbv[0] < lbv[1] ? lbv[0] : lbv[1]);
+        const unsigned code = __reduce_min_sync(kFull, v1 == hb ? c1 : kNone);
+        if (code == kNone)
+            break;
+        const int i = (int)(code >> 8), j = (int)(code & 0xffu);
+        if (hb >= lbmin) {
+            // equal values: whole keys against the bounds that are keys (those
+            // of merged clusters are values)
+            const u64 kA = ((u64)hb << 32) | (unsigned)tm.mem[i];
+            const unsigned kC = (unsigned)tm.mem[j];
+            bool ok = kA < tm.thA || (kA == tm.thA && kC < tm.thC);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int a = lane + 32 * h;
+                if (lv[h]) {
+                    if ((merged >> a) & 1ull)
+                        ok = ok && hb < lbv[h];
+                    else
+                        ok = ok && (kA < tm.lbA[a] || (kA == tm.lbA[a] && kC < tm.lbC[a]));
+                }
+            }
+            if (!__all_sync(kFull, ok))
+                break;
+        }
+        float ca[2], cb[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            ca[h] = row[h][i];
+            cb[h] = row[h][j];
+        }
+        const int2 si = tm.sl[i], sj = tm.sl[j];
+        const float hgt = __uint_as_float(hb);
+        const float fi = (float)si.x, fj = (float)sj.x, fs = (float)(si.x + sj.x);
+        const float4 co = merge_coefs<LK>(si.x, sj.x, hgt);
+        const u64 bi = 1ull << i, bj = 1ull << j;
+        bool low[2], lost[2];
+        float v[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = lane + 32 * h;
+            v[h] = LK == 3 ? ward_cell(fi, fj, fs, fk[h], hgt, ca[h], cb[h])
+                           : lw_sum(co.x, co.y, co.z, co.w, ca[h], cb[h]);
+            row[h][i] = v[h];
+            tm.S[i][k] = v[h];
+            lv[h] = lv[h] && k != j;
+            low[h] = lv[h] && k != i && __float_as_uint(v[h]) <= thv;
+            const unsigned c = nc[h] & 0xffu;
+            lost[h] = (c == (unsigned)i || c == (unsigned)j) && k != i;  // (a column above k)
+            mk[h] &= ~(bi | bj);
+            nv[h] = lost[h] || k == j ? kNone : nv[h];
+            nc[h] = lost[h] || k == j ? kNone : nc[h];
+        }
+        const unsigned nbits = merged_bound<LK>(si.y, sj.y, fi, fs, hgt, tm.dmax);
+        merged |= bi;
+        const unsigned more = __ballot_sync(kFull, (lost[0] && mk[0] != 0ull && lv[0]) || (lost[1] && mk[1] != 0ull && lv[1]));
+        const unsigned l0 = __ballot_sync(kFull, low[0]), l1 = __ballot_sync(kFull, low[1]);
+        if (more) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = lane + 32 * h;
+                if (lost[h] && lv[h]) {
+                    for (u64 q = mk[h]; q; q &= q - 1) {
+                        const int c = __ffsll((long long)q) - 1;
+                        const unsigned x = __float_as_uint(row[h][c]), y = (unsigned)(k << 8 | c);
+                        if (x < nv[h] || (x == nv[h] && y < nc[h])) {
+                            nv[h] = x;
+                            nc[h] = y;
+                        }
+                    }
+                }
+            }
+        }
+        unsigned ri = kNone, rc = kNone;
+        u64 rm = 0ull;
+        if (l0 | l1) {
+            // new cells at or below the bound: those of rows k < i, and row i's
+            unsigned w[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = lane + 32 * h;
+                const unsigned x = __float_as_uint(v[h]), y = (unsigned)(k << 8 | i);
+                if (low[h] && k < i) {
+                    mk[h] |= bi;
+                    if (x < nv[h] || (x == nv[h] && y < nc[h])) {
+                        nv[h] = x;
+                        nc[h] = y;
+                    }
+                }
+                w[h] = low[h] && k > i ? x : kNone;
+            }
+            rm = (((u64)l1 << 32) | l0) & ~((bi << 1) - 1ull);
+            ri = __reduce_min_sync(kFull, w[0] < w[1] ? w[0] : w[1]);
+            const unsigned k0 = w[0] == ri ? (unsigned)lane : 64u, k1 = w[1] == ri ? (unsigned)lane + 32u : 64u;
+            const unsigned kk = __reduce_min_sync(kFull, k0 < k1 ? k0 : k1);
+            rc = rm ? ((unsigned)i << 8 | kk) : kNone;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = lane + 32 * h;
+            if (k == i) {
+                mk[h] = rm;
+                nv[h] = ri;
+                nc[h] = rc;
+                lbv[h] = nbits;
+                fk[h] = fs;
+            }
+            if (k == j) {
+                mk[h] = 0ull;
+                lbv[h] = kNone;
+            }
+        }
+        const int qi = tm.res[i], qj = tm.res[j];
+        dep = dep || (qi | qj) != 0;
+        __syncwarp();
+        if (lane == 0) {
+            tm.rec[L] = make_int4(i | j << 8 | qi << 16 | qj << 24, (int)hb, si.x, sj.x);
+            if (LK != 3)
+                tm.co[L] = co;
+            tm.res[i] = L + 1;
+            tm.sl[i] = make_int2(si.x + sj.x, (int)nbits);
+        }
+        ++L;
+        __syncwarp();
+    }
+    L_out = L;
+    dep_out = dep;
+}
+
+// The round's merges by simulate_steps (warp 0, the members' cells in S and
+// their minima ready), and those that lead to each survivor, in order.  For
+// single and centroid linkage, whose merges mostly take part in one another,
+// and where the chain (below) breaks off early for that reason.
+__device__ __noinline__ void simulate(Team &tm, int linkage)
+{
+    const int lane = threadIdx.x & 31;
+    int L;
+    bool dep;
+    switch (linkage) {
+    case 0: simulate_steps<0>(tm, L, dep); break;
+    case 1: simulate_steps<1>(tm, L, dep); break;
+    case 2: simulate_steps<2>(tm, L, dep); break;
+    case 3: simulate_steps<3>(tm, L, dep); break;
+    case 4: simulate_steps<4>(tm, L, dep); break;
+    default: simulate_steps<5>(tm, L, dep); break;
+    }
+    int ns = L;
+    if (!dep) {
+        // every merge joins two clusters of the round before: its own survivor
+        // (at most kSurv of them, two members each)
+        if (lane < L) {
+            tm.prog[lane] = lane;
+            tm.sfirst[lane] = lane;
+            tm.sq[lane] = lane;
+            tm.sslot[lane] = tm.mem[tm.mi(lane)];
+        }
+    } else {
+        tm.root[lane] = lane;
+        tm.root[lane + 32] = lane + 32;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int q = lane + 32 * h;
+            if (q < L) {
+                const int x = tm.rec[q].x;
+                const int si = (x >> 16) & 0xff, sj = (x >> 24) & 0xff;
+                if (si)
+                    tm.root[si - 1] = q;  // (merge q consumes that result)
+                if (sj)
+                    tm.root[sj - 1] = q;
+            }
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int it = 0; it < 6; ++it) {
+            const int x0 = tm.root[tm.root[lane]], x1 = tm.root[tm.root[lane + 32]];
+            __syncwarp();
+            tm.root[lane] = x0;
+            tm.root[lane + 32] = x1;
+            __syncwarp();
+        }
+        int rt[2];
+        rt[0] = lane < L ? tm.root[lane] : -1;
+        rt[1] = lane + 32 < L ? tm.root[lane + 32] : -1;
+        const unsigned e0 = __ballot_sync(kFull, rt[0] == lane), e1 = __ballot_sync(kFull, rt[1] == lane + 32);
+        const u64 ends = ((u64)e1 << 32) | e0;
+        ns = __popcll(ends);
+        // survivor of merge q: rank of its last merge among the last merges
+        int sidx[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            sidx[h] = rt[h] >= 0 ? __popcll(ends & ((1ull << rt[h]) - 1ull)) : -1;
+        // merges of survivor s: masks of both halves
+        unsigned w0 = 0u, w1 = 0u, g0 = 0u, g1 = 0u, g10 = 0u;
+        for (int s = 0; s < ns; ++s) {
+            const unsigned x0 = __ballot_sync(kFull, sidx[0] == s), x1 = __ballot_sync(kFull, sidx[1] == s);
+            if (lane == s) {
+                w0 = x0;
+                w1 = x1;
+            }
+            if (sidx[0] == s)
+                g0 = x0;
+            if (sidx[1] == s) {
+                g10 = x0;
+                g1 = x1;
+            }
+        }
+        const int len = __popc(w0) + __popc(w1);
+        int inc = len;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(kFull, inc, off);
+            if (lane >= off)
+                inc += o;
+        }
+        const int first = inc - len;
+        const unsigned below = (1u << lane) - 1u;
+        const int f0 = __shfl_sync(kFull, first, sidx[0] & 31), f1 = __shfl_sync(kFull, first, sidx[1] & 31);
+        if (sidx[0] >= 0)
+            tm.prog[f0 + __popc(g0 & below)] = lane;
+        if (sidx[1] >= 0)
+            tm.prog[f1 + __popc(g10) + __popc(g1 & below)] = lane + 32;
+        if (lane < ns)
+            tm.sfirst[lane] = first;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int q = lane + 32 * h;
+            if (rt[h] == q && q < L) {
+                tm.sq[sidx[h]] = q;
+                tm.sslot[sidx[h]] = tm.mem[tm.mi(q)];
+            }
+        }
+    }
+    if (lane == 0) {
+        tm.sfirst[ns] = L;
+        tm.L = L;
+        tm.ns = ns;
+        tm.tie = 0;
+    }
+    __syncwarp();
+    // the survivors' cells to one another
+    if (lane < ns) {
+        const int a = tm.mi(tm.sq[lane]);
+        for (int s = 0; s < ns; ++s)
+            tm.C[s][lane] = tm.S[tm.mi(tm.sq[s])][a];
+    }
+    __syncwarp();
+}
+
+// ---- the round's merges where they follow the entries (complete, group and
+// weighted average, Ward): the chain of entries that share no member, each
+// the next merge of the step-by-step iteration unless a cell made by an
+// earlier one comes first.  The chain is taken by bit scans; then every cell
+// its merges make between members is computed at once and compared.
+
+// Warp 0: the chain.  Lane q gets the entry of merge q; returns their number.
+// A step is a bit scan and one shared-memory read.
+__device__ __forceinline__ int chain_select(Team &tm)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned lo, hi;
+    {
+        bool in[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int e = lane + 32 * h;
+            in[h] = e < tm.ne && tm.ent[e].x != 0xffffu;
+            if (in[h]) {
+                const unsigned x = tm.ent[e].x;
+                const u64 w = tm.em[x & 0xffu] | tm.em[x >> 8];
+                tm.enm[e] = make_uint2((unsigned)w, (unsigned)(w >> 32));
+            }
+            tm.step[e] = 0xff;
+        }
+        lo = __ballot_sync(kFull, in[0]);
+        hi = __ballot_sync(kFull, in[1]);
+    }
+    __syncwarp();
+    int L = 0, mine = 0;
+    while ((lo | hi) != 0u && L < kSurv) {
+        const int e = lo ? __ffs(lo) - 1 : __ffs(hi) + 31;
+        const uint2 w = tm.enm[e];
+        lo &= ~w.x;
+        hi &= ~w.y;
+        mine = lane == L ? e : mine;
+        ++L;
+    }
+    if (lane < L) {
+        const uint2 w = tm.ent[mine];
+        const int i = (int)(w.x & 0xffu), j = (int)(w.x >> 8);
+        tm.rec[lane] = make_int4(i | j << 8, (int)w.y, tm.sz0[i], tm.sz0[j]);
+        tm.ce[lane] = (unsigned char)mine;
+        tm.step[i] = (unsigned char)lane;
+        tm.step[j] = (unsigned char)lane;
+    }
+    tm.lim[lane] = 0xffffffffu;
+    if (lane == 0)
+        tm.L = L;
+    __syncwarp();
+    return L;
+}
+
+// Warp q of a team of nw: coefficients of merges q, q + nw, .. and the cells
+// X[q][k] they make with every member k (those of later merges included).
+template <int LK>
+__device__ __forceinline__ void chain_cells_made(Team &tm, int q0, int nw)
+{
+    const int lane = threadIdx.x & 31;
+    const int L = tm.L;
+    for (int q = q0; q < L; q += nw) {
+        const int4 rec = tm.rec[q];
+        const int i = rec.x & 0xff, j = (rec.x >> 8) & 0xff;
+        const float hgt = __int_as_float(rec.y);
+        const float4 co = merge_coefs<LK>(rec.z, rec.w, hgt);
+        if (LK != 3 && lane == 0)
+            tm.co[q] = co;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = lane + 32 * h;
+            const float a = tm.S[k][i], b = tm.S[k][j];
+            tm.X[q][k] = LK == 3 ? ward_cell((float)rec.z, (float)rec.w, (float)(rec.z + rec.w), (float)tm.sz0[k],
+                                             hgt, a, b)
+                                 : lw_sum(co.x, co.y, co.z, co.w, a, b);
+        }
+    }
+}
+
+// Then, for merge q and every later merge p (lane p): the smallest cell that
+// merge q made and that is there when p comes (value bits, lim[p] the least
+// over q): the cells X[q] to members that no merge takes and to those that
+// merges p and later take, and C[q][c], the cell to cluster c after merges q
+// and c, for the merges c between.
+template <int LK>
+__device__ __forceinline__ void chain_limits(Team &tm, int q0, int nw)
+{
+    const int lane = threadIdx.x & 31;
+    const int L = tm.L, m = tm.m;
+    const unsigned thv = tm.thv;
+    for (int q = q0; q < L; q += nw) {
+        const int4 rq = tm.rec[q];
+        unsigned xy = 0xffffffffu, cc = 0xffffffffu, un = 0xffffffffu;
+        if (lane > q && lane < L) {
+            const int4 rc = tm.rec[lane];
+            const float a = tm.X[q][rc.x & 0xff], b = tm.X[q][(rc.x >> 8) & 0xff];
+            const float c = merge_cell(tm, LK, lane, a, b, (float)(rq.z + rq.w));
+            tm.C[q][lane] = c;
+            tm.C[lane][q] = c;
+            const unsigned ua = __float_as_uint(a), ub = __float_as_uint(b);
+            xy = ua < ub ? ua : ub;
+            cc = __float_as_uint(c);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = lane + 32 * h;
+            if (k < m && tm.step[k] == 0xff) {
+                const unsigned u = __float_as_uint(tm.X[q][k]);
+                un = u < un ? u : un;
+            }
+        }
+        // (cells above the bound of the round never matter)
+        if (__any_sync(kFull, xy <= thv || cc <= thv || un <= thv)) {
+            un = __reduce_min_sync(kFull, un);
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const unsigned y = __shfl_down_sync(kFull, xy, d), z = __shfl_up_sync(kFull, cc, d);
+                if (lane + d < 32)
+                    xy = y < xy ? y : xy;
+                if (lane >= d)
+                    cc = z < cc ? z : cc;
+            }
+            const unsigned z = __shfl_up_sync(kFull, cc, 1);  // the merges before p only
+            if (lane > q && lane < L) {
+                unsigned v = un < xy ? un : xy;
+                v = z < v ? z : v;
+                if (v <= thv)
+                    atomicMin(&tm.lim[lane], v);
+            }
+        }
+    }
+}
+
+// Warp 0: the merges of the chain that the step-by-step iteration takes, lane
+// p for merge p.  It has to be smaller than (1) every cell earlier merges made
+// between members (lim; equal values end the chain), (2) the cells not listed
+// that no earlier merge changed: it comes before the marks that end the rows
+// of the members not merged before it, (3) the cells earlier merges made with
+// clusters outside.  For (3) there are bounds (see merged_bound); where they
+// would cost merges (values tied with the bound of the round, or within its
+// margin), the merges that pass (1) and (2) are taken on condition: the cells
+// are computed before anything is written, and every CTA is asked whether one
+// comes first (tie; only with `allow`).  The first merge is the smallest cell
+// of all.
+template <int LK>
+__device__ __forceinline__ void chain_accept(Team &tm, bool allow)
+{
+    const int lane = threadIdx.x & 31;
+    const int L = tm.L;
+    constexpr unsigned kNone = 0xffffffffu;
+    unsigned own = 0xffu, made = kNone, un = 0xffu, hb = kNone, e = 0u;
+    if (lane < L) {
+        const int4 rec = tm.rec[lane];
+        const int i = rec.x & 0xff, j = (rec.x >> 8) & 0xff;
+        own = min(tm.ex[i], tm.ex[j]);
+        e = tm.ce[lane];
+        hb = (unsigned)rec.y;
+        made = merged_bound<LK>(tm.sl[i].y, tm.sl[j].y, (float)rec.z, (float)(rec.z + rec.w), __int_as_float(rec.y),
+                                0u);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h;
+        if (k < tm.m && tm.step[k] == 0xff)
+            un = min(un, (unsigned)tm.ex[k]);
+    }
+    un = __reduce_min_sync(kFull, un);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned y = __shfl_down_sync(kFull, own, d), z = __shfl_up_sync(kFull, made, d);
+        if (lane + d < 32)
+            own = min(own, y);
+        if (lane >= d)
+            made = min(made, z);
+    }
+    const unsigned z = __shfl_up_sync(kFull, made, 1);
+    const bool in = lane > 0 && lane < L;
+    const unsigned made_first = __ballot_sync(kFull, in && hb >= tm.lim[lane]);
+    const unsigned bad = __ballot_sync(kFull, in && e >= min(un, own)) | made_first;
+    const unsigned out = __ballot_sync(kFull, in && hb >= z) | bad;
+    const int most = bad ? __ffs(bad) - 1 : L, sure = out ? __ffs(out) - 1 : L;
+    const bool tie = allow && most >= sure + kTieGain;
+    const int La = tie ? most : sure;
+    if (lane < La) {
+        tm.prog[lane] = lane;
+        tm.sfirst[lane] = lane;
+        tm.sq[lane] = lane;
+        tm.sslot[lane] = tm.mem[tm.mi(lane)];
+    }
+    if (lane == 0) {
+        tm.sfirst[La] = La;
+        tm.L = La;
+        tm.ns = La;
+        tm.tie = tie;
+        // a cell made between members comes first: many merges are still known
+        tm.redo = most < L && ((made_first >> most) & 1u) && most < kRedoBelow && 2 * most < L + kRedoGap;
+    }
+    __syncwarp();
+}
+
+// The chain's cells, limits and accepted prefix, by team A (the whole CTA in a
+// one-CTA job).
+template <int NT, bool ONE>
+__device__ __noinline__ void chain_phase(Team &tm, int linkage, bool allow)
+{
+    constexpr int WA = ONE ? NT / 32 : NT / 64, TA = WA * 32;
+    const int warp = threadIdx.x >> 5;
+    auto sync_a = [&]() {
+        if constexpr (ONE)
+            __syncthreads();
+        else
+            asm volatile("barrier.cta.sync.aligned 3, %0;" ::"n"(TA) : "memory");
+    };
+    switch (linkage) {
+    case 1: chain_cells_made<1>(tm, warp, WA); break;
+    case 2: chain_cells_made<2>(tm, warp, WA); break;
+    case 3: chain_cells_made<3>(tm, warp, WA); break;
+    default: chain_cells_made<4>(tm, warp, WA); break;
+    }
+    sync_a();
+    if (linkage == 3)
+        chain_limits<3>(tm, warp, WA);
+    else
+        chain_limits<2>(tm, warp, WA);
+    sync_a();
+    if (warp == 0) {
+        switch (linkage) {
+        case 1: chain_accept<1>(tm, allow); break;
+        case 4: chain_accept<4>(tm, allow); break;
+        default: chain_accept<2>(tm, allow); break;
+        }
+    }
+    sync_a();
+}
+
+// Merges f + 1 .. f + len - 1 of a survivor's program for row k, whose first
+// merge gave v: the new cell after the last one.  An operand is a cell in
+// memory or the result of an earlier merge of the program, mostly of the one
+// just before.
+template <bool ONE>
+__device__ __noinline__ float chain_cells(const MergeParams &p, const Team &tm, int f, int len, float v, float nk,
+                                          long long k, int sk, bool ok)
+{
+    float tmp[kTeam];
+    const bool full = !ONE && p.full;
+    const long long bk = row_base(p, k);
+    auto load = [&](int a) -> float {
+        if (!ok)
+            return 0.0f;
+        if (full)
+            return LDCG(tm.mst[a] >= sk ? p.D + tm.mbase[a] + k : p.TL + tm.mbase[a] + sk);
+        const long long x = tm.mem[a];
+        return LDCG(p.D + (k > x ? tm.mbase[a] + k : bk + x));
+    };
+    int prev = tm.prog[f];
+    for (int e = 1; e < len; ++e) {
+        const int q = tm.prog[f + e];
+        const int x = tm.rec[q].x;
+        const int si = ((x >> 16) & 0xff) - 1, sj = ((x >> 24) & 0xff) - 1;
+        if (si != prev && sj != prev)
+            tmp[prev] = v;
+        const float a = si < 0 ? load(x & 0xff) : si == prev ? v : tmp[si];
+        const float b = sj < 0 ? load((x >> 8) & 0xff) : sj == prev ? v : tmp[sj];
+        v = merge_cell(tm, p.linkage, q, a, b, nk);
+        prev = q;
+    }
+    return v;
+}
+
+// Pieces per row when nexec refill rows are served by G CTAs.
+// Long rows: about two per CTA (a CTA with one more than the others holds the
+// round up by less; n = 65536 complete: one per CTA 166 ms, two 161).  Shorter
+// ones: one (two: n = 8191 2 % slower, each piece pays a reduction).
+__device__ __forceinline__ int scan_pieces(int G, int nexec, bool early)
+{
+    const int np = nexec > 0 ? (early ? 2 : 1) * G / nexec : 1;
+    return np < 1 ? 1 : np > kPieces ? kPieces : np;
+}
+
+// Entry of the published lists: (value bits << 32) | (row << kRankBits) | rank,
+// unique and ordered like (value, row, column).
+__device__ __forceinline__ u64 entry_key(u64 cell_key, u64 rowbits, unsigned rank)
+{
+    return (cell_key & kHi) | rowbits | rank;
+}
+
+// The largest key, or one in between, such that lo to hi of the counted ones
+// are at or below it (all of them, up to `top`, if they are no more than hi;
+// fewer if the keys next to it are too many): gallops from the smallest key
+// by way of `guess`, then bisects.  Every thread calls it and gets the same.
+template <class F>
+__device__ __forceinline__ u64 find_pivot(F &&count, u64 least, u64 top, u64 guess, int lo_n, int hi_n)
+{
+    if (count(top) <= hi_n)
+        return top;
+    u64 lo = least, hi = top, step = 1ull << 42;
+    u64 mid = guess > lo && guess < hi ? guess : lo + (step < hi - lo ? step : (hi - lo) / 2);
+    bool open = true;  // hi not met yet
+    while (true) {
+        const int c = count(mid);
+        if (c > hi_n) {
+            hi = mid;
+            open = false;
+        } else if (c < lo_n) {
+            lo = mid;
+        } else {
+            return mid;
+        }
+        if (hi - lo <= 1)
+            return lo;
+        mid = lo + (hi - lo) / 2;
+        if (open && lo - least + step < mid - lo) {
+            mid = lo + (lo - least) + step;
+            step *= 2;
+        }
+    }
+}
+
+// The new cells D(k, survivor) of Section 4 step 3 for the rows l0 .. l0 + rows
+// of a CTA outside the round's merges: into kvs (kvs[q * (kSurv + 1) + s]:
+// chunk row q, survivor s) and, unless the merges wait (tie), into memory.  A
+// warp takes 32 rows and 8 survivors at a time from a counter (team B comes in
+// when its scans are done): 16 loads in flight per thread; the rows of a warp
+// are consecutive, so row cells are read and written in whole lines.
+template <int NT, bool ONE>
+__device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> &sh, int l0, int rows, int ns, int L,
+                                       bool tie)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int b = sh.cx.b, G = ONE ? 1 : sh.cx.G;
+    auto rows_at = [&](int l) -> long long {
+        return ONE ? (long long)l : (long long)((long long)b + (long long)G * (l >> 5)) * kRowBlock + (l & 31);
+    };
+    constexpr int KVP = kSurv + 1;
+    const long long n = p.n;
+    const bool full = !ONE && p.full;
+    const unsigned *bitmap = sh.cx.bitmap, *touched = sh.cx.touched;
+    float *kvs = sh.cx.kvs;
+    const int *rsize = sh.cx.rsize, *rstamp = sh.cx.rstamp;
+    const int nblk = rows / 32;
+    const unsigned last = L > 0 ? (unsigned)sh.tm.rec[L - 1].y : 0u;
+    constexpr int U = 8;
+    // (fewer survivors at a time when that leaves no warp without an item)
+    int ug = U;
+    while (ug > 2 && nblk * ((ns + ug / 2 - 1) / (ug / 2)) <= NT / 32)
+        ug /= 2;
+    const int ng = (ns + ug - 1) / ug;
+    // (a warp takes the next item: team B comes in when its scans are done)
+    const int nit = nblk * ng;
+    while (true) {
+        int it = 0;
+        if (lane == 0)
+            it = atomicAdd(&sh.item, 1);
+        it = __shfl_sync(kFull, it, 0);
+        if (it >= nit)
+            break;
+        const int blk = it % nblk, s0 = (it / nblk) * ug;
+        const int l = l0 + blk * 32 + lane;
+        const long long k = rows_at(l);
+        const bool ok = k < n && live(bitmap, k) && !live(touched, k);
+        const unsigned okb = __ballot_sync(kFull, ok);
+        if (s0 == 0 && lane == 0)
+            sh.okm[blk] = okb;
+        if (okb == 0)
+            continue;
+        const float nk = (float)rsize[l];
+        const long long bk = row_base(p, k);
+        const int sk = full ? rstamp[l] : 0;
+        // cell (k, member): packed, row x for k > x (consecutive k of a
+        // warp read consecutive words) and row k for k < x; row-log
+        // layout, row x of M when x was stamped no earlier than k, else
+        // x's log at k's stamp (words of one contiguous range)
+        auto cell = [&](int a) -> const float * {
+            if (full)
+                return sh.tm.mst[a] >= sk ? p.D + sh.tm.mbase[a] + k : p.TL + sh.tm.mbase[a] + sk;
+            const long long x = sh.tm.mem[a];
+            return p.D + (k > x ? sh.tm.mbase[a] + k : bk + x);
+        };
+        float va[U], vb[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int s = s0 + u;
+            va[u] = 0.0f;
+            vb[u] = 0.0f;
+            if (u < ug && s < ns && ok) {
+                const int q = sh.tm.prog[sh.tm.sfirst[s]];
+                const int x = sh.tm.rec[q].x;
+                va[u] = LDCG(cell(x & 0xff));
+                vb[u] = LDCG(cell((x >> 8) & 0xff));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int s = s0 + u;
+            if (u >= ug || s >= ns)
+                break;
+            const int f = sh.tm.sfirst[s], len = sh.tm.sfirst[s + 1] - f;
+            const int q = sh.tm.prog[f];
+            float v = merge_cell(sh.tm, p.linkage, q, va[u], vb[u], nk);
+            if (len > 1)
+                v = chain_cells<ONE>(p, sh.tm, f, len, v, nk, k, sk, ok);
+            if (ok) {
+                const long long x = sh.tm.sslot[s];
+                kvs[(size_t)(blk * 32 + lane) * KVP + s] = v;
+                if (tie) {
+                    // does it come before a later merge of the round?  (s = q)
+                    const unsigned vb = __float_as_uint(v);
+                    if (vb <= last) {
+                        const u64 kA = ((u64)vb << 32) | (unsigned)(k < x ? k : x);
+                        const unsigned kC = (unsigned)(k < x ? x : k);
+                        for (int e = s + 1; e < L; ++e) {
+                            const int4 rec = sh.tm.rec[e];
+                            const u64 eA = ((u64)(unsigned)rec.y << 32) | (unsigned)sh.tm.mem[rec.x & 0xff];
+                            if (eA > kA || (eA == kA && (unsigned)sh.tm.mem[(rec.x >> 8) & 0xff] > kC)) {
+                                atomicMin(&sh.viol, e);
+                                break;
+                            }
+                        }
+                    }
+                } else if (full) {
+                    // row x is rewritten whole; row k keeps its stale copy
+                    // and the new value goes to k's log (below)
+                    STCG(p.D + x * p.pitch + k, v);
+                } else {
+                    STCG(p.D + (k > x ? row_base(p, x) + k : bk + x), v);
+                }
+            }
+        }
+    }
+}
+
+// The record for round rr: this CTA's kPub smallest entries (cached keys and
+// bound marks of its rows) and its refill requests of round rr - 1.  Also lists
+// the refills to install in round rr (served in round rr - 1).
+template <int NT, bool ONE>
+__device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &sh, int rr)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = sh.cx.b, G = ONE ? 1 : sh.cx.G;
+    auto rows_at = [&](int l) -> long long {
+        return ONE ? (long long)l : (long long)((long long)b + (long long)G * (l >> 5)) * kRowBlock + (l & 31);
+    };
+    constexpr int W = NT / 32;
+    const int R = sh.cx.R;
+    const long long Rmax = sh.cx.Rmax;
+    const u64 *ck = sh.cx.ck, *cB = sh.cx.cB;
+    const unsigned char *ccnt = sh.cx.ccnt;
+    const int *pend_t = sh.cx.pend_t;
+    auto slot_of = [&](long long r) -> int { return (int)(((r / kRowBlock) / G) * kRowBlock + (r & 31)); };
+    RecA *rec = p.recA + (size_t)(rr & 1) * G + b;
+    // a pivot that takes in at least kPub rows' first entries, then the
+    // entries up to it in order by counting
+    u64 head = kNoKey;
+    for (int l = tid; l < R; l += NT) {
+        const int c = ccnt[l];
+        const u64 B = cB[l];
+        if (c > 0 || B != kNoKey) {
+            const u64 e = entry_key(c > 0 ? ck[l] : B, (u64)rows_at(l) << kRankBits, 0);
+            head = e < head ? e : head;
+        }
+        if (rr >= 2 && pend_t[l] == rr - 2) {
+            const int s2 = atomicAdd(&sh.ninst, 1);
+            sh.inst_slot[s2] = l;
+        }
+    }
+    auto entry_at = [&](int l, int q, int c, u64 &e) -> u64 {
+        const u64 x = q < c ? ck[(size_t)q * Rmax + l] : cB[l];
+        e = x == kNoKey ? kNoKey : entry_key(x, (u64)rows_at(l) << kRankBits, q);
+        return x;
+    };
+    if (R > 4 * NT) {
+        // (a CTA of few threads with very many rows: the entries behind few
+        // heads could outnumber kCand)
+        u64 Lst[kPub];
+#pragma unroll
+        for (int q = 0; q < kPub; ++q)
+            Lst[q] = kNoKey;
+        for (int l = tid; l < R; l += NT) {
+            const int c = ccnt[l];
+            for (int q = 0; q <= c; ++q) {
+                u64 e;
+                entry_at(l, q, c, e);
+                if (e < Lst[kPub - 1])
+                    list_insert_n(Lst, e);
+            }
+        }
+        block_topk(Lst, sh);
+        if (tid < kPub) {
+            const u64 key = sh.tko[tid];
+            unsigned col = 0;
+            if (key != kNoKey) {
+                const int l = slot_of((long long)((unsigned)key >> kRankBits));
+                const int q = (int)((unsigned)key & kRankMask);
+                col = q < ccnt[l] ? (unsigned)ck[(size_t)q * Rmax + l] : kRowStop | (unsigned)cB[l];
+                if (tid == kPub - 1)
+                    col |= kHardStop;
+            }
+            STCG(&rec->key[tid], key);
+            STCG(&rec->col[tid], col);
+        }
+    } else {
+    {
+        const u64 x = warp_u64_min(head);
+        if (lane == 0)
+            sh.wmin[warp][0] = x;
+    }
+    if (tid == 0)
+        sh.ncand = 0;
+    __syncthreads();
+    const u64 gmin = warp_u64_min(lane < W ? sh.wmin[lane][0] : kNoKey);
+    auto count = [&](u64 x) -> int { return __syncthreads_count(head <= x && head != kNoKey); };
+    const u64 pivot = find_pivot(count, gmin, kNoKey, sh.ppivot, kPub, 3 * kPub);
+    int have = 0;
+    if (head <= pivot && head != kNoKey) {
+        for (int l = tid; l < R; l += NT) {
+            const int c = ccnt[l];
+            for (int q = 0; q <= c; ++q) {
+                u64 e;
+                entry_at(l, q, c, e);
+                have += e <= pivot && e != kNoKey;
+            }
+        }
+    }
+    int at = have;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(kFull, at, off);
+        if (lane >= off)
+            at += o;
+    }
+    {
+        int base = 0;
+        if (lane == 31 && at > 0)
+            base = atomicAdd(&sh.ncand, at);
+        base = __shfl_sync(kFull, base, 31);
+        at = base + at - have;
+    }
+    if (have > 0) {
+        for (int l = tid; l < R; l += NT) {
+            const int c = ccnt[l];
+            for (int q = 0; q <= c; ++q) {
+                u64 e;
+                const u64 x = entry_at(l, q, c, e);
+                if (e == kNoKey || e > pivot)
+                    break;
+                if (at < kCand) {
+                    sh.ckey[at] = e;
+                    sh.ccol[at] = q < c ? (unsigned)x : kRowStop | (unsigned)x;
+                }
+                ++at;
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0)
+        sh.ppivot = pivot;
+    // (at most 3 * kPub threads of 4 rows and K + 1 entries each: they fit)
+    static_assert(3 * kPub * 4 * (K + 1) <= kCand, "published entries fit");
+    const int N = sh.ncand < kCand ? sh.ncand : kCand;
+    for (int c0 = (tid >> 5) * 8; c0 < N; c0 += NT / 4) {
+        const int c = c0 + (lane >> 2);
+        const u64 key = c < N ? sh.ckey[c] : kNoKey;
+        int rank = 0;
+        for (int f = lane & 3; f < N; f += 4)
+            rank += sh.ckey[f] < key;
+        rank += __shfl_xor_sync(kFull, rank, 1);
+        rank += __shfl_xor_sync(kFull, rank, 2);
+        if (c < N && (lane & 3) == 0 && rank < kPub) {
+            STCG(&rec->key[rank], key);
+            // (more entries may follow the last: none is published)
+            STCG(&rec->col[rank], sh.ccol[c] | (rank == kPub - 1 ? kHardStop : 0u));
+        }
+    }
+    if (tid >= N && tid < kPub) {
+        STCG(&rec->key[tid], kNoKey);
+        STCG(&rec->col[tid], 0u);
+    }
+    }
+    if (tid == 0) {
+        const int par = (rr - 1) & 1;
+        int nq = rr >= 1 ? sh.nmyreq[par] : 0;
+        nq = nq < kReqPerCta ? nq : kReqPerCta;
+        if (rr >= 1)
+            sh.nmyreq[par] = nq;
+        int rows[kReqPerCta];
+#pragma unroll
+        for (int q = 0; q < kReqPerCta; ++q)
+            rows[q] = q < nq ? (int)rows_at(sh.myreq_l[par][q]) : -1;
+        uint4 *dst = reinterpret_cast<uint4 *>(&rec->nreq);
+        STCG(dst + 0, make_uint4((unsigned)nq, (unsigned)rows[0], (unsigned)rows[1], (unsigned)rows[2]));
+        STCG(dst + 1, make_uint4((unsigned)rows[3], (unsigned)rows[4], (unsigned)rows[5], (unsigned)rows[6]));
+        STCG(dst + 2, make_uint4((unsigned)rows[7], sh.tm.dmax, 0u, 0u));
+    }
 }
 
 // All n - 1 merges of one job, run by CTA b of the job's G CTAs (every CTA
 // of the job calls this with the same p).  smem_raw: merge_smem_bytes(n, G)
 // bytes of dynamic shared memory.
-template <int NT, int PUB>
-__device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem_raw,
-                          Shared<NT, round_of(PUB)> &sh)
+template <int NT, bool ONE>
+__device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem_raw, Shared<NT, ONE> &sh)
 {
-    constexpr int S = round_of(PUB);
     constexpr int W = NT / 32;
+    // the team that selects the round's merges (warps 0 .. WA - 1: all of them in
+    // a one-CTA job); the other half of a grid's CTA installs and serves refills
+    // beside it
+    constexpr int WA = ONE ? W : W / 2, TA = WA * 32;
+    constexpr int P = K + 1;  // one-CTA job: keys kept per survivor
+    constexpr int KVP = kSurv + 1;
     const long long n = p.n;
-    const int G = p.G;
+    const int G = ONE ? 1 : p.G;
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
     const long long nb = (n + kRowBlock - 1) / kRowBlock;      // row blocks
@@ -1017,49 +1906,63 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
     const int R = (int)(my_blocks * kRowBlock);                 // owned row slots
     const long long Rmax = ((nb + G - 1) / G) * kRowBlock;
     const long long nwords = (n + 31) / 32;
+    const int CH = p.chunk;                                     // rows per chunk of the apply pass
+    const bool full = !ONE && p.full;
+    const int refill_at = n <= kRefillEarlyN ? 1 : 0;
+    const bool early = !ONE && n > kRefillEarlyN;  // team B scans beside the selection as well
 
-    // dynamic shared memory: liveness bitmap; the published entries of every
-    // CTA (keys, column words); then per owned slot l: cache
+    // dynamic shared memory: liveness bitmap; slots touched by the round's
+    // merges; the published entries of every CTA; per owned slot l: cache
     // keys (key q of slot l at ck[q * Rmax + l]: consecutive threads read
-    // consecutive words), bound, size, key count, pending refill (round,
-    // list position) and a flag for rows in this round's chain
-    unsigned char *q0 = smem_raw;
-    unsigned *bitmap = reinterpret_cast<unsigned *>(q0);
-    q0 += (nwords * 4 + 15) & ~15LL;
-    // row-log layout: merges whose survivor is live and has not merged again
-    // (bit q), and a scratch bitmap of columns for the row scans
-    unsigned *vpos = reinterpret_cast<unsigned *>(q0);
-    unsigned *newer = vpos + nwords;
-    q0 += G > 1 ? (2 * nwords * 4 + 15) & ~15LL : 0;
-    u64 *wkey = reinterpret_cast<u64 *>(q0);
-    q0 += (size_t)G * PUB * 8;
-    u64 *ck = reinterpret_cast<u64 *>(q0);
-    q0 += (size_t)Rmax * K * 8;
-    u64 *cB = reinterpret_cast<u64 *>(q0);
-    q0 += (size_t)Rmax * 8;
-    unsigned *wcol = reinterpret_cast<unsigned *>(q0);
-    q0 += (size_t)G * PUB * 4;
-    // more than 16 pairs per round: pass-1 values of the rows of one chunk of
-    // NT owned rows, kvs[q * KVP + a] for chunk row q and pair a (up to 16
-    // pairs they stay in registers)
-    constexpr int KVP = S + 1;
-    float *kvs = reinterpret_cast<float *>(q0);
-    q0 += S > 16 ? (size_t)(Rmax < NT ? Rmax : NT) * KVP * 4 : 0;
-    int *rsize = reinterpret_cast<int *>(q0);
-    int *ccnt = rsize + Rmax;
-    int *pend_t = ccnt + Rmax;
-    int *pend_s = pend_t + Rmax;
-    int *rlist = pend_s + Rmax;
-    int *rstamp = rlist + Rmax;  // row-log layout: each owned row's stamp
-    unsigned char *mflag = reinterpret_cast<unsigned char *>(rstamp + Rmax);
-    unsigned char *okf = mflag + Rmax;  // [NT]: chunk row q got pass-1 values
+    // consecutive words), bound, size, rescan list, pending refill (round,
+    // list position), stamp, key count; the new cells of one chunk of rows
+    // (their addresses are kept in shared memory too: as registers they would be
+    // live all through the round loop)
+    if (threadIdx.x == 0) {
+        unsigned char *q0 = smem_raw;
+        auto &cx = sh.cx;
+        cx.bitmap = reinterpret_cast<unsigned *>(q0);
+        q0 += (nwords * 4 + 15) & ~15LL;
+        cx.touched = reinterpret_cast<unsigned *>(q0);
+        q0 += (nwords * 4 + 15) & ~15LL;
+        cx.wkey = reinterpret_cast<u64 *>(q0);
+        q0 += ONE ? 0 : (size_t)G * kPub * 8;
+        cx.ck = reinterpret_cast<u64 *>(q0);
+        q0 += (size_t)Rmax * K * 8;
+        cx.cB = reinterpret_cast<u64 *>(q0);
+        q0 += (size_t)Rmax * 8;
+        cx.wcol = reinterpret_cast<unsigned *>(q0);
+        q0 += ONE ? 0 : (size_t)G * kPub * 4;
+        cx.kvs = reinterpret_cast<float *>(q0);  // kvs[q * KVP + s]: chunk row q, survivor s
+        q0 += (size_t)CH * KVP * 4;
+        cx.rsize = reinterpret_cast<int *>(q0);
+        cx.rlist = cx.rsize + Rmax;
+        q0 += (size_t)Rmax * 8;
+        cx.pend_t = reinterpret_cast<int *>(q0);
+        cx.pend_s = cx.pend_t + Rmax;
+        cx.rstamp = cx.pend_s + Rmax;  // row-log layout: each owned row's stamp
+        q0 += ONE ? 0 : (size_t)Rmax * 12;
+        cx.ccnt = q0;
+        cx.Rmax = Rmax;
+        cx.R = R;
+        cx.b = b;
+        cx.G = G;
+    }
+    __syncthreads();
+    unsigned *const &bitmap = sh.cx.bitmap, *const &touched = sh.cx.touched, *const &wcol = sh.cx.wcol;
+    u64 *const &wkey = sh.cx.wkey, *const &ck = sh.cx.ck, *const &cB = sh.cx.cB;
+    float *const &kvs = sh.cx.kvs;
+    int *const &rsize = sh.cx.rsize, *const &rlist = sh.cx.rlist, *const &pend_t = sh.cx.pend_t;
+    int *const &pend_s = sh.cx.pend_s, *const &rstamp = sh.cx.rstamp;
+    unsigned char *const &ccnt = sh.cx.ccnt;
 
     auto row_of = [&](int l) -> long long {
-        return (long long)((long long)b + (long long)G * (l >> 5)) * kRowBlock + (l & 31);
+        return ONE ? (long long)l
+                   : (long long)((long long)b + (long long)G * (l >> 5)) * kRowBlock + (l & 31);
     };
-    auto owner_of = [&](long long r) -> int { return (int)((r / kRowBlock) % G); };
+    auto owner_of = [&](long long r) -> int { return ONE ? 0 : (int)((r / kRowBlock) % G); };
     auto slot_of = [&](long long r) -> int {
-        return (int)(((r / kRowBlock) / G) * kRowBlock + (r & 31));
+        return ONE ? (int)r : (int)(((r / kRowBlock) / G) * kRowBlock + (r & 31));
     };
     auto cache_load = [&](u64 (&L)[K], int l) {
 #pragma unroll
@@ -1083,167 +1986,95 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
 
     // per-phase wall-clock totals of this CTA (thread 0), when timing is on
     auto &ty = sh.ty;
-    u64 &ph0 = ty.ph[0], &ph1 = ty.ph[1], &ph2 = ty.ph[2], &ph3 = ty.ph[3], &ph4 = ty.ph[4], &ph5 = ty.ph[5];
-    // finer split: ph1 = xs0 (records) + xs1 (walk, installs) + xs2 (chain
-    // sizes, stamps, member cells); ph4 = xs3 (cross-CTA minima) + xs4
-    // (certification) + xs5 (bookkeeping, survivor caches); ph5 = xs6 (pass 2)
-    // + xs7 (owner rescans) + the publish
-    u64 &xs0 = ty.xs[0], &xs1 = ty.xs[1], &xs2 = ty.xs[2], &xs3 = ty.xs[3];
-    u64 &xs4 = ty.xs[4], &xs5 = ty.xs[5], &xs6 = ty.xs[6], &xs7 = ty.xs[7];
-    // ty.xscan: refill scans in the row-log layout (log part, matrix part);
-    // ty.xwalk: the walk itself (warp 0); ty.xlast, ty.nlast: barriers this
-    // CTA completed (arrived last at), its wait then being the barrier's own
-    // latency, with counts of those at B (nlast_b) and of those while serving
-    // a refill scan (at B, at A)
     if (tid == 0) {
         for (int q = 0; q < 6; ++q)
             ty.ph[q] = 0;
         for (int q = 0; q < 8; ++q)
             ty.xs[q] = 0;
-        ty.xscan[0] = ty.xscan[1] = ty.xwalk = ty.xlast = ty.tmark = 0;
+        ty.xscan[0] = ty.xscan[1] = ty.tmark = 0;
         ty.fills = ty.installs = ty.rounds = ty.idle = ty.walk = ty.rescans = 0;
-        ty.nlast = ty.nlast_b = ty.nlast_b_scan = ty.nlast_a_scan = 0;
     }
+    // (the whole of warp 0, every lane with the same values: a branch on the
+    // thread index would leave lane 0 running apart from its warp)
     auto lap = [&](u64 &acc) {
-        if (p.timing && threadIdx.x == 0) {
-            const u64 now = global_ns();
-            acc += now - ty.tmark;
+        if (p.timing && warp == 0) {
+            const u64 now = __shfl_sync(kFull, global_ns(), 0);
+            const u64 was = ty.tmark, sum = acc;
+            __syncwarp();
+            acc = sum + (now - was);
             ty.tmark = now;
+            __syncwarp();
         }
     };
 
-    long long st_updates = 0, st_fill_cells = 0, st_resc_cells = 0;
-
-    // The records of round rr: this CTA's PUB smallest entries (cached keys
-    // and bound marks of its rows) and its refill requests of round rr - 1.
-    // Also lists the refills to install in round rr (served in round rr - 1).
-    auto publish = [&](int rr) {
-        u64 Lst[PUB];
-#pragma unroll
-        for (int q = 0; q < PUB; ++q)
-            Lst[q] = kNoKey;
-        for (int l = tid; l < R; l += NT) {
-            const int c = ccnt[l];
-            const u64 B = cB[l];
-            if (c > 0 || B != kNoKey) {
-                const u64 rowbits = (u64)row_of(l) << 3;
-                // a row's entries ascend: skip the ones that cannot enter
-#pragma unroll
-                for (int q = 0; q < K; ++q) {
-                    if (q < c) {
-                        const u64 e = (ck[(size_t)q * Rmax + l] & kHi) | rowbits | (u64)q;
-                        if (e < Lst[PUB - 1])
-                            list_insert_n(Lst, e);
-                    }
-                }
-                if (B != kNoKey) {
-                    const u64 e = (B & kHi) | rowbits | (u64)c;
-                    if (e < Lst[PUB - 1])
-                        list_insert_n(Lst, e);
-                }
-            }
-            if (rr >= 2 && pend_t[l] == rr - 2) {
-                const int s2 = atomicAdd(&sh.ninst, 1);
-                sh.inst_slot[s2] = l;
-            }
-        }
-        block_topk(Lst, sh);
-        if (tid < PUB) {
-            // entry tid: its column word
-            const u64 key = sh.tko[tid];
-            unsigned col = 0;
-            if (key != kNoKey) {
-                const unsigned lo = (unsigned)key;
-                const int slot = slot_of((long long)(lo >> 3));
-                const int rank = (int)(lo & 7u);
-                col = rank < ccnt[slot] ? (unsigned)ck[(size_t)rank * Rmax + slot] : kRowStop;
-                if (tid == PUB - 1)
-                    col |= kHardStop;  // more entries may follow: none is published
-            }
-            STCG(&p.recA[b].key[tid], key);
-            STCG(&p.recA[b].col[tid], col);
-        }
-        if (tid == 0) {
-            const int par = (rr - 1) & 1;
-            int nq = rr >= 1 ? sh.nmyreq[par] : 0;
-            nq = nq < kReqPerCta ? nq : kReqPerCta;
-            if (rr >= 1)
-                sh.nmyreq[par] = nq;
-            int rows[kReqPerCta];
-#pragma unroll
-            for (int q = 0; q < kReqPerCta; ++q)
-                rows[q] = q < nq ? (int)row_of(sh.myreq_l[par][q]) : -1;
-            uint4 *dst = reinterpret_cast<uint4 *>(&p.recA[b].nreq);
-            STCG(dst + 0, make_uint4((unsigned)nq, (unsigned)rows[0], (unsigned)rows[1], (unsigned)rows[2]));
-            STCG(dst + 1, make_uint4((unsigned)rows[3], (unsigned)rows[4], (unsigned)rows[5], (unsigned)rows[6]));
-            STCG(dst + 2, make_uint4((unsigned)rows[7], 0u, 0u, 0u));
-        }
-    };
+    long long st_fill_cells = 0, st_resc_cells = 0;
 
     // ---- setup
     for (long long w = tid; w < nwords; w += NT) {
         const long long live_n = n - w * 32;
         bitmap[w] = live_n >= 32 ? 0xffffffffu : ((1u << live_n) - 1u);
-        if (G > 1)
-            vpos[w] = 0u;
+        touched[w] = 0u;
     }
     for (int l = tid; l < R; l += NT) {
         rsize[l] = 1;
-        pend_t[l] = -1;
-        rstamp[l] = -1;
-        mflag[l] = 0;
+        if (!ONE) {
+            pend_t[l] = -1;
+            rstamp[l] = -1;
+        }
     }
     for (long long r = (long long)b * NT + tid; r < n; r += (long long)G * NT) {
         STCG(p.size_g + r, 1);
-        if (p.full)
+        if (full)
             STCG(p.stamp + r, -1);
+    }
+    if (!ONE && b == 0 && tid < 2 * kSurv) {
+        STCG(p.svcnt + tid, 0);
+        STCG(p.svovf + tid, kNoKey);
     }
     if (tid == 0) {
         sh.ninst = 0;
+        sh.npieces = 1;
         sh.nexec = 0;
         sh.nmyreq[0] = 0;
         sh.nmyreq[1] = 0;
-        sh.nprev = 0;
+        sh.nps = 0;
+        sh.nptouch = 0;
         sh.nresc = 0;
+        sh.tm.dmax = 0u;
+        sh.pivot = 0ull;
+        sh.ppivot = 0ull;
+        sh.limit = sh.width = 0u;
     }
+    __syncthreads();
 
     // ---- phase 0: validate the matrix and fill the caches of owned rows
     // (one warp per owned row; the rows of a CTA are spread over the whole
     // triangle, so every CTA reads about the same number of cells)
     {
         int bad = 0;
+        unsigned mx = 0u;
         for (int l = warp; l < R; l += W) {
             const long long r = row_of(l);
-            u64 top[K];
+            u64 top[K], next = kNoKey;
 #pragma unroll
             for (int q = 0; q < K; ++q)
                 top[q] = kNoKey;
             if (r < n - 1)
-                warp_row_topk(p, r, top, bad);
+                warp_row_topk(p, r, top, next, bad, mx);
             if (lane == 0) {
                 cache_store(l, top);
-                const int c = list_count(top);
-                ccnt[l] = c;
-                cB[l] = c == K ? top[K - 1] : kNoKey;
+                ccnt[l] = (unsigned char)list_count(top);
+                cB[l] = next;
             }
         }
         if (bad)
             atomicCAS(p.status, 0, kErrInput);
+        mx = __reduce_max_sync(kFull, mx);
+        if (lane == 0)
+            atomicMax(&sh.tm.dmax, mx);
     }
     __syncthreads();
-    publish(0);
-
-    unsigned epoch = 0;
-    if (b == p.skip_arrive_cta)
-        return;
-    grid_arrive(p, epoch);
-    if (!grid_wait(p, epoch, sh))
-        return;
-    if (tid == 0)
-        sh.flag = ld_relaxed_s32(p.status);
-    __syncthreads();
-    if (sh.flag != 0)
-        return;
+    unsigned epoch = 0, epoch2 = 0, epoch3 = 0;
     if (p.timing && tid == 0)
         ty.tmark = global_ns();
 
@@ -1258,33 +2089,40 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 atomicCAS(p.status, 0, kErrInternal);
             return;
         }
+        if (!ONE) {
+            publish(p, sh, r);
+            lap(ty.ph[5]);
+            if (b == p.skip_arrive_cta)
+                return;
+            grid_arrive(p, p.bar, epoch);
+            if (!grid_wait(p, p.bar, epoch, sh))
+                return;
+            lap(ty.ph[0]);
+        }
+        if (r == 0) {
+            // (the input's check)
+            if (tid == 0)
+                sh.flag = ld_relaxed_s32(p.status);
+            __syncthreads();
+            if (sh.flag != 0)
+                return;
+        }
+        if (tid == 0) {
+            sh.nmyreq[par] = 0;
+            sh.ncand = 0;
+            sh.svsum = 0;
+        }
 
-        // ---- A: every CTA's published entries and refill requests
-        {
+        // ---- every CTA's published entries and refill requests
+        if (!ONE) {
+            const RecA *recs = p.recA + (size_t)par * G;
             int rcnt = 0;
             int rq[kReqPerCta];
 #pragma unroll
             for (int q = 0; q < kReqPerCta; ++q)
                 rq[q] = -1;
             if (tid < G) {
-                const RecA *rec = p.recA + tid;
-                const ulonglong2 *ks = reinterpret_cast<const ulonglong2 *>(rec->key);
-#pragma unroll
-                for (int q = 0; q < PUB / 2; ++q) {
-                    const ulonglong2 kk = LDCG(ks + q);
-                    wkey[tid * PUB + 2 * q] = kk.x;
-                    wkey[tid * PUB + 2 * q + 1] = kk.y;
-                }
-                const uint4 *cs = reinterpret_cast<const uint4 *>(rec->col);
-#pragma unroll
-                for (int q = 0; q < PUB / 4; ++q) {
-                    const uint4 cc = LDCG(cs + q);
-                    wcol[tid * PUB + 4 * q] = cc.x;
-                    wcol[tid * PUB + 4 * q + 1] = cc.y;
-                    wcol[tid * PUB + 4 * q + 2] = cc.z;
-                    wcol[tid * PUB + 4 * q + 3] = cc.w;
-                }
-                const uint4 *src = reinterpret_cast<const uint4 *>(&rec->nreq);
+                const uint4 *src = reinterpret_cast<const uint4 *>(&recs[tid].nreq);
                 const uint4 w3 = LDCG(src), w4 = LDCG(src + 1), w5 = LDCG(src + 2);
                 rcnt = (int)w3.x;
                 rq[0] = (int)w3.y;
@@ -1295,1025 +2133,1041 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 rq[5] = (int)w4.z;
                 rq[6] = (int)w4.w;
                 rq[7] = (int)w5.x;
+                if (r == 0)
+                    atomicMax(&sh.tm.dmax, w5.y);
+            }
+            // keys and column words, entry q of CTA g at [q * G + g]
+            constexpr int KW = kPub / 2, CW = kPub / 4;  // 16-byte words of both
+            for (int w = tid; w < (KW + CW) * G; w += NT) {
+                const int g = w / (KW + CW), part = w % (KW + CW);
+                const uint4 v = LDCG(reinterpret_cast<const uint4 *>(recs + g) + part);
+                if (part < KW) {
+                    wkey[(2 * part) * G + g] = ((u64)v.y << 32) | v.x;
+                    wkey[(2 * part + 1) * G + g] = ((u64)v.w << 32) | v.z;
+                } else {
+                    const int q = 4 * (part - KW);
+                    wcol[q * G + g] = v.x;
+                    wcol[(q + 1) * G + g] = v.y;
+                    wcol[(q + 2) * G + g] = v.z;
+                    wcol[(q + 3) * G + g] = v.w;
+                }
             }
             exchange_requests(rcnt, rq, b, sh, par ^ 1, pend_t, pend_s);
+            lap(ty.xs[5]);
         }
-        if (tid == 0)
-            sh.nmyreq[par] = 0;
-        lap(xs0);
+        epoch2 += 1;
 
-        const u64 twalk0 = p.timing && tid == 0 ? global_ns() : 0;
-        if (warp == 0) {
-            // ---- the walk: merge the G published lists in key order.  Lane
-            // l keeps the heads of the lists of CTAs l, l + 32, ... in registers.
-            constexpr int UMAX = 8;  // G <= 256
-            u64 hk[UMAX];
-            int hp[UMAX];
-#pragma unroll
-            for (int u = 0; u < UMAX; ++u) {
-                const int g = lane + 32 * u;
-                hp[u] = 0;
-                hk[u] = g < G ? wkey[g * PUB] : kNoKey;
-            }
-            auto local_min = [&](u64 &lm, int &lu) {
-                lm = hk[0];
-                lu = 0;
-#pragma unroll
-                for (int u = 1; u < UMAX; ++u) {
-                    if (hk[u] < lm) {
-                        lm = hk[u];
-                        lu = u;
-                    }
+        if (!ONE) {
+            // ---- the caches of the previous round's survivors: every cell of a
+            // survivor's row below that round's limit is in its list (those over
+            // the list's size: above svovf) or among the cells to other survivors
+            for (int s = warp; s < sh.nps; s += W) {
+                u64 x = kNoKey, B = kNoKey;
+                const size_t at = (size_t)(par ^ 1) * kSurv + s;
+                const int cnt = LDCG(p.svcnt + at);
+                u64 x2;
+                {
+                    const ulonglong2 y = LDCG(reinterpret_cast<const ulonglong2 *>(p.svlist + at * kSvList) + lane);
+                    x = 2 * lane < cnt ? y.x : kNoKey;
+                    x2 = 2 * lane + 1 < cnt ? y.y : kNoKey;
                 }
-            };
-            u64 lm;
-            int lu;
-            local_min(lm, lu);
-            int np = 0;
-            // member 2a = i_a, 2a + 1 = j_a: lane l holds members l and l + 32
-            int member0 = -1, member1 = -1;
-            unsigned front = 0;  // value bits of the last entry visited
-            // lane a fetches the sizes and stamps of pair a as soon as it is
-            // accepted: they arrive while the walk goes on (asynchronous copies
-            // of the aligned words around them, when the arrays allow it)
-            const bool qa = ((reinterpret_cast<uintptr_t>(p.size_g) |
-                              reinterpret_cast<uintptr_t>(p.stamp)) & 15u) == 0;
-            int q_szi = 0, q_szj = 0, q_si = 0, q_sj = 0;
-            int nwalk = 0;
-            for (int guard = 0; guard <= G * PUB; ++guard) {
-                const u64 m = warp_u64_min(lm);
-                if (m == kNoKey)
-                    break;
-                ++nwalk;
-                front = (unsigned)(m >> 32);
-                const int src = __ffs(__ballot_sync(kFull, lm == m)) - 1;
-                unsigned col = 0;
-                if (lane == src) {
+                u64 x3 = lane < K ? sh.tm.tT[s][lane] : kNoKey;
+                if (lane == K)
+                    B = sh.tm.tB[s];
+                else if (lane == K + 1)
+                    B = LDCG(p.svovf + at);
+                else if (lane == K + 2)
+                    B = sh.limit == 0xffffffffu ? kNoKey : (u64)sh.limit << 32;
+                B = warp_u64_min(B);
+                u64 top[K];
+                int c = 0;
 #pragma unroll
-                    for (int u = 0; u < UMAX; ++u) {
-                        if (u == lu) {
-                            const int g = lane + 32 * u;
-                            col = wcol[g * PUB + hp[u]];
-                            hp[u] += 1;
-                            hk[u] = hp[u] < PUB ? wkey[g * PUB + hp[u]] : kNoKey;
-                        }
-                    }
-                    local_min(lm, lu);
-                }
-                col = __shfl_sync(kFull, col, src);
-                const int row = (int)(((unsigned)m) >> 3);
-                bool stop = (col & kHardStop) != 0;
-                if (!__any_sync(kFull, member0 == row || member1 == row)) {
-                    if (col & kRowStop) {
-                        stop = true;  // the row's smallest untouched cell is unknown
+                for (int q = 0; q <= K; ++q) {
+                    u64 y = x < x2 ? x : x2;
+                    y = x3 < y ? x3 : y;
+                    y = warp_u64_min(y);
+                    x = x == y ? kNoKey : x;
+                    x2 = x2 == y ? kNoKey : x2;
+                    x3 = x3 == y ? kNoKey : x3;
+                    if (q < K) {
+                        top[q < K ? q : 0] = y < B ? y : kNoKey;
+                        c += y < B;
                     } else {
-                        const int c = (int)(col & kColMask);
-                        if (!__any_sync(kFull, member0 == c || member1 == c)) {
-                            if (2 * np < 32) {
-                                if (lane == 2 * np)
-                                    member0 = row;
-                                if (lane == 2 * np + 1)
-                                    member0 = c;
-                            } else {
-                                if (lane == 2 * np - 32)
-                                    member1 = row;
-                                if (lane == 2 * np - 31)
-                                    member1 = c;
-                            }
-                            if (lane == 0) {
-                                sh.pi[np] = row;
-                                sh.pj[np] = c;
-                                sh.ph[np] = __uint_as_float((unsigned)(m >> 32));
-                            }
-                            // (a pair out of range is caught before any other access)
-                            if (lane == np && row >= 0 && row < c && c < n) {
-                                if (qa) {
-                                    // (the arrays are padded to whole 16-byte words)
-                                    int *w = sh.qw[np];
-                                    if (CHECKED_16(p.size_g + (row & ~3)) && CHECKED_16(p.size_g + (c & ~3))) {
-                                        copy16_async(w, p.size_g + (row & ~3));
-                                        copy16_async(w + 4, p.size_g + (c & ~3));
-                                    }
-                                    if (p.full && CHECKED_16(p.stamp + (row & ~3)) && CHECKED_16(p.stamp + (c & ~3))) {
-                                        copy16_async(w + 8, p.stamp + (row & ~3));
-                                        copy16_async(w + 12, p.stamp + (c & ~3));
-                                    }
-                                } else {
-                                    q_szi = LDCG(p.size_g + row);
-                                    q_szj = LDCG(p.size_g + c);
-                                    if (p.full) {
-                                        q_si = LDCG(p.stamp + row);
-                                        q_sj = LDCG(p.stamp + c);
-                                    }
-                                }
-                            }
-                            ++np;
-                            if (np == S)
-                                stop = true;
-                        }
+                        B = y < B ? y : B;
                     }
                 }
-                if (stop)
-                    break;
-            }
-            if (lane == 0) {
-                sh.np = np;
-                sh.front = front;
-                ty.walk += nwalk;
-            }
-            copy_async_wait_all();
-            __syncwarp();
-            if (lane < np) {
-                const int row = sh.pi[lane], c = sh.pj[lane];
-                if (qa && row >= 0 && row < c && c < n) {
-                    // lane a issued pair a's copies, so they are complete
-                    const int *w = sh.qw[lane];
-                    q_szi = w[row & 3];
-                    q_szj = w[4 + (c & 3)];
-                    if (p.full) {
-                        q_si = w[8 + (row & 3)];
-                        q_sj = w[12 + (c & 3)];
+                if (lane == 0) {
+                    atomicAdd(&sh.svsum, cnt < 8 ? cnt : 8);
+#pragma unroll
+                    for (int q = 0; q < K; ++q)
+                        sh.svk[s][q] = top[q];
+                    sh.svB[s] = B;
+                    sh.svc[s] = c;
+                    const long long row = sh.pslot[s];
+                    if (owner_of(row) == b) {
+                        const int l = slot_of(row);
+                        cache_store(l, top);
+                        ccnt[l] = (unsigned char)c;
+                        cB[l] = B;
+                        if (c <= kSurvivorRefillAt && B != kNoKey)
+                            request(l, r);
                     }
                 }
-                sh.szi[lane] = q_szi;
-                sh.szj[lane] = q_szj;
-                sh.si[lane] = q_si;
-                sh.sj[lane] = q_sj;
-                sh.bi[lane] = row_base(p, sh.pi[lane]);  // cell (i, c) at bi + c (packed: for c > i)
-                sh.bj[lane] = row_base(p, sh.pj[lane]);
             }
-            if (p.timing && tid == 0)
-                ty.xwalk += global_ns() - twalk0;
-        } else {
             // ---- refills served in the previous round: take the row's list,
             // then replay that round's merges (the scan ran before them, or
             // while they were being written)
             const int ninst = sh.ninst;
             const int ipar = par ^ 1;
-            for (int s2 = warp - 1; s2 < ninst; s2 += W - 1) {
+            const int inp = sh.npieces;  // pieces per row of the previous round
+            const int nps = sh.nps;
+            for (int s2 = W - 1 - warp; s2 < ninst; s2 += W) {
                 const int l = sh.inst_slot[s2];
                 const int pos = pend_s[l];
-                const long long row = row_of(l);
-                u64 M[K];
-                {
-                    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(
-                        p.parts + ((size_t)ipar * kMaxReq + pos) * K);
-#pragma unroll
-                    for (int q = 0; q < K / 2; ++q) {
-                        const ulonglong2 v = LDCG(src + q);
-                        M[2 * q] = v.x;
-                        M[2 * q + 1] = v.y;
-                    }
+                if (inp == 0) {
+                    if (lane == 0)
+                        pend_t[l] = -1;  // no list: the row may ask again
+                    continue;
                 }
-                // the new cells (row, i_a) of the previous round's merges, one lane each
-                const int np2 = sh.nprev;
+                const long long row = row_of(l);
+                // (one key per lane, kPartWords lanes per piece, then the K smallest
+                // of them; B, a lower bound of the row's other cells)
+                u64 M[K], B;
+                {
+                    const int q1 = lane % kPartWords;
+                    u64 x = kNoKey;
+                    if (lane < inp * kPartWords && q1 <= K)
+                        x = LDCG(p.parts + ((size_t)ipar * kMaxReq + pos) * kPieces * kPartWords + lane);
+                    u64 y = q1 < K ? x : kNoKey;
+#pragma unroll
+                    for (int q = 0; q < K; ++q) {
+                        M[q] = warp_u64_min(y);
+                        y = y == M[q] ? kNoKey : y;
+                    }
+                    B = warp_u64_min(q1 == K ? x : y);
+                }
+                // the new cells (row, survivor) of the previous round, one lane each
                 const long long base = row_base(p, row);  // cell (row, c) at base + c
                 u64 xr = kNoKey;
-                if (lane < np2) {
-                    const long long ia = sh.ppi[lane];
+                if (lane < nps) {
+                    const long long ia = sh.pslot[lane];
                     if (ia > row)
-                        xr = make_key(LDCG(p.full ? p.D + ia * p.pitch + row : p.D + base + ia), (unsigned)ia);
+                        xr = make_key(LDCG(full ? p.D + ia * p.pitch + row : p.D + base + ia), (unsigned)ia);
                 }
-                u64 xs[S];
+                // keys whose column a merge of that round retired or rewrote go
 #pragma unroll
-                for (int a = 0; a < S; ++a)
-                    xs[a] = __shfl_sync(kFull, xr, a);
-                // keys whose column a merge of that round retired or rewrote
-                const int c0 = list_count(M);
-                const u64 B0 = c0 == K ? M[K - 1] : kNoKey;
-                const int mi = lane < np2 ? sh.ppi[lane] : -1;
-                const int mj = lane < np2 ? sh.ppj[lane] : -1;
-#pragma unroll
-                for (int q = 0; q < K; ++q) {
-                    const int col = (int)(unsigned)M[q];
-                    if (__any_sync(kFull, M[q] != kNoKey && (col == mi || col == mj)))
+                for (int q = 0; q < K; ++q)
+                    if (M[q] != kNoKey && live(touched, (unsigned)M[q]))
                         M[q] = kNoKey;
+                sort_list(M);
+                int c = list_count(M);
+                for (unsigned w = __ballot_sync(kFull, xr < B); w; w &= w - 1) {
+                    const u64 x = __shfl_sync(kFull, xr, __ffs(w) - 1);
+                    if (x < B) {
+                        const u64 out = list_insert(M, x);
+                        if (c == K)
+                            B = out;
+                        else
+                            ++c;
+                    }
                 }
                 if (lane == 0) {
-                    u64 B = B0;
-                    sort_list(M);
-                    int c = list_count(M);
-#pragma unroll
-                    for (int a = 0; a < S; ++a) {
-                        const u64 x = xs[a];
-                        if (x != kNoKey && x <= B) {
-                            list_insert(M, x);
-                            if (c == K)
-                                B = M[K - 1];
-                            else
-                                ++c;
-                        }
-                    }
                     cache_store(l, M);
-                    ccnt[l] = c;
+                    ccnt[l] = (unsigned char)c;
                     cB[l] = B;
                     pend_t[l] = -1;
                 }
             }
-            if (tid == 32)
+            if (tid == TA)
                 ty.installs += ninst;
+            __syncthreads();
+        }
+        // (the previous round's bits; the selection's barriers follow)
+        for (int q = tid; q < sh.nptouch; q += NT)
+            atomicAnd(&touched[sh.ptouch[q] >> 5], ~(1u << (sh.ptouch[q] & 31)));
+        lap(ty.xs[0]);
+
+        // Team A's barrier (the whole CTA in a one-CTA job).
+        auto sync_a = [&]() {
+            if constexpr (ONE)
+                __syncthreads();
+            else
+                asm volatile("barrier.cta.sync.aligned 3, %0;" ::"n"(TA) : "memory");
+        };
+        // The selection's threads: the whole CTA, or (long rows: their scans take
+        // longer than the rest of a round, so team B begins at once) team A.
+        const int TS = early ? TA : NT;
+        auto sync_s = [&]() {
+            if constexpr (ONE)
+                __syncthreads();
+            else
+                asm volatile("barrier.cta.sync.aligned 5, %0;" ::"r"(TS) : "memory");
+        };
+        auto count_s = [&](bool x) -> int {
+            if constexpr (ONE) {
+                return __syncthreads_count(x);
+            } else {
+                unsigned c;
+                asm volatile("{ .reg .pred q; setp.ne.u32 q, %1, 0; barrier.cta.red.popc.aligned.u32 %0, 5, %2, q; }"
+                             : "=r"(c)
+                             : "r"((unsigned)x), "r"(TS)
+                             : "memory");
+                return (int)c;
+            }
+        };
+        int bad = 0;
+        if (!early || warp < WA) {
+            // ---- selection: a pivot such that the entries up to it number some
+            // fifty to a hundred.  A thread's head is its smallest entry.
+            {
+                u64 head = kNoKey, hard = kNoKey;
+                if (ONE) {
+                    for (int l = tid; l < R; l += TS) {
+                        const int c = ccnt[l];
+                        const u64 B = cB[l];
+                        if (c > 0 || B != kNoKey) {
+                            const u64 e = entry_key(c > 0 ? ck[l] : B, (u64)l << kRankBits, 0);
+                            head = e < head ? e : head;
+                        }
+                    }
+                } else {
+                    for (int g = tid; g < G; g += TS) {
+                        const u64 x = wkey[g], y = wkey[(kPub - 1) * G + g];  // (a list that is full may go on)
+                        head = x < head ? x : head;
+                        hard = y < hard ? y : hard;
+                    }
+                }
+                // survivors' heads (every warp counts them itself)
+                u64 svh = kNoKey;
+                const int nps = ONE ? 0 : sh.nps;
+                if (lane < nps && (sh.svc[lane] > 0 || sh.svB[lane] != kNoKey))
+                    svh = entry_key(sh.svc[lane] > 0 ? sh.svk[lane][0] : sh.svB[lane],
+                                    (u64)sh.pslot[lane] << kRankBits, 0);
+                {
+                    const u64 x = warp_u64_min(head), y = warp_u64_min(hard);
+                    if (lane == 0) {
+                        sh.wmin[warp][0] = x;
+                        sh.wmin[warp][1] = y;
+                    }
+                }
+                sync_s();
+                u64 gmin = warp_u64_min(32 * lane < TS ? sh.wmin[lane][0] : kNoKey);
+                hard = warp_u64_min(32 * lane < TS ? sh.wmin[lane][1] : kNoKey);
+                const u64 sv = warp_u64_min(svh);
+                gmin = sv < gmin ? sv : gmin;
+                auto count = [&](u64 x) -> int {
+                    return count_s(head <= x && head != kNoKey) +
+                           (ONE ? 0 : __popc(__ballot_sync(kFull, svh <= x && svh != kNoKey)));
+                };
+                u64 pivot = hard;
+                int want = kHeadsHi;
+                while (true) {
+                    pivot = find_pivot(count, gmin, hard, sh.pivot, want * 5 / 8, want);
+                    // every entry up to the pivot: counted per thread, placed by a
+                    // scan of the warp and one addition per warp
+                    int have = 0, svn = 0;
+                    const bool svw = !ONE && 32 * (warp + 1) == TS;
+                    if (head <= pivot && head != kNoKey) {
+                        if (ONE) {
+                            for (int l = tid; l < R; l += TS) {
+                                const int cc = ccnt[l];
+                                const u64 B = cB[l];
+                                const u64 rowbits = (u64)l << kRankBits;
+                                for (int q = 0; q < cc; ++q)
+                                    have += entry_key(ck[(size_t)q * Rmax + l], rowbits, q) <= pivot;
+                                have += B != kNoKey && entry_key(B, rowbits, cc) <= pivot;
+                            }
+                        } else {
+                            for (int g = tid; g < G; g += TS) {
+#pragma unroll
+                                for (int q = 0; q < kPub; ++q) {
+                                    const u64 e = wkey[q * G + g];
+                                    have += e <= pivot && e != kNoKey;
+                                }
+                            }
+                        }
+                    }
+                    if (svw && svh <= pivot && svh != kNoKey) {
+                        const u64 rowbits = (u64)sh.pslot[lane] << kRankBits;
+                        const int cc = sh.svc[lane];
+                        const u64 B = sh.svB[lane];
+                        for (int q = 0; q < cc; ++q)
+                            svn += entry_key(sh.svk[lane][q], rowbits, q) <= pivot;
+                        svn += B != kNoKey && entry_key(B, rowbits, cc) <= pivot;
+                    }
+                    int at = have + svn;
+#pragma unroll
+                    for (int off = 1; off < 32; off <<= 1) {
+                        const int o = __shfl_up_sync(kFull, at, off);
+                        if (lane >= off)
+                            at += o;
+                    }
+                    {
+                        int base = 0;
+                        if (lane == 31 && at > 0)
+                            base = atomicAdd(&sh.ncand, at);
+                        base = __shfl_sync(kFull, base, 31);
+                        at = base + at - (have + svn);
+                    }
+                    auto put = [&](u64 key, unsigned col) {
+                        if (at < kCand) {
+                            sh.ckey[at] = key;
+                            sh.ccol[at] = col;
+                        }
+                        ++at;
+                    };
+                    if (have > 0) {
+                        if (ONE) {
+                            for (int l = tid; l < R; l += TS) {
+                                const int cc = ccnt[l];
+                                const u64 B = cB[l];
+                                const u64 rowbits = (u64)l << kRankBits;
+                                for (int q = 0; q < cc; ++q) {
+                                    const u64 x = ck[(size_t)q * Rmax + l];
+                                    const u64 e = entry_key(x, rowbits, q);
+                                    if (e > pivot)
+                                        break;
+                                    put(e, (unsigned)x);
+                                }
+                                if (B != kNoKey && entry_key(B, rowbits, cc) <= pivot)
+                                    put(entry_key(B, rowbits, cc), kRowStop | (unsigned)B);
+                            }
+                        } else {
+                            for (int g = tid; g < G; g += TS) {
+                                for (int q = 0; q < kPub; ++q) {
+                                    const u64 e = wkey[q * G + g];
+                                    if (e > pivot || e == kNoKey)
+                                        break;
+                                    put(e, wcol[q * G + g]);
+                                }
+                            }
+                        }
+                    }
+                    if (svn > 0) {
+                        const u64 rowbits = (u64)sh.pslot[lane] << kRankBits;
+                        const int cc = sh.svc[lane];
+                        const u64 B = sh.svB[lane];
+                        for (int q = 0; q < cc; ++q) {
+                            const u64 x = sh.svk[lane][q];
+                            const u64 e = entry_key(x, rowbits, q);
+                            if (e <= pivot)
+                                put(e, (unsigned)x);
+                        }
+                        if (B != kNoKey && entry_key(B, rowbits, cc) <= pivot)
+                            put(entry_key(B, rowbits, cc), kRowStop | (unsigned)B);
+                    }
+                    sync_s();
+                    if (sh.ncand <= kCand)
+                        break;
+                    // too many entries behind so few heads: take fewer heads
+                    want = want / 2 > 1 ? want / 2 : 1;
+                    sync_s();
+                    if (tid == 0)
+                        sh.ncand = 0;
+                    hard = pivot;
+                    sync_s();
+                }
+                const int N = sh.ncand;
+                // key order by counting (entries are distinct), four threads per entry
+                for (int c0 = (tid >> 5) * 8; c0 < N; c0 += TS / 4) {
+                    const int c = c0 + (lane >> 2);
+                    const u64 key = c < N ? sh.ckey[c] : kNoKey;
+                    int rank = 0;
+                    for (int f = lane & 3; f < N; f += 4)
+                        rank += sh.ckey[f] < key;
+                    rank += __shfl_xor_sync(kFull, rank, 1);
+                    rank += __shfl_xor_sync(kFull, rank, 2);
+                    if (c < N && (lane & 3) == 0 && rank <= kEntries) {
+                        sh.ekey[rank] = key;
+                        sh.erc[rank] = make_uint2((unsigned)key >> kRankBits, sh.ccol[c]);
+                    }
+                }
+                if (tid == 0)
+                    sh.pivot = pivot;
+                sync_s();
+                // which entries bring a row or column that no earlier one has
+                const int E = N < kEntries ? N : kEntries;
+                // (eight threads per entry)
+                for (int c0 = (tid >> 5) * 4; c0 < E; c0 += TS / 8) {
+                    const int e = c0 + (lane >> 3);
+                    const uint2 w = e < E ? sh.erc[e] : make_uint2(0u, 0u);
+                    const unsigned row = w.x, col = w.y & kColMask;
+                    int in = 0;
+                    for (int f = lane & 7; f < e; f += 8) {
+                        const uint2 o = sh.erc[f];
+                        const unsigned fc = o.y & kColMask;
+                        const bool mark = (o.y & kRowStop) != 0;  // (a mark brings no member)
+                        in |= !mark && (o.x == row || fc == row) ? 1 : 0;
+                        in |= !mark && (o.x == col || fc == col) ? 2 : 0;
+                    }
+                    in |= __shfl_xor_sync(kFull, in, 1);
+                    in |= __shfl_xor_sync(kFull, in, 2);
+                    in |= __shfl_xor_sync(kFull, in, 4);
+                    if (e < E && (lane & 7) == 0) {
+                        if (w.y & kHardStop)
+                            sh.enew[e] = 4;
+                        else if (w.y & kRowStop)
+                            sh.enew[e] = (in & 1) ? 0 : 4;
+                        else
+                            sh.enew[e] = (unsigned char)(~in & 3);
+                    }
+                }
+                sync_s();
+                if (warp == 0) {
+                    // the selection ends at the bound of a row without a member, at the
+                    // last entry of a CTA (the ones behind it are not known), at kTeam
+                    // members, or with the list; lane l looks at two entries
+                    const int e0 = 2 * lane;
+                    const int f0 = e0 < E ? sh.enew[e0] : 4, f1 = e0 + 1 < E ? sh.enew[e0 + 1] : 4;
+                    const int a0 = __popc(f0 & 3), a1 = __popc(f1 & 3);
+                    int inc = a0 + a1;
+#pragma unroll
+                    for (int off = 1; off < 32; off <<= 1) {
+                        const int o = __shfl_up_sync(kFull, inc, off);
+                        if (lane >= off)
+                            inc += o;
+                    }
+                    int at = inc - a0 - a1, stop = kEntries;
+                    if ((f1 & 4) || inc > kTeam)
+                        stop = e0 + 1;
+                    if ((f0 & 4) || at + a0 > kTeam)
+                        stop = e0;
+                    stop = (int)__reduce_min_sync(kFull, (unsigned)stop);
+                    // entries left out of a list that ends at a pivot lie above its last
+                    const bool cut = stop == E && N <= kEntries && pivot != kNoKey;
+                    if (cut && E >= 2)
+                        stop = E - 1;
+                    int mm = 0;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int f = q ? f1 : f0;
+                        if (e0 + q < stop) {
+                            const uint2 w = sh.erc[e0 + q];
+                            if (f & 1)
+                                sh.umem[at++] = (int)w.x;
+                            if (f & 2)
+                                sh.umem[at++] = (int)(w.y & kColMask);
+                            mm = at;
+                        }
+                    }
+                    mm = (int)__reduce_max_sync(kFull, (unsigned)mm);
+                    if (lane == 0) {
+                        sh.tm.ne = stop;
+                        sh.tm.m = mm;
+                        // every cell not listed is at or above the first entry not taken
+                        u64 A = kNoKey;
+                        unsigned C = 0xffffffffu;
+                        if (stop < N) {
+                            A = (sh.ekey[stop] & kHi) | sh.erc[stop].x;
+                            C = sh.erc[stop].y & kColMask;
+                        } else if (cut && E == 1) {
+                            A = (sh.ekey[0] & kHi) | sh.erc[0].x;
+                            C = (sh.erc[0].y & kColMask) + 1u;
+                        }
+                        sh.tm.thA = A;
+                        sh.tm.thC = C;
+                        const unsigned tv = (unsigned)(A >> 32);
+                    sh.tm.thv = tv;
+                    if (!ONE) {
+                        // survivors' cells below a limit above the bound are listed;
+                        // its distance follows the lists' lengths
+                        const unsigned v0 = E > 0 ? (unsigned)(sh.ekey[0] >> 32) : tv;
+                        unsigned w = sh.width;
+                        if (w == 0u)
+                            w = tv > v0 && tv < 0x7f800000u ? 8u * min(tv - v0, 0x100000u) : 0u;
+                        else if (nps > 0 && sh.svsum < 4 * nps)
+                            w += w / 2;
+                        else if (nps > 0 && sh.svsum > 6 * nps)
+                            w -= w / 4;
+                        sh.width = w = min(max(w, 64u), 0x4000000u);
+                        sh.limit = tv < 0x7f000000u ? min(tv + w, 0x7f800000u) : 0xffffffffu;
+                    }
+                        ty.walk += stop;
+                    }
+                }
+                sync_s();
+            }
+            const int m = sh.tm.m, ne = sh.tm.ne;
+            {
+                // members in slot order, with their sizes, stamps and bounds: eight
+                // threads per member
+                for (int a0 = (tid >> 5) * 4; a0 < m; a0 += TS / 8) {
+                    const int a = a0 + (lane >> 3), part = lane & 7;
+                    const int x = a < m ? sh.umem[a] : -1;
+                    const bool in = x >= 0 && x < n;
+                    bad |= a < m && !in;
+                    int sz = 0, st = 0;
+                    if (part == 0 && in) {
+                        sz = LDCG(p.size_g + x);
+                        if (full)
+                            st = LDCG(p.stamp + x);
+                    }
+                    int rank = 0;
+                    for (int q = part; q < m; q += 8)
+                        rank += sh.umem[q] < x;
+                    u64 A = kNoKey;
+                    unsigned C = 0u, ex = 0xffu;
+                    for (int e = part; e < ne; e += 8) {
+                        const uint2 w = sh.erc[e];
+                        if ((w.y & kRowStop) && w.x == (unsigned)x) {
+                            A = (sh.ekey[e] & kHi) | (unsigned)x;
+                            C = w.y & kColMask;
+                            ex = (unsigned)e;
+                        }
+                    }
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) {
+                        rank += __shfl_xor_sync(kFull, rank, o);
+                        ex = min(ex, __shfl_xor_sync(kFull, ex, o));
+                        const u64 A2 = __shfl_xor_sync(kFull, A, o);
+                        const unsigned C2 = __shfl_xor_sync(kFull, C, o);
+                        if (A2 < A) {
+                            A = A2;
+                            C = C2;
+                        }
+                    }
+                    if (part == 0 && in) {
+                        sh.tm.mem[rank] = x;
+                        sh.tm.sz0[rank] = sz;
+                        sh.tm.em[rank] = 0ull;
+                        {
+                            const unsigned lv = (unsigned)(A >> 32), tv = sh.tm.thv;
+                            sh.tm.sl[rank] = make_int2(sz, (int)(lv < tv ? lv : tv));
+                        }
+                        sh.tm.mst[rank] = st;
+                        sh.tm.mbase[rank] = row_base(p, x);
+                        sh.tm.lbA[rank] = A;
+                        sh.tm.lbC[rank] = C;
+                        sh.tm.ex[rank] = (unsigned char)ex;
+                    }
+                }
+            }
+            // every CTA read the same records and selected the same way, so every
+            // CTA takes this exit together
+            bad = count_s(bad != 0);
+            {
+                // the entries by member (eight threads per entry)
+                for (int c0 = (tid >> 5) * 4; c0 < ne; c0 += TS / 8) {
+                    const int e = c0 + (lane >> 3);
+                    const uint2 w = e < ne ? sh.erc[e] : make_uint2(0u, kRowStop);
+                    unsigned at = 0xffffu;
+                    if (!(w.y & kRowStop)) {
+                        const int row = (int)w.x, col = (int)(w.y & kColMask);
+                        at = 0u;
+                        for (int a = lane & 7; a < m; a += 8) {
+                            const int x = sh.tm.mem[a];
+                            at |= x == row ? (unsigned)a : x == col ? (unsigned)a << 8 : 0u;
+                        }
+                    }
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1)
+                        at |= __shfl_xor_sync(kFull, at, o);
+                    if (e < ne && (lane & 7) == 0) {
+                        sh.tm.ent[e] = make_uint2(at, (unsigned)(sh.ekey[e] >> 32));
+                        if (at != 0xffffu) {
+                            atomicOr(&sh.tm.em[at & 0xffu], 1ull << e);
+                            atomicOr(&sh.tm.em[at >> 8], 1ull << e);
+                        }
+                    }
+                }
+                sync_s();
+                lap(ty.xs[1]);
+            }
+        }
+        {
+            if (warp < WA && bad) {
+                if (tid == 0) {
+                    atomicCAS(p.status, 0, kErrInternal);
+                    sh.flag = kErrInternal;
+                }
+                if constexpr (ONE)
+                    __syncthreads();
+                else
+                    asm volatile("barrier.cta.sync.aligned 3, %0;\n\tbarrier.cta.arrive.aligned 4, %1;" ::"n"(TA), "n"(NT)
+                                 : "memory");
+            } else if (warp < WA) {
+                const int m = sh.tm.m;
+                // ---- the cells between members: pair (a, a + d mod kTeam); warp 0
+                // takes the chain while its loads are on their way
+                const int linkage = p.linkage;
+                const bool chain = linkage != 0 && linkage != 5;
+                constexpr int ALL = kTeam * kTeam / 2, U = (ALL + TA - 1) / TA > 8 ? 8 : (ALL + TA - 1) / TA;
+                for (int e0 = tid; e0 < ALL; e0 += U * TA) {
+                    float v[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int e = e0 + u * TA;
+                        const int a = e & (kTeam - 1), c = (a + (e / kTeam) + 1) & (kTeam - 1);
+                        v[u] = 0.0f;
+                        if (e < ALL && a < m && c < m)
+                            v[u] = member_cell(p, sh.tm.mem[a], sh.tm.mst[a], sh.tm.mem[c], sh.tm.mst[c]);
+                    }
+                    if (chain && warp == 0 && e0 == tid)
+                        chain_select(sh.tm);
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int e = e0 + u * TA;
+                        const int a = e & (kTeam - 1), c = (a + (e / kTeam) + 1) & (kTeam - 1);
+                        if (e < ALL && a < m && c < m) {
+                            sh.tm.S[a][c] = v[u];
+                            sh.tm.S[c][a] = v[u];
+                        }
+                    }
+                }
+                sync_a();
+                // (nobody rewrites a member's cell, size or stamp before every CTA got here)
+                if (!ONE && tid == 0)
+                    red_release_add(p.bar + kBar2, 1u);
+                if (full) {
+                    // the lines of the members' rows that the merges will read
+                    const int nblk = R / 32;
+                    for (int e = tid; e < m * nblk; e += TA) {
+                        const long long k = row_of((e / m) * 32);
+                        const float *line = p.D + sh.tm.mbase[e % m] + k;
+                        if (k < n && CHECK_PREFETCH(line))
+                            prefetch_l2(line);
+                    }
+                }
+                lap(ty.xs[2]);
+                if (chain)
+                    chain_phase<NT, ONE>(sh.tm, linkage, Rmax <= CH);
+                if (!chain || sh.tm.redo) {
+                    // per member row (columns above it): which cells are at or below
+                    // the bound, and the smallest of them
+                    const unsigned thv = sh.tm.thv;
+                    for (int a = warp; a < m; a += WA) {
+                        const unsigned v0 = __float_as_uint(sh.tm.S[a][lane]);
+                        const unsigned v1 = __float_as_uint(sh.tm.S[a][lane + 32]);
+                        const bool o0 = lane > a && lane < m && v0 <= thv;
+                        const bool o1 = lane + 32 > a && lane + 32 < m && v1 <= thv;
+                        const unsigned b0 = __ballot_sync(kFull, o0), b1 = __ballot_sync(kFull, o1);
+                        unsigned v = 0xffffffffu, c = 0xffffffffu;
+                        if (b0 | b1) {
+                            const unsigned w0 = o0 ? v0 : 0xffffffffu, w1 = o1 ? v1 : 0xffffffffu;
+                            v = __reduce_min_sync(kFull, w0 < w1 ? w0 : w1);
+                            const unsigned k0 = o0 && v0 == v ? (unsigned)lane : 64u;
+                            const unsigned k1 = o1 && v1 == v ? (unsigned)lane + 32u : 64u;
+                            c = (unsigned)a << 8 | __reduce_min_sync(kFull, k0 < k1 ? k0 : k1);
+                        }
+                        if (lane == 0) {
+                            sh.tm.nnv[a] = v;
+                            sh.tm.nnc[a] = c;
+                            sh.tm.mask[a] = ((u64)b1 << 32) | b0;
+                        }
+                    }
+                    sync_a();
+                    if (warp == 0)
+                        simulate(sh.tm, linkage);
+                }
+                sync_a();
+                lap(ty.xs[3]);
+                // the merges wait until every CTA holds the members' cells; then the
+                // slots they take part in are marked, and slot j retires (Section 4
+                // step 2)
+                if (grid_wait(p, p.bar + kBar2, epoch2, sh, sync_a)) {
+                    const int L = sh.tm.L;
+                    for (int q = tid; q < 2 * L; q += TA) {
+                        const int x = sh.tm.mem[q < L ? sh.tm.mi(q) : sh.tm.mj(q - L)];
+                        atomicOr(&touched[x >> 5], 1u << (x & 31));
+                        if (q >= L)
+                            atomicAnd(&bitmap[x >> 5], ~(1u << (x & 31)));
+                    }
+                }
+                if (tid == 0) {
+                    sh.item = 0;
+                    sh.viol = kSurv;
+                }
+                if constexpr (ONE)
+                    __syncthreads();
+                else
+                    asm volatile("barrier.cta.sync.aligned 3, %0;\n\tbarrier.cta.arrive.aligned 4, %1;" ::"n"(TA), "n"(NT)
+                                 : "memory");
+                lap(ty.ph[3]);
+            } else if constexpr (!ONE) {
+            constexpr int TB = NT - TA;
             // ---- the refills asked for in the previous round, served now by
-            // warps 1.. while warp 0 walks (row s of the list by CTA
-            // G - 1 - s mod G: rows are owned in blocks of 32 from CTA 0 up,
-            // so the last CTAs own a block fewer and take the scans first):
-            // the K smallest keys of the row over live columns, as the
-            // previous round left it; the owner installs the list at the start
-            // of the next round and replays this round's merges on it
-            constexpr int TB = NT - 32;
+            // team B (row s of the list by CTA G - 1 - s mod G: rows are
+            // owned in blocks of 32 from CTA 0 up, so the last CTAs own a block
+            // fewer and take the scans first): the K smallest keys of the row
+            // over live columns.  Other CTAs may already be writing this
+            // round's merges: the columns those touch are dropped when the
+            // owner installs the list and replays the round.
+            // A row is cut in pieces when there are CTAs for them: a whole row
+            // scanned by one CTA outlasts the steps beside it, and every other
+            // CTA would wait for it.
             const int nexec = sh.nexec;
-            const bool cols_ok = ((reinterpret_cast<uintptr_t>(p.D) | reinterpret_cast<uintptr_t>(p.stamp)) & 15u) == 0;
-            for (int s2 = G - 1 - b; s2 < nexec; s2 += G) {
+            const int np = scan_pieces(G, nexec, early);
+            for (int w = G - 1 - b; w < nexec * np; w += G) {
+                const int s2 = w / np, piece = w % np;
                 const long long rr = sh.exec_row[s2];
                 if (rr < 0 || rr >= n - 1)
                     continue;  // the same for every thread of the team
-                if (p.full && cols_ok)
-                    block_row_topk_cols<NT, S, TB>(p, rr, bitmap, sh, st_fill_cells, p.timing ? ty.xscan : nullptr);
-                else if (p.full)
-                    block_row_topk_log<NT, S, TB>(p, rr, bitmap, vpos, newer, sh, t, 0, st_fill_cells,
-                                                  p.timing ? ty.xscan : nullptr);
+                if (full)
+                    block_row_topk_cols<NT, ONE, TB>(p, rr, piece, np, (int)t, bitmap, sh, st_fill_cells,
+                                                     p.timing ? ty.xscan : nullptr);
                 else
-                    block_row_topk<NT, S, TB>(p, rr, bitmap, sh, st_fill_cells);
-                if (tid - 32 < K / 2) {
-                    const int h = tid - 32;
-                    ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(p.parts + ((size_t)par * kMaxReq + s2) * K);
-                    STCG(dst + h, make_ulonglong2(sh.tko[2 * h], sh.tko[2 * h + 1]));
-                }
+                    block_row_topk<NT, ONE, TB>(p, rr, piece, np, bitmap, sh, st_fill_cells);
+                if (tid - TA < K + 1)
+                    STCG(p.parts + (((size_t)par * kMaxReq + s2) * kPieces + piece) * kPartWords + (tid - TA),
+                         tid - TA < K ? sh.tko[tid - TA] : sh.tnext);
             }
-            if (tid == 32)
+            if (tid == TA)
                 ty.fills += nexec;
-        }
-        __syncthreads();
-        lap(xs1);
-        const int s = sh.np;
-        {
-            // every CTA read the same records and walked them the same way, so
-            // every CTA takes this exit together
-            int bad = 0;
-            if (tid < s) {
-                const int i = sh.pi[tid], j = sh.pj[tid];
-                bad = !(i >= 0 && i < j && j < n);
+            // (team A does not wait: it begins with the new cells)
+            asm volatile("barrier.cta.sync.aligned 4, %0;" ::"n"(NT) : "memory");
             }
-            if (__syncthreads_or(bad)) {
+        }
+        if (sh.flag != 0)
+            return;  // (a wait ran out, here or in another CTA)
+        lap(ty.ph[2]);
+        const int m = sh.tm.m;
+        int L = sh.tm.L, ns = sh.tm.ns;
+        const bool tie = sh.tm.tie != 0;
+
+
+        // ---- apply the L merges to every live row k outside them, a chunk of
+        // rows at a time; per chunk (1) the new cells D(k, survivor) of
+        // Section 4 step 3, a warp per 32 rows and 8 survivors, stored and kept
+        // in kvs, (2) per survivor the smallest of them above it, NT / kSurv
+        // threads each, and the rows' caches, a thread each
+        auto bookkeeping = [&]() {
+            if (!ONE && b == 0 && tid < kSurv) {
+                // (every CTA has read the previous round's lists)
+                STCG(p.svcnt + (par ^ 1) * kSurv + tid, 0);
+                STCG(p.svovf + (par ^ 1) * kSurv + tid, kNoKey);
                 if (tid == 0)
-                    atomicCAS(p.status, 0, kErrInternal);
-                return;
+                    STCG(p.bar + kViol + (par ^ 1), 0u);
             }
-        }
-
-        // ---- the chain's sizes, member flags and the cells between members
-        for (int e = tid; e < W * S; e += NT) {
-            sh.wam[e / S][e % S] = kNoKey;
-            sh.whm[e / S][e % S] = kNoKey;
-        }
-        if (tid < 2 * s) {
-            const long long m = (tid & 1) ? sh.pj[tid >> 1] : sh.pi[tid >> 1];
-            if (owner_of(m) == b)
-                mflag[slot_of(m)] = 1;
-        }
-        // the cells between members of different pairs: loaded now, landed in
-        // shared memory after pass 1 (member u = 2a + (0 for i_a, 1 for j_a))
-        // (more than eight per thread go to shared memory at once)
-        constexpr int DMALL = (4 * S * S + NT - 1) / NT;
-        constexpr bool DM_REG = DMALL <= 8;
-        constexpr int DMR = DM_REG ? DMALL : 1;
-        float dmv[DMR];
-        if (DM_REG) {
-#pragma unroll
-            for (int q = 0; q < DMR; ++q) {
-                const int e = tid + q * NT;
-                const int u = e / (2 * S), v = e % (2 * S);
-                dmv[q] = 0.0f;
-                if (e < 4 * S * S && u < v && v < 2 * s && (u >> 1) != (v >> 1)) {
-                    const long long mu = (u & 1) ? sh.pj[u >> 1] : sh.pi[u >> 1];
-                    const long long mv = (v & 1) ? sh.pj[v >> 1] : sh.pi[v >> 1];
-                    const int su = (u & 1) ? sh.sj[u >> 1] : sh.si[u >> 1];
-                    const int sv = (v & 1) ? sh.sj[v >> 1] : sh.si[v >> 1];
-                    dmv[q] = member_cell(p, mu, su, mv, sv);
+            if (b == 0) {
+                for (int q = tid; q < L; q += NT) {
+                    STCG(p.merges + 2 * (t + q), (int32_t)sh.tm.mem[sh.tm.mi(q)]);
+                    STCG(p.merges + 2 * (t + q) + 1, (int32_t)sh.tm.mem[sh.tm.mj(q)]);
+                    STCG(p.heights + t + q, __int_as_float(sh.tm.rec[q].y));
+                }
+                if (tid < ns)
+                    STCG(p.size_g + sh.tm.sslot[tid], sh.tm.rec[sh.tm.sq[tid]].z + sh.tm.rec[sh.tm.sq[tid]].w);
+            }
+            for (int q = tid; q < 2 * L; q += NT) {
+                const int x = sh.tm.mem[q < L ? sh.tm.mi(q) : sh.tm.mj(q - L)];
+                if (owner_of(x) == b) {
+                    const int l = slot_of(x);
+                    ccnt[l] = 0;
+                    cB[l] = kNoKey;
+                    if (!ONE)
+                        pend_t[l] = -1;
                 }
             }
-        } else {
-            for (int e = tid; e < 4 * S * S; e += NT) {
-                const int u = e / (2 * S), v = e % (2 * S);
-                if (u < v && v < 2 * s && (u >> 1) != (v >> 1)) {
-                    const long long mu = (u & 1) ? sh.pj[u >> 1] : sh.pi[u >> 1];
-                    const long long mv = (v & 1) ? sh.pj[v >> 1] : sh.pi[v >> 1];
-                    const int su = (u & 1) ? sh.sj[u >> 1] : sh.si[u >> 1];
-                    const int sv = (v & 1) ? sh.sj[v >> 1] : sh.si[v >> 1];
-                    const float d = member_cell(p, mu, su, mv, sv);
-                    sh.Dm[u][v] = d;
-                    sh.Dm[v][u] = d;
+            if (tid < ns) {
+                const int x = sh.tm.sslot[tid];
+                sh.pslot[tid] = x;
+                const int tq = (int)(t + sh.tm.sq[tid]);
+                // row-log layout: the last merge rewrites row x (every CTA writes the
+                // same value, so each one sees the new stamps in its own rescans)
+                if (full)
+                    STCG(p.stamp + x, tq);
+                if (owner_of(x) == b) {
+                    const int l = slot_of(x);
+                    rsize[l] = sh.tm.rec[sh.tm.sq[tid]].z + sh.tm.rec[sh.tm.sq[tid]].w;
+                    if (!ONE)
+                        rstamp[l] = tq;
                 }
             }
-        }
-        __syncthreads();
-        lap(xs2);
-
-        // ---- pass 1: new cells of every live k outside the chain (reads only),
-        // the pairs in groups of 16; the values of each thread's first row are
-        // kept in shared memory for pass 2
-        constexpr int PG = 16;
-        // up to 16 pairs the values stay in registers; more go to shared memory
-        constexpr bool KV_REG = S <= PG;
-        float kv[KV_REG ? S : 1];
+            if (tid == 0) {
+                sh.ninst = 0;
+                sh.nps = ns;
+                if (!ONE)
+                    // (a scan beside merges that were put off again may have left
+                    // their columns out: its list is dropped)
+                    sh.npieces = sh.viol < sh.tm.L ? 0 : scan_pieces(G, sh.nexec, early);
+            }
+            // slots to clear from `touched` after the next round
+            for (int a = tid; a < m; a += NT)
+                sh.ptouch[a] = sh.tm.mem[a];
+            if (tid == 0)
+                sh.nptouch = m;
+        };
+        constexpr int TPP = NT / kSurv;
+        const int ra = tid / TPP, rpart = tid % TPP;
+        u64 ps[P];
 #pragma unroll
-        for (int a = 0; a < (KV_REG ? S : 1); ++a)
-            kv[a] = 0.0f;
-        bool kok = false;
-        constexpr int PC = 8;  // pairs whose cells one thread loads at once
-        if constexpr (S > PG) {
-            // every owned row's new cells, a chunk of NT rows at a time (the
-            // last chunk first, so chunk 0 stays in kvs for pass 2); after each
-            // chunk, NT / S threads per pair take its smallest new cell over
-            // the chunk's rows (all k and k > i_a), then reduce across lanes
-            constexpr int TPP = NT / S;
-            const int ra = tid / TPP, rpart = tid % TPP;
-            u64 ma = kNoKey, mh = kNoKey;
-            if (s > 0) {
-                for (int l0 = ((R - 1) / NT) * NT; l0 >= 0; l0 -= NT) {
-                    const int l = l0 + tid;
-                    bool ok = false;
-                    long long k = 0;
-                    if (l < R) {
-                        k = row_of(l);
-                        ok = k < n && live(bitmap, k) && !mflag[l];
-                    }
-                    okf[tid] = ok;
-                    if (ok) {
-                        const int nk = rsize[l];
-                        const long long bk = row_base(p, k);
-                        const bool full = p.full;
-                        const int sk = full ? rstamp[l] : 0;
-                        float *kr = kvs + (size_t)tid * KVP;
-#pragma unroll 1
-                        for (int a0 = 0; a0 < s; a0 += PC) {
-                            float va[PC], vb[PC];
-#pragma unroll
-                            for (int u = 0; u < PC; ++u) {
-                                const int a = a0 + u;
-                                va[u] = 0.0f;
-                                vb[u] = 0.0f;
-                                if (a < s) {
-                                    if (full) {
-                                        va[u] = LDCG(sh.si[a] >= sk ? p.D + sh.bi[a] + k : p.TL + sh.bi[a] + sk);
-                                        vb[u] = LDCG(sh.sj[a] >= sk ? p.D + sh.bj[a] + k : p.TL + sh.bj[a] + sk);
-                                    } else {
-                                        const long long i = sh.pi[a], j = sh.pj[a];
-                                        va[u] = LDCG(p.D + (k > i ? sh.bi[a] + k : bk + i));
-                                        vb[u] = LDCG(p.D + (k > j ? sh.bj[a] + k : bk + j));
-                                    }
-                                }
-                            }
-#pragma unroll
-                            for (int u = 0; u < PC; ++u) {
-                                const int a = a0 + u;
-                                if (a < s)
-                                    kr[a] = lw_cell(p.linkage, va[u], vb[u], sh.ph[a], sh.szi[a], sh.szj[a], nk);
-                            }
-                        }
-                    }
-                    __syncthreads();
-                    if (ra < s) {
-                        const long long ia = sh.pi[ra];
-                        for (int q = rpart; q < NT && l0 + q < R; q += TPP) {
-                            if (!okf[q])
-                                continue;
-                            const long long kq = row_of(l0 + q);
-                            const u64 key = make_key(kvs[(size_t)q * KVP + ra], (unsigned)kq);
-                            ma = key < ma ? key : ma;
-                            if (kq > ia && key < mh)
-                                mh = key;
-                        }
-                    }
+        for (int q = 0; q < P; ++q)
+            ps[q] = kNoKey;
+        for (int l0 = 0; l0 < R; l0 += CH) {
+            const int rows = R - l0 < CH ? R - l0 : CH;
+            bool wait = tie;
+            while (true) {
+                new_cells(p, sh, l0, rows, ns, L, wait);
+                __syncthreads();
+                lap(ty.xs[4]);
+                if (!wait)
+                    break;
+                // the merges taken on condition: has any CTA found a cell that comes
+                // before one of them?
+                if (!ONE) {
+                    if (tid == 0 && sh.viol < L)
+                        atomicMax(p.bar + kViol + par, (unsigned)(kSurv - sh.viol));
+                    grid_arrive(p, p.bar + kBar3, epoch3);
+                    if (!grid_wait(p, p.bar + kBar3, epoch3, sh))
+                        return;
+                    if (tid == 0)
+                        sh.viol = kSurv - ld_relaxed_s32(reinterpret_cast<const int *>(p.bar + kViol + par));
                     __syncthreads();
                 }
-            }
-#pragma unroll
-            for (int o = TPP / 2; o > 0; o >>= 1) {
-                const u64 x = __shfl_xor_sync(kFull, ma, o);
-                const u64 y = __shfl_xor_sync(kFull, mh, o);
-                ma = x < ma ? x : ma;
-                mh = y < mh ? y : mh;
-            }
-            if (rpart == 0) {
-                STCG(p.recB + (size_t)b * 2 * kRound + ra, ma);
-                STCG(p.recB + (size_t)b * 2 * kRound + kRound + ra, mh);
-            }
-        } else if (s > 0) {
-            for (int l0 = 0; l0 < R; l0 += NT) {
-                const int l = l0 + tid;
-                bool ok = false;
-                long long k = 0;
-                int nk = 1;
-                if (l < R) {
-                    k = row_of(l);
-                    ok = k < n && live(bitmap, k) && !mflag[l];
-                    if (ok)
-                        nk = rsize[l];
-                }
-                // cell (k, i): packed, row i for k > i (consecutive k of a warp
-                // read consecutive words) and row k for k < i; row-log layout,
-                // row i of M when i was stamped no earlier than k, else i's
-                // log at k's stamp (words of one contiguous range)
-                const long long bk = row_base(p, k);
-                const bool full = p.full;
-                const int sk = full && l < R ? rstamp[l] : 0;
-#pragma unroll
-                for (int a0 = 0; a0 < S; a0 += PG) {
-                    if (a0 >= s)
-                        break;
-                    float va[PG], vb[PG];
-#pragma unroll
-                    for (int u = 0; u < PG; ++u) {
-                        const int a = a0 + u;
-                        va[u] = 0.0f;
-                        vb[u] = 0.0f;
-                        if (ok && a < s) {
-                            const long long i = sh.pi[a], j = sh.pj[a];
-                            if (full) {
-                                va[u] = LDCG(sh.si[a] >= sk ? p.D + sh.bi[a] + k : p.TL + sh.bi[a] + sk);
-                                vb[u] = LDCG(sh.sj[a] >= sk ? p.D + sh.bj[a] + k : p.TL + sh.bj[a] + sk);
-                            } else {
-                                va[u] = LDCG(p.D + (k > i ? sh.bi[a] + k : bk + i));
-                                vb[u] = LDCG(p.D + (k > j ? sh.bj[a] + k : bk + j));
-                            }
-                        }
+                const int V = sh.viol;
+                if (V >= L) {
+                    for (int it = warp; it < rows / 32 * ns; it += W) {
+                        const int blk = it / ns, s = it % ns;
+                        const int l = l0 + blk * 32 + lane;
+                        const long long k = row_of(l), x = sh.tm.sslot[s];
+                        if ((sh.okm[blk] >> lane) & 1u)
+                            STCG(full ? p.D + x * p.pitch + k : p.D + (k > x ? row_base(p, x) + k : row_base(p, k) + x),
+                                 kvs[(size_t)(blk * 32 + lane) * KVP + s]);
                     }
-#pragma unroll
-                    for (int u = 0; u < PG; ++u) {
-                        const int a = a0 + u;
-                        if (a >= s)
-                            break;
-                        u64 ka = kNoKey, kh = kNoKey;
-                        if (ok) {
-                            const float v = lw_cell(p.linkage, va[u], vb[u], sh.ph[a], sh.szi[a], sh.szj[a], nk);
-                            if (l0 == 0) {
-                                kv[KV_REG ? a : 0] = v;
-                            }
-                            ka = make_key(v, (unsigned)k);
-                            if (k > sh.pi[a])
-                                kh = ka;
-                        }
-                        // a warp's rows are one block of 32 consecutive k: unless the
-                        // block holds i_a, "k > i_a" is all of it or none of it
-                        const long long k0 = (long long)(b + (long long)G * (l >> 5)) * kRowBlock;
-                        const u64 ma = warp_u64_min(ka);
-                        u64 mh;
-                        if (k0 > sh.pi[a])
-                            mh = ma;
-                        else if (k0 + kRowBlock <= sh.pi[a])
-                            mh = kNoKey;
-                        else
-                            mh = warp_u64_min(kh);
-                        // each warp keeps its own minima (no shared-memory atomics)
-                        if (lane == 0) {
-                            if (ma < sh.wam[warp][a])
-                                sh.wam[warp][a] = ma;
-                            if (mh < sh.whm[warp][a])
-                                sh.whm[warp][a] = mh;
-                        }
-                    }
-                }
-                if (l0 == 0)
-                    kok = ok;
-            }
-        }
-        if (DM_REG) {
-#pragma unroll
-            for (int q = 0; q < DMR; ++q) {
-                const int e = tid + q * NT;
-                const int u = e / (2 * S), v = e % (2 * S);
-                if (e < 4 * S * S && u < v && v < 2 * s && (u >> 1) != (v >> 1)) {
-                    sh.Dm[u][v] = dmv[q];
-                    sh.Dm[v][u] = dmv[q];
-                }
-            }
-        }
-        if constexpr (S <= PG) {
-            __syncthreads();
-            if (tid < 2 * S) {
-                // this CTA's minima per pair: over its warps
-                const int a = tid % S;
-                u64 m = kNoKey;
-                for (int w = 0; w < W; ++w) {
-                    const u64 x = tid < S ? sh.wam[w][a] : sh.whm[w][a];
-                    m = x < m ? x : m;
-                }
-                STCG(p.recB + (size_t)b * 2 * kRound + (tid < S ? tid : kRound + tid - S), m);
-            }
-        }
-        lap(ph2);
-        bool last_b = false;
-        grid_arrive(p, epoch, p.timing ? &last_b : nullptr);
-
-        // ---- window of barrier B: the cells (i_a, i_b) and (i_a, j_b) after
-        // merge a alone, then (i_a, i_b) after merges a and b (read only after
-        // barrier B)
-        for (int e = tid; e < s * s; e += NT) {
-            const int a = e / s, c = e % s;
-            if (a != c) {
-                sh.X[a][c] = lw_cell(p.linkage, sh.Dm[2 * c][2 * a], sh.Dm[2 * c][2 * a + 1], sh.ph[a],
-                                     sh.szi[a], sh.szj[a], sh.szi[c]);
-                sh.Y[a][c] = lw_cell(p.linkage, sh.Dm[2 * c + 1][2 * a], sh.Dm[2 * c + 1][2 * a + 1],
-                                     sh.ph[a], sh.szi[a], sh.szj[a], sh.szj[c]);
-            }
-        }
-        __syncthreads();
-        for (int e = tid; e < s * s; e += NT) {
-            const int a = e / s, c = e % s;
-            if (a < c)
-                sh.C[a][c] = lw_cell(p.linkage, sh.X[a][c], sh.Y[a][c], sh.ph[c], sh.szi[c], sh.szj[c],
-                                     sh.szi[a] + sh.szj[a]);
-        }
-        lap(ph3);
-        const u64 twb = p.timing && tid == 0 ? global_ns() : 0;
-        if (!grid_wait(p, epoch, sh))
-            return;
-        if (p.timing && tid == 0 && last_b) {
-            ty.xlast += global_ns() - twb;
-            ++ty.nlast;
-            ++ty.nlast_b;
-            ty.nlast_b_scan += G - 1 - b < sh.nexec;
-        }
-        lap(ph0);
-
-        // ---- B: the global per-pair minima, then the certified prefix
-        if (s > 0) {
-            const int a = tid % S;
-            u64 ma = kNoKey, mh = kNoKey;
-            if (a < s) {
-                for (int g = tid / S; g < G; g += NT / S) {
-                    const u64 x = LDCG(p.recB + (size_t)g * 2 * kRound + a);
-                    const u64 y = LDCG(p.recB + (size_t)g * 2 * kRound + kRound + a);
-                    ma = x < ma ? x : ma;
-                    mh = y < mh ? y : mh;
-                }
-            }
-#pragma unroll
-            for (int o = S; o < 32; o <<= 1) {
-                const u64 x = __shfl_xor_sync(kFull, ma, o);
-                const u64 y = __shfl_xor_sync(kFull, mh, o);
-                ma = x < ma ? x : ma;
-                mh = y < mh ? y : mh;
-            }
-            // lanes below S of every warp hold the warp's minima per pair
-            if (lane < S) {
-                sh.wam[warp][lane] = ma;
-                sh.whm[warp][lane] = mh;
-            }
-            __syncthreads();
-            if (tid < 2 * S) {
-                const int a2 = tid % S;
-                u64 m = kNoKey;
-                for (int w = 0; w < W; ++w) {
-                    const u64 x = tid < S ? sh.wam[w][a2] : sh.whm[w][a2];
-                    m = x < m ? x : m;
-                }
-                if (tid < S)
-                    sh.gamin[a2] = m;
-                else
-                    sh.ghmin[a2] = m;
-            }
-        }
-        __syncthreads();
-        lap(xs3);
-        // certification: P_p is accepted when it is smaller than every cell
-        // that merges a < p rewrote, as seen after merge p - 1: for merge a,
-        // its published minimum over the other rows, the cells (i_a, i_c) and
-        // (i_a, j_c) after merge a alone for the pairs c >= p not merged yet,
-        // and (i_a, i_c) after merges a and c for a < c < p.  Warp per row a,
-        // lane c: the first term by a suffix minimum over the lanes, the second
-        // by an exclusive prefix minimum, so candidate R(a, p) sits in lane p;
-        // then warp per p, lane a: the minimum over a < p.  (R is kept in the
-        // member-cell table, whose values the round no longer needs.)
-        {
-            static_assert(sizeof(float) * 2 * S * (2 * S + 1) >= 12 * S * S, "candidates fit the member-cell table");
-            u64 *RA = reinterpret_cast<u64 *>(&sh.Dm[0][0]);
-            unsigned *Rc = reinterpret_cast<unsigned *>(RA + S * S);
-            const Cand none = {kNoKey, 0xffffffffu};
-            for (int a = warp; a + 1 < s; a += W) {  // (row s - 1 rewrites nothing a later p sees)
-                const int c = lane;
-                const bool in = c > a && c < s;
-                Cand xy = none, cc = none;
-                if (in) {
-                    const unsigned ia = (unsigned)sh.pi[a];
-                    xy = cell_cand(__float_as_uint(sh.X[a][c]), ia, (unsigned)sh.pi[c]);
-                    cand_min(xy, cell_cand(__float_as_uint(sh.Y[a][c]), ia, (unsigned)sh.pj[c]));
-                    cc = cell_cand(__float_as_uint(sh.C[a][c]), ia, (unsigned)sh.pi[c]);
-                }
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    Cand y, z;
-                    y.A = __shfl_down_sync(kFull, xy.A, d);
-                    y.c = __shfl_down_sync(kFull, xy.c, d);
-                    z.A = __shfl_up_sync(kFull, cc.A, d);
-                    z.c = __shfl_up_sync(kFull, cc.c, d);
-                    if (lane + d < 32)
-                        cand_min(xy, y);
-                    if (lane >= d)
-                        cand_min(cc, z);
-                }
-                Cand e;
-                e.A = __shfl_up_sync(kFull, cc.A, 1);
-                e.c = __shfl_up_sync(kFull, cc.c, 1);
-                if (in) {
-                    cand_min(xy, lane >= 1 ? e : none);
-                    const u64 g = sh.gamin[a];
-                    if (g != kNoKey)
-                        cand_min(xy, cell_cand((unsigned)(g >> 32), (unsigned)sh.pi[a], (unsigned)g));
-                    RA[a * S + c] = xy.A;
-                    Rc[a * S + c] = xy.c;
-                }
-            }
-            __syncthreads();
-            for (int pp = 1 + warp; pp < s; pp += W) {
-                Cand M = none;
-                if (lane < pp) {
-                    M.A = RA[lane * S + pp];
-                    M.c = Rc[lane * S + pp];
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    Cand y;
-                    y.A = __shfl_xor_sync(kFull, M.A, o);
-                    y.c = __shfl_xor_sync(kFull, M.c, o);
-                    cand_min(M, y);
-                }
-                if (lane == 0) {
-                    const u64 PA = ((u64)__float_as_uint(sh.ph[pp]) << 32) | (unsigned)sh.pi[pp];
-                    const unsigned Pc = (unsigned)sh.pj[pp];
-                    sh.okp[pp] = PA < M.A || (PA == M.A && Pc < M.c);
-                }
-            }
-        }
-        __syncthreads();
-        if (tid == 0) {
-            int L = s;
-            for (int pp = 1; pp < s; ++pp) {
-                if (!sh.okp[pp]) {
-                    L = pp;
                     break;
                 }
-            }
-            sh.nacc = L;
-            sh.ninst = 0;
-        }
-        __syncthreads();
-        const int L = sh.nacc;
-        lap(xs4);
-
-        // ---- bookkeeping of the L merges
-        if (b == 0) {
-            if (tid < L) {
-                STCG(p.merges + 2 * (t + tid), (int32_t)sh.pi[tid]);
-                STCG(p.merges + 2 * (t + tid) + 1, (int32_t)sh.pj[tid]);
-                STCG(p.heights + t + tid, sh.ph[tid]);
-                STCG(p.size_g + sh.pi[tid], sh.szi[tid] + sh.szj[tid]);
-            }
-            for (int e = tid; e < L * L; e += NT) {
-                const int a = e / L, c = e % L;
-                if (a < c) {
-                    if (p.full) {
-                        // merge c, the later one, rewrites row i_c; i_a's log at merge c
-                        STCG(p.D + (long long)sh.pi[c] * p.pitch + sh.pi[a], sh.C[a][c]);
-                        STCG(p.TL + (long long)sh.pi[a] * p.pitch + t + c, sh.C[a][c]);
-                    } else {
-                        STCG(p.D + pair_idx(sh.pi[a], sh.pi[c], n), sh.C[a][c]);
-                    }
+                // the merges from V on wait for another round
+                for (int q = V + tid; q < L; q += NT) {
+                    const int x = sh.tm.mem[sh.tm.mi(q)], y = sh.tm.mem[sh.tm.mj(q)];
+                    atomicAnd(&touched[x >> 5], ~(1u << (x & 31)));
+                    atomicAnd(&touched[y >> 5], ~(1u << (y & 31)));
+                    atomicOr(&bitmap[y >> 5], 1u << (y & 31));
                 }
+                L = ns = V;
+                wait = false;
+                if (tid == 0) {
+                    sh.tm.sfirst[V] = V;
+                    sh.item = 0;
+                }
+                __syncthreads();
             }
-            // each pair a < c stands for three updates of the step-by-step
-            // order: merge a rewrites (i_a, i_c) and (i_a, j_c), merge c (i_c, i_a)
-            if (tid == 0)
-                st_updates += 3LL * L * (L - 1) / 2;
-        }
-        if (tid < L) {
-            const int j = sh.pj[tid];
-            atomicAnd(&bitmap[j >> 5], ~(1u << (j & 31)));  // Section 4 step 2: slot j retires
-            // row-log layout: merge t + tid rewrites row i (every CTA writes the
-            // same value, so each one sees the new stamps in its own rescans)
-            if (p.full) {
-                STCG(p.stamp + sh.pi[tid], (int)(t + tid));
-                // the members' earlier merges are no longer the latest; this one is
-                const int si = sh.si[tid], sj = sh.sj[tid];
-                if (si >= 0)
-                    atomicAnd(&vpos[si >> 5], ~(1u << (si & 31)));
-                if (sj >= 0)
-                    atomicAnd(&vpos[sj >> 5], ~(1u << (sj & 31)));
-                const long long q = t + tid;
-                atomicOr(&vpos[q >> 5], 1u << (q & 31));
-            }
-        }
-        if (tid >= 2 * L && tid < 2 * s) {
-            const long long m = (tid & 1) ? sh.pj[tid >> 1] : sh.pi[tid >> 1];
-            if (owner_of(m) == b)
-                mflag[slot_of(m)] = 0;  // proposed but not merged this round
-        }
-        if (tid < L) {
-            const int a = tid;
-            const long long ja = sh.pj[a];
-            if (owner_of(ja) == b) {
-                const int l = slot_of(ja);
-                ccnt[l] = 0;
-                cB[l] = kNoKey;
-                pend_t[l] = -1;
-            }
-            const long long ia = sh.pi[a];
-            if (G == 1) {
-                // a job's only CTA sees every write after pass 2: it rescans
-                // the survivor row then
-                const int l = slot_of(ia);
-                ccnt[l] = 0;
-                cB[l] = kNoKey;
-                rsize[l] = sh.szi[a] + sh.szj[a];
-                pend_t[l] = -1;
-                rlist[atomicAdd(&sh.nresc, 1)] = l;
-            } else if (owner_of(ia) == b) {
-                // the survivor's cache: its smallest new cell outside the chain
-                // and, below it, the new cells to chain members
-                const int l = slot_of(ia);
-                rstamp[l] = (int)(t + a);
-                const u64 m = sh.ghmin[a];
-                u64 M[K];
+            if (l0 == 0) {
+                bookkeeping();
+                // the survivors' smallest cells to other survivors (those to the other
+                // members are among their owners' new cells), a lane each
+                for (int s = warp; s < ns; s += W) {
+                    u64 x = kNoKey;
+                    if (lane < ns && sh.tm.sslot[lane] > sh.tm.sslot[s])
+                        x = make_key(sh.tm.C[s][lane], (unsigned)sh.tm.sslot[lane]);
 #pragma unroll
-                for (int q = 0; q < K; ++q)
-                    M[q] = kNoKey;
-                int ncand = 0;
-                for (int c = 0; c < s; ++c) {
-                    if (c == a)
-                        continue;
-                    u64 x0 = kNoKey, x1 = kNoKey;
-                    if (c < L) {
-                        if (sh.pi[c] > ia)
-                            x0 = make_key(a < c ? sh.C[a][c] : sh.C[c][a], (unsigned)sh.pi[c]);
-                    } else {
-                        if (sh.pi[c] > ia)
-                            x0 = make_key(sh.X[a][c], (unsigned)sh.pi[c]);
-                        if (sh.pj[c] > ia)
-                            x1 = make_key(sh.Y[a][c], (unsigned)sh.pj[c]);
-                    }
-                    if (x0 != kNoKey && x0 < m) {
-                        list_insert(M, x0);
-                        ++ncand;
-                    }
-                    if (x1 != kNoKey && x1 < m) {
-                        list_insert(M, x1);
-                        ++ncand;
+                    for (int q = 0; q <= K; ++q) {
+                        const u64 y = warp_u64_min(x);
+                        x = x == y ? kNoKey : x;
+                        if (lane == 0) {
+                            if (q < K)
+                                sh.tm.tT[s][q] = y;
+                            else
+                                sh.tm.tB[s] = y;  // bounds the others
+                        }
                     }
                 }
-                int c;
-                u64 B;
-                if (m != kNoKey) {
-                    list_insert(M, m);
-                    c = list_count(M);
-                    B = M[c - 1];
-                } else {
-                    c = list_count(M);
-                    B = ncand > K ? M[K - 1] : kNoKey;
+                if (b == 0) {
+                    for (int e = tid; e < ns * ns; e += NT) {
+                        const int x = e / ns, y = e % ns;
+                        if (x < y) {  // (the later last merge has the larger index)
+                            const float v = sh.tm.C[x][y];
+                            if (full) {
+                                STCG(p.D + (long long)sh.tm.sslot[y] * p.pitch + sh.tm.sslot[x], v);
+                                STCG(p.TL + (long long)sh.tm.sslot[x] * p.pitch + t + sh.tm.sq[y], v);
+                            } else {
+                                STCG(p.D + pair_idx(sh.tm.sslot[x], sh.tm.sslot[y], n), v);
+                            }
+                        }
+                    }
                 }
-                cache_store(l, M);
-                ccnt[l] = c;
-                cB[l] = B;
-                rsize[l] = sh.szi[a] + sh.szj[a];
-                pend_t[l] = -1;
-                // a survivor holds little more than its smallest cell: ask for
-                // its row now (other rows wait until their cache empties)
-                if (c <= kSurvivorRefillAt && B != kNoKey)
-                    request(l, r);
             }
-        }
-        __syncthreads();
-        lap(xs5);
-
-        // ---- pass 2: apply the L merges to every live k outside them (in a
-        // round without merges it only renews refill requests that the
-        // per-round cap turned away: a row waiting for one may hold every
-        // later round up)
-        {
-            for (int l0 = 0; l0 < R; l0 += NT) {
-                const int l = l0 + tid;
-                bool ok = false;
-                long long k = 0;
-                int nk = 1;
-                if (l < R) {
-                    k = row_of(l);
-                    ok = k < n && live(bitmap, k) && !mflag[l];
-                    if (ok)
-                        nk = rsize[l];
+            if (full) {
+                // row k's log at the survivors' last merges, from kvs: lane per
+                // survivor, so a row's words of the round go out together (by
+                // rows they would be one sector each)
+                const int sq = lane < ns ? sh.tm.sq[lane] : 0;
+                for (int q = warp; q < rows; q += W) {
+                    if (lane < ns && ((sh.okm[q >> 5] >> (q & 31)) & 1u))
+                        STCG(p.TL + row_of(l0 + q) * p.pitch + t + sq, kvs[(size_t)q * KVP + lane]);
                 }
-                if (!ok)
+            }
+            if (ra < ns) {
+                const long long ia = sh.tm.sslot[ra];
+#pragma unroll 4
+                for (int q = rpart; q < rows; q += TPP) {
+                    const unsigned vb = __float_as_uint(kvs[(size_t)q * KVP + ra]);
+                    const bool in = (sh.okm[q >> 5] >> (q & 31)) & 1u;
+                    if (ONE) {
+                        if (in && vb <= (unsigned)(ps[P - 1] >> 32)) {
+                            const long long kq = row_of(l0 + q);
+                            const u64 key = ((u64)vb << 32) | (unsigned)kq;
+                            if (kq > ia && key < ps[P - 1])
+                                list_insert_n(ps, key);
+                        }
+                    } else if (in && vb < sh.limit) {
+                        const long long kq = row_of(l0 + q);
+                        if (kq > ia) {
+                            const size_t at = (size_t)par * kSurv + ra;
+                            const u64 key = ((u64)vb << 32) | (unsigned)kq;
+                            const int e = atomicAdd(p.svcnt + at, 1);
+                            if (e < kSvList)
+                                STCG(p.svlist + at * kSvList + e, key);
+                            else
+                                atomicMin(p.svovf + at, key);
+                        }
+                    }
+                }
+            }
+            for (int q = tid; q < rows; q += NT) {
+                const int l = l0 + q;
+                const long long k = row_of(l);
+                if (!(k < n && live(bitmap, k) && !live(touched, k)))
                     continue;
-                // rows outside the chain kept their pass-1 values; rows of
-                // pairs the round did not merge, and rows past the first
-                // chunk, compute them now
-                const long long bk = row_base(p, k);
-                const bool full = p.full;
-                const int sk = full ? rstamp[l] : 0;
-                u64 Cc[K];
-                cache_load(Cc, l);
                 int c = ccnt[l];
                 u64 B = cB[l];
-                // merge a gave row k the new cell v = D(k, i_a + j_a): store it
-                // and keep the cache
-                auto apply = [&](int a, float v) {
-                    const long long ia = sh.pi[a], ja = sh.pj[a];
-                    if (full) {
-                        // row i_a is rewritten whole; row k keeps its stale copy
-                        // and the new value goes to k's log at this merge
-                        STCG(p.D + sh.bi[a] + k, v);
-                        STCG(p.TL + bk + t + a, v);
-                    } else {
-                        STCG(p.D + (k > ia ? sh.bi[a] + k : bk + ia), v);
-                    }
-                    ++st_updates;
-                    if (k < ja) {
-                        // row k loses column j; if k < i its cell (k, i) changed as well
-                        bool drop = false;
+                if (ns > 0) {
+                    u64 Cc[K];
+                    cache_load(Cc, l);
+                    bool drop = false;
 #pragma unroll
-                        for (int q = 0; q < K; ++q) {
-                            const long long col = (long long)(unsigned)Cc[q];
-                            if (Cc[q] != kNoKey && (col == ja || (k < ia && col == ia))) {
-                                Cc[q] = kNoKey;
-                                drop = true;
-                            }
-                        }
-                        if (drop) {
-                            close_holes(Cc);
-                            c = list_count(Cc);
-                        }
-                        if (k < ia) {
-                            const u64 x = make_key(v, (unsigned)ia);
-                            if (x <= B) {
-                                list_insert(Cc, x);
-                                if (c == K)
-                                    B = Cc[K - 1];
-                                else
-                                    ++c;
-                            }
+                    for (int e = 0; e < K; ++e) {
+                        if (Cc[e] != kNoKey && live(touched, (unsigned)Cc[e])) {
+                            Cc[e] = kNoKey;
+                            drop = true;
                         }
                     }
-                };
-                if constexpr (S > PG) {
-                    if (l0 == 0 && okf[tid]) {
-                        const float *kr = kvs + (size_t)tid * KVP;
-#pragma unroll 1
-                        for (int a = 0; a < L; ++a)
-                            apply(a, kr[a]);
-                    } else {
-#pragma unroll 1
-                        for (int a0 = 0; a0 < L; a0 += PC) {
-                            float va[PC], vb[PC];
-#pragma unroll
-                            for (int u = 0; u < PC; ++u) {
-                                const int a = a0 + u;
-                                va[u] = 0.0f;
-                                vb[u] = 0.0f;
-                                if (a < L) {
-                                    if (full) {
-                                        va[u] = LDCG(sh.si[a] >= sk ? p.D + sh.bi[a] + k : p.TL + sh.bi[a] + sk);
-                                        vb[u] = LDCG(sh.sj[a] >= sk ? p.D + sh.bj[a] + k : p.TL + sh.bj[a] + sk);
-                                    } else {
-                                        const long long i = sh.pi[a], j = sh.pj[a];
-                                        va[u] = LDCG(p.D + (k > i ? sh.bi[a] + k : bk + i));
-                                        vb[u] = LDCG(p.D + (k > j ? sh.bj[a] + k : bk + j));
-                                    }
-                                }
-                            }
-#pragma unroll
-                            for (int u = 0; u < PC; ++u) {
-                                const int a = a0 + u;
-                                if (a < L)
-                                    apply(a, lw_cell(p.linkage, va[u], vb[u], sh.ph[a], sh.szi[a], sh.szj[a], nk));
-                            }
+                    bool dirty = drop;
+                    if (drop) {
+                        sort_list(Cc);
+                        c = list_count(Cc);
+                    }
+                    const float *kr = kvs + (size_t)q * KVP;
+#pragma unroll 4
+                    for (int s = 0; s < ns; ++s) {
+                        const unsigned vb = __float_as_uint(kr[s]);
+                        if (vb > (unsigned)(B >> 32))
+                            continue;
+                        const long long x = sh.tm.sslot[s];
+                        const u64 key = ((u64)vb << 32) | (unsigned)x;
+                        if (x > k && key < B) {
+                            const u64 out = list_insert(Cc, key);
+                            dirty = true;
+                            if (c == K)
+                                B = out;
+                            else
+                                ++c;
                         }
                     }
-                } else {
-                    const bool have = l0 == 0 && kok;
-#pragma unroll
-                    for (int a0 = 0; a0 < S; a0 += PG) {
-                        if (a0 >= L)
-                            break;
-                        float va[PG], vb[PG];
-#pragma unroll
-                        for (int u = 0; u < PG; ++u) {
-                            const int a = a0 + u;
-                            va[u] = 0.0f;
-                            vb[u] = 0.0f;
-                            if (!have && a < L) {
-                                const long long i = sh.pi[a], j = sh.pj[a];
-                                va[u] = LDCG(p.D + (k > i ? sh.bi[a] + k : bk + i));
-                                vb[u] = LDCG(p.D + (k > j ? sh.bj[a] + k : bk + j));
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < PG; ++u) {
-                            const int a = a0 + u;
-                            if (a >= L)
-                                break;
-                            apply(a, have ? kv[KV_REG ? a : 0]
-                                          : lw_cell(p.linkage, va[u], vb[u], sh.ph[a], sh.szi[a], sh.szj[a], nk));
-                        }
+                    if (dirty) {
+                        cache_store(l, Cc);
+                        ccnt[l] = (unsigned char)c;
+                        cB[l] = B;
                     }
                 }
-                cache_store(l, Cc);
-                ccnt[l] = c;
-                cB[l] = B;
-                if (G == 1) {
+                if (ONE) {
                     // one CTA: no one else to ask, refill right after this pass
-                    if (c <= kRefillAt && B != kNoKey)
+                    if (c == 0 && B != kNoKey)
                         rlist[atomicAdd(&sh.nresc, 1)] = l;
-                } else if (c == 0 && B != kNoKey && (unsigned)(B >> 32) <= sh.front) {
+                } else if (c == 0 && B != kNoKey && (unsigned)(B >> 32) <= sh.tm.thv) {
                     // live cells remain, none is cached, and the bound sits at
-                    // the front of the merges: its bare stop mark would hold
-                    // the next rounds up until a refill lands, so rescan now
+                    // the front of the merges: its bare mark would hold the next
+                    // rounds up until a refill lands, so rescan now
                     rlist[atomicAdd(&sh.nresc, 1)] = l;
                     pend_t[l] = -1;
-                } else if (c <= kRefillAt && B != kNoKey && pend_t[l] < 0) {
+                } else if (c <= refill_at && B != kNoKey && pend_t[l] < 0) {
                     // (a cache that holds every live cell of its row needs no refill)
                     request(l, r);
                 }
             }
+            if (l0 + CH < R) {
+                if (tid == 0)
+                    sh.item = 0;
+                __syncthreads();
+            }
+        }
+        // a one-CTA job: per survivor, over the TPP threads
+        if constexpr (ONE) {
+            __syncthreads();  // (the members' lists)
+            u64 out[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q)
+                out[q] = ps[q];
+#pragma unroll
+            for (int o = TPP / 2; o > 0; o >>= 1) {
+                u64 x[P];
+#pragma unroll
+                for (int q = 0; q < P; ++q)
+                    x[q] = __shfl_xor_sync(kFull, out[q], o);
+#pragma unroll
+                for (int q = 0; q < P; ++q)
+                    list_insert_n(out, x[q]);
+            }
+            {
+                // the smallest cells of the survivor's row: to other rows (the last of
+                // out bounds the rest) and to survivors
+                if (ra < ns && rpart == 0) {
+                    const int l = slot_of(sh.tm.sslot[ra]);
+                    u64 M[K], next = out[P - 1];
+#pragma unroll
+                    for (int q = 0; q < K; ++q)
+                        M[q] = out[q < P - 1 ? q : 0];
+#pragma unroll
+                    for (int q = 0; q < K; ++q) {
+                        const u64 x = list_insert(M, sh.tm.tT[ra][q]);
+                        next = x < next ? x : next;
+                    }
+                    next = sh.tm.tB[ra] < next ? sh.tm.tB[ra] : next;
+                    cache_store(l, M);
+                    ccnt[l] = (unsigned char)list_count(M);
+                    cB[l] = next;
+                }
+            }
         }
         __syncthreads();
-        lap(xs6);
-        // ---- rows whose cache emptied (one-CTA job: also survivors and rows
-        // running low, a warp each)
-        if (G == 1) {
+        lap(ty.xs[6]);
+        // ---- rows whose cache emptied
+        {
             const int nresc = sh.nresc;
-            for (int q = warp; q < nresc; q += W) {
-                const int l = rlist[q];
-                u64 top[K];
-                warp_row_refresh(p, row_of(l), bitmap, top, st_resc_cells);
-                if (lane == 0) {
-                    cache_store(l, top);
-                    const int c = list_count(top);
-                    ccnt[l] = c;
-                    cB[l] = c == K ? top[K - 1] : kNoKey;
+            if (ONE) {
+                for (int q = warp; q < nresc; q += W) {
+                    const int l = rlist[q];
+                    u64 top[K], next;
+                    warp_row_refresh(p, row_of(l), bitmap, top, next, st_resc_cells);
+                    if (lane == 0) {
+                        cache_store(l, top);
+                        ccnt[l] = (unsigned char)list_count(top);
+                        cB[l] = next;
+                    }
+                }
+            } else {
+                for (int q = 0; q < nresc; ++q) {
+                    const int l = rlist[q];
+                    if (full)
+                        block_row_topk_cols(p, row_of(l), 0, 1, 0x7fffffff, bitmap, sh, st_resc_cells);
+                    else
+                        block_row_topk(p, row_of(l), 0, 1, bitmap, sh, st_resc_cells);
+                    if (tid == 0) {
+                        cache_store(l, sh.tko);
+                        ccnt[l] = (unsigned char)list_count(sh.tko);
+                        cB[l] = sh.tnext;
+                    }
                 }
             }
-            if (tid == 0)
-                ty.rescans += nresc;
             if (nresc > 0)
-                __syncthreads();
-        } else {
-            const int nresc = sh.nresc;
-            for (int q = 0; q < nresc; ++q) {
-                const int l = rlist[q];
-                if (p.full)
-                    block_row_topk_log(p, row_of(l), bitmap, vpos, newer, sh, t, L, st_resc_cells);
-                else
-                    block_row_topk(p, row_of(l), bitmap, sh, st_resc_cells);
-                if (tid == 0) {
-                    cache_store(l, sh.tko);
-                    const int c = list_count(sh.tko);
-                    ccnt[l] = c;
-                    cB[l] = c == K ? sh.tko[K - 1] : kNoKey;
-                }
+                __syncthreads();  // the rescanned caches before anyone reads them
+            if (tid == 0) {
+                ty.rescans += nresc;
+                sh.nresc = 0;
+                ++ty.rounds;
+                ty.idle += L == 0;
             }
-            if (tid == 0)
-                ty.rescans += nresc;
-            if (nresc > 0)
-                __syncthreads();  // the rescanned caches (written by thread 0) before anyone reads them
         }
-        if (tid < 2 * L) {
-            const long long m = (tid & 1) ? sh.pj[tid >> 1] : sh.pi[tid >> 1];
-            if (owner_of(m) == b)
-                mflag[slot_of(m)] = 0;
-        }
-        lap(xs7);
-        if (tid < L) {
-            sh.ppi[tid] = sh.pi[tid];
-            sh.ppj[tid] = sh.pj[tid];
-        }
-        if (tid == 0) {
-            sh.nprev = L;
-            sh.nresc = 0;
-            ++ty.rounds;
-            ty.idle += L == 0;
-        }
+        lap(ty.xs[7]);
         t += L;
         if (t >= n - 1)
             break;  // that was the last merge
-        publish(r + 1);
-        lap(ph5);
-        bool last_a = false;
-        grid_arrive(p, epoch, p.timing ? &last_a : nullptr);
-        const u64 twa = p.timing && tid == 0 ? global_ns() : 0;
-        if (!grid_wait(p, epoch, sh))
-            return;
-        if (p.timing && tid == 0 && last_a) {
-            ty.xlast += global_ns() - twa;
-            ++ty.nlast;
-            ty.nlast_a_scan += G - 1 - b < sh.nexec;
-        }
-        lap(ph0);
+        __syncthreads();
     }
 
     if (p.stats) {
         u64 *St = reinterpret_cast<u64 *>(p.stats);
-        atomicAdd(St + 2, (u64)st_updates);
         atomicAdd(St + 5, (u64)st_fill_cells);
         atomicAdd(St + 15, (u64)st_resc_cells);
-        if (tid == 32) {
+        if (tid == (ONE ? 32 : TA)) {
             atomicAdd(St + 6, (u64)ty.installs);
             if (b == 0)
                 St[4] = (u64)ty.fills;  // every CTA read the same request lists
@@ -2327,36 +3181,28 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             if (b == 0) {
                 St[0] = (u64)ty.rounds;
                 St[1] = (u64)ty.idle;
+                St[2] = (u64)((n - 1) * (n - 2) / 2);  // m_t - 2 cells per merge
                 St[7] = (u64)ty.walk;
                 St[3] = (u64)G;
             }
             if (p.timing) {
-                ph1 += xs0 + xs1 + xs2;
-                ph4 += xs3 + xs4 + xs5;
-                ph5 += xs6 + xs7;
+                ty.ph[1] += ty.xs[5] + ty.xs[0] + ty.xs[1] + ty.xs[2] + ty.xs[3];
+                ty.ph[5] += ty.xs[4] + ty.xs[6] + ty.xs[7];
                 for (int q = 0; q < 6; ++q)
                     atomicAdd(St + 8 + q, ty.ph[q]);
                 for (int q = 0; q < 8; ++q)
                     atomicAdd(St + 16 + q, ty.xs[q]);
-                atomicAdd(St + 26, ty.xwalk);
-                atomicAdd(St + 27, ty.xlast);
-                atomicAdd(St + 28, (u64)ty.nlast);
-                atomicAdd(St + 29, (u64)ty.nlast_b);
-                atomicAdd(St + 30, (u64)ty.nlast_b_scan);
-                atomicAdd(St + 31, (u64)ty.nlast_a_scan);
-                if (b == 0)
-                    St[32] = (u64)ty.nlast;
             }
         }
     }
 }
 
-template <int NT, int MINB, int PUB>
+template <int NT, int MINB, bool ONE>
 __global__ void __launch_bounds__(NT, MINB) merge_kernel(MergeParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ Shared<NT, round_of(PUB)> sh;
-    merge_job<NT, PUB>(p, blockIdx.x, smem_raw, sh);
+    __shared__ Shared<NT, ONE> sh;
+    merge_job<NT, ONE>(p, blockIdx.x, smem_raw, sh);
 }
 
 // Many independent jobs in one persistent launch: each CTA takes the next job
@@ -2367,7 +3213,7 @@ template <int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) batch_kernel(BatchParams bp)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ Shared<NT, kRoundOne> sh;
+    __shared__ Shared<NT, true> sh;
     __shared__ int job;
     const WorkspaceLayout L = workspace_layout(bp.n_max, 1);
     char *ws = bp.ws + (size_t)blockIdx.x * L.total;
@@ -2389,6 +3235,7 @@ __global__ void __launch_bounds__(NT, MINB) batch_kernel(BatchParams bp)
         p.pitch = J.n;
         p.linkage = J.linkage;
         p.G = 1;
+        p.chunk = bp.chunk;
         p.aligned16 = ((uintptr_t)J.D & 15u) == 0;
         p.merges = J.merges;
         p.heights = J.heights;
@@ -2405,7 +3252,7 @@ __global__ void __launch_bounds__(NT, MINB) batch_kernel(BatchParams bp)
             reinterpret_cast<int *>(ws + L.zero)[q] = 0;
         __syncthreads();
         if (J.n > 1)
-            merge_job<NT, kPubOne>(p, 0, smem_raw, sh);
+            merge_job<NT, true>(p, 0, smem_raw, sh);
         __syncthreads();
         if (threadIdx.x == 0) {
             bp.job_status[jb] = J.n > 1 ? LDCG(p.status) : 0;
@@ -2465,41 +3312,22 @@ cudaError_t launch_expand(const float *packed, float *full, long long n, long lo
     return cudaGetLastError();
 }
 
-size_t merge_smem_bytes(long long n, int G, int nt)
-{
-    const long long nb = (n + kRowBlock - 1) / kRowBlock;
-    const long long Rmax = ((nb + G - 1) / G) * kRowBlock;
-    const long long nwords = (n + 31) / 32;
-    // bitmap; published entries (keys, column words); per
-    // slot: K keys, bound, size, count, refill round and position, rescan
-    // list entry, stamp, chain flag; pass-1 values of one chunk of rows (one
-    // float per pair) and their flags
-    const long long pub = G == 1 ? kPubOne : kPub;
-    const long long S = round_of((int)pub);
-    const long long chunk = Rmax < nt ? Rmax : nt;
-    const long long logbits = G > 1 ? (2 * nwords * 4 + 15) & ~15LL : 0;
-    return (size_t)(((nwords * 4 + 15) & ~15LL) + logbits + (long long)G * pub * 12 +
-                    (S > 16 ? chunk * (S + 1) * 4 : 0) +
-                    ((Rmax * (8 * K + 8 + 4 * 6 + 1) + nt + 15) & ~15LL));
-}
-
 namespace {
 
 // The kernel instantiations: CTA size nt and the CTAs per SM its registers allow.
-// A one-CTA job publishes more entries per round (nothing else is read).
 const void *merge_fn(int nt, int G)
 {
     if (G == 1) {
         switch (nt) {
-        case 128: return (const void *)merge_kernel<128, 4, kPubOne>;
-        case 256: return (const void *)merge_kernel<256, 2, kPubOne>;
-        default: return (const void *)merge_kernel<512, 1, kPubOne>;
+        case 128: return (const void *)merge_kernel<128, 4, true>;
+        case 256: return (const void *)merge_kernel<256, 2, true>;
+        default: return (const void *)merge_kernel<512, 1, true>;
         }
     }
     switch (nt) {
-    case 128: return (const void *)merge_kernel<128, 4, kPub>;
-    case 256: return (const void *)merge_kernel<256, 2, kPub>;
-    default: return (const void *)merge_kernel<512, 1, kPub>;
+    case 128: return (const void *)merge_kernel<128, 4, false>;
+    case 256: return (const void *)merge_kernel<256, 2, false>;
+    default: return (const void *)merge_kernel<512, 1, false>;
     }
 }
 
@@ -2516,17 +3344,85 @@ size_t static_smem(int nt, int G)
 {
     if (G == 1) {
         switch (nt) {
-        case 128: return sizeof(Shared<128, kRoundOne>);
-        case 256: return sizeof(Shared<256, kRoundOne>);
-        default: return sizeof(Shared<512, kRoundOne>);
+        case 128: return sizeof(Shared<128, true>) + 16;
+        case 256: return sizeof(Shared<256, true>) + 16;
+        default: return sizeof(Shared<512, true>) + 16;
         }
     }
     switch (nt) {
-    case 128: return sizeof(Shared<128, kRound>);
-    case 256: return sizeof(Shared<256, kRound>);
-    default: return sizeof(Shared<512, kRound>);
+    case 128: return sizeof(Shared<128, false>);
+    case 256: return sizeof(Shared<256, false>);
+    default: return sizeof(Shared<512, false>);
     }
 }
+
+// Dynamic shared memory for n objects on G CTAs of nt threads with chunks of
+// `chunk` rows: two bitmaps; published entries (keys, column words); per slot
+// K keys, bound, size, rescan list entry and key count, on a grid also the
+// pending refill (round, position) and the stamp; the new cells of a chunk.
+size_t smem_for(long long n, int G, int chunk)
+{
+    const long long nb = (n + kRowBlock - 1) / kRowBlock;
+    const long long Rmax = ((nb + G - 1) / G) * kRowBlock;
+    const long long words = (((n + 31) / 32) * 4 + 15) & ~15LL;
+    const long long row = 8 * K + 8 + 8 + 1 + (G > 1 ? 12 : 0);
+    return (size_t)(2 * words + (G > 1 ? (long long)G * kPub * 12 : 0) + (long long)chunk * (kSurv + 1) * 4 +
+                    ((Rmax * row + 15) & ~15LL));
+}
+
+}  // namespace
+
+// CTAs for n objects when the caller names no number.  One up to 416 objects: a
+// block of 32 rows per CTA and grid barriers are slower there (complete, ms,
+// one CTA / grid: n = 300 0.69 / 0.82, n = 400 0.96 / 1.01, n = 512 1.24 / 1.07,
+// n = 1000 3.30 / 1.64, n = 2048 12.6 / 2.8).  Centroid linkage makes few merges
+// per round and none side by side, so the barriers weigh more: 16.7 / 21.5 at
+// n = 1000, 36.6 / 35.7 at 1600, 54.4 / 46.0 at 2048.  Above, one CTA per block
+// up to 64 of them, then one per two blocks (complete: n = 3500 64 CTAs 4.64,
+// 96 4.57; average: n = 5003 80 CTAs 6.42, 152 6.49; n = 8191 96 10.9, 128 10.3),
+// at most one per SM.  Single linkage (the merges of a round are worked out one
+// by one, and every CTA repeats them) runs better on fewer CTAs with the same
+// most blocks per CTA (n = 16384: 128 35.8, 152 36.4; the others 25.5 and 25.0).
+int default_grid(long long n, int linkage, int num_sms)
+{
+    const long long nb = (n + kRowBlock - 1) / kRowBlock;
+    if (n <= (linkage == LW_CENTROID ? 1536 : 416))
+        return 1;
+    long long G = nb <= 64 ? nb : nb / 2 > 64 ? nb / 2 : 64;
+    if (G > num_sms)
+        G = num_sms;
+    if (linkage == LW_SINGLE) {
+        const long long per = (nb + G - 1) / G, even = (nb + per - 1) / per;
+        if (10 * even <= 9 * G)
+            G = even;
+    }
+    return (int)G;
+}
+
+int merge_chunk_rows(long long n, int G, int nt)
+{
+    const long long nb = (n + kRowBlock - 1) / kRowBlock;
+    const long long Rmax = ((nb + G - 1) / G) * kRowBlock;
+    const int most = (int)(Rmax < nt ? Rmax : nt);
+    // half a CTA's threads per chunk if that lets as many CTAs share an SM as
+    // the registers allow, else whatever fits at all
+    const long long sm = 228 * 1024, cta = 227 * 1024, fixed = (long long)static_smem(nt, G);
+    const long long share = sm / (kThreads / nt) - 1024 - fixed;
+    for (int c = most; c >= 32 && 2 * c >= most; c = (c / 2) & ~31)
+        if ((long long)smem_for(n, G, c) <= share)
+            return c;
+    int c = most;
+    while (c > 32 && (long long)smem_for(n, G, c) > cta - fixed)
+        c = c / 2 >= 32 ? (c / 2) & ~31 : 32;
+    return c;
+}
+
+size_t merge_smem_bytes(long long n, int G, int nt)
+{
+    return smem_for(n, G, merge_chunk_rows(n, G, nt));
+}
+
+namespace {
 
 int fit_per_sm(const void *fn, int nt, int G, size_t smem)
 {
@@ -2566,6 +3462,7 @@ cudaError_t launch_batch(const BatchParams &bp, int grid, int nt, cudaStream_t s
     // (this launch may be recorded into a graph, where no attribute is set)
     const size_t smem = merge_smem_bytes(bp.n_max, 1, nt);
     BatchParams q = bp;
+    q.chunk = merge_chunk_rows(bp.n_max, 1, nt);
     void *args[] = {&q};
     return cudaLaunchKernel(batch_fn(nt), dim3(grid), dim3(nt), args, smem, stream);
 }
@@ -2578,6 +3475,7 @@ cudaError_t launch_merge(const MergeParams &p, int nt, cudaStream_t stream)
     if (e != cudaSuccess)
         return e;
     MergeParams q = p;
+    q.chunk = merge_chunk_rows(p.n, p.G, nt);
     void *args[] = {&q};
     return cudaLaunchCooperativeKernel(fn, dim3(p.G), dim3(nt), args, smem, stream);
 }

@@ -7,8 +7,8 @@
 // and real-time loops that must not call the allocator at all.  This entry
 // point serves them: the caller passes its own device buffers for the
 // matrix and the outputs, and the kernel's global scratch (cluster sizes,
-// per-CTA exchange records and pair minima, refill lists, barrier, status
-// and counter words) lives in one file-scope __device__ array of fixed size.
+// per-CTA exchange records, refill and survivors' lists, barrier, status and
+// counter words) lives in one file-scope __device__ array of fixed size.
 // The array comes into being on a device when the library's device code is
 // loaded there -- with CUDA's lazy module loading, during the first call on
 // that device -- and stays until the process exits.  The row caches live in
@@ -26,9 +26,9 @@
 namespace {
 
 // Largest n this entry point accepts and the scratch that serves it
-// (workspace_layout): cluster sizes 4n B; per CTA a 240 B record and 512 B of
-// pair minima; 16 KB of refill lists; barrier, status and counter words.  At
-// n = 16384 on a 256-CTA grid that is about 275 KB; the array holds 2 MB,
+// (workspace_layout): cluster sizes 4n B; per CTA two records of 144 B; 64 KB of
+// refill lists; 34 KB of survivors' lists; barrier, status and counter words.
+// At n = 16384 on a 256-CTA grid that is about 305 KB; the array holds 2 MB,
 // and every call checks its layout against that size.
 constexpr long long kNoAllocMaxN = LW_NOALLOC_MAX_N;
 constexpr size_t kScratchBytes = 2 * 1024 * 1024;
@@ -72,11 +72,7 @@ extern "C" lw_status lw_cluster_noalloc(float *dist, int64_t n, int linkage, int
         cudaGetLastError();
         return LW_ERR_CUDA;
     }
-    // the same grid policy as lw_cluster: one CTA for small matrices, every SM otherwise
-    int G = n <= 4096 ? 1 : num_sms;
-    const long long nb = (n + lw::kRowBlock - 1) / lw::kRowBlock;
-    if (G > nb)
-        G = (int)nb;
+    int G = lw::default_grid(n, linkage, num_sms);  // lw_cluster's
     while (G < num_sms && !lw::merge_config_ok(n, G, num_sms))
         ++G;
     if (!lw::merge_config_ok(n, G, num_sms))
