@@ -8,6 +8,7 @@
 #include "../../include/lw.h"
 #include "lw_internal.h"
 
+#include <algorithm>
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
@@ -750,6 +751,8 @@ lw_status lw_batch_create(lw_ctx *ctx, const lw_job *jobs, int32_t njobs, lw_bat
     };
     int nstat = (int)b->big_idx.size();
     for (auto &c : b->classes) {
+        // largest first: the last job to start is a short one
+        std::stable_sort(c.idx.begin(), c.idx.end(), [&](int x, int y) { return jobs[x].n > jobs[y].n; });
         c.status_off = nstat;
         nstat += (int)c.idx.size();
     }
