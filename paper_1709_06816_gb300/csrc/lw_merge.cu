@@ -395,6 +395,7 @@ struct Shared {
     int nptouch;                 // slots the previous round touched
     int ptouch[kTeam];
     unsigned okm[NT / 32];       // rows of the chunk that take the round's merges
+    unsigned hit[NT];            // per row of the chunk: new cells that may enter its cache
     int nresc;                   // rows to rescan at once this round
     int item, viol;              // apply pass: next item, first merge that must wait
     unsigned limit, width;       // see the selection
@@ -1657,6 +1658,8 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
         const float nk = (float)rsize[l];
         const long long bk = row_base(p, k);
         const int sk = full ? rstamp[l] : 0;
+        const unsigned bhi = (unsigned)(sh.cx.cB[l] >> 32);
+        unsigned hm = 0u;
         // cell (k, member): packed, row x for k > x (consecutive k of a
         // warp read consecutive words) and row k for k < x; row-log
         // layout, row x of M when x was stamped no earlier than k, else
@@ -1693,6 +1696,8 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
             if (ok) {
                 const long long x = sh.tm.sslot[s];
                 kvs[(size_t)(blk * 32 + lane) * KVP + s] = v;
+                if (x > k && __float_as_uint(v) <= bhi)
+                    hm |= 1u << s;
                 if (tie) {
                     // does it come before a later merge of the round?  (s = q)
                     const unsigned vb = __float_as_uint(v);
@@ -1717,6 +1722,8 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
                 }
             }
         }
+        if (hm != 0u)
+            atomicOr(&sh.hit[blk * 32 + lane], hm);
     }
 }
 
@@ -2010,6 +2017,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
     long long st_fill_cells = 0, st_resc_cells = 0;
 
     // ---- setup
+    sh.hit[tid] = 0u;
     for (long long w = tid; w < nwords; w += NT) {
         const long long live_n = n - w * 32;
         bitmap[w] = live_n >= 32 ? 0xffffffffu : ((1u << live_n) - 1u);
@@ -2161,22 +2169,22 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             // ---- the caches of the previous round's survivors: every cell of a
             // survivor's row below that round's limit is in its list (those over
             // the list's size: above svovf) or among the cells to other survivors
-            for (int s = warp; s < sh.nps; s += W) {
-                u64 x = kNoKey, B = kNoKey;
+            const int nsv = sh.nps;
+            for (int s = warp; s < nsv; s += W) {
                 const size_t at = (size_t)(par ^ 1) * kSurv + s;
                 const int cnt = LDCG(p.svcnt + at);
-                u64 x2;
-                {
-                    const ulonglong2 y = LDCG(reinterpret_cast<const ulonglong2 *>(p.svlist + at * kSvList) + lane);
-                    x = 2 * lane < cnt ? y.x : kNoKey;
-                    x2 = 2 * lane + 1 < cnt ? y.y : kNoKey;
-                }
-                u64 x3 = lane < K ? sh.tm.tT[s][lane] : kNoKey;
-                if (lane == K)
-                    B = sh.tm.tB[s];
-                else if (lane == K + 1)
-                    B = LDCG(p.svovf + at);
-                else if (lane == K + 2)
+                const u64 ovf = LDCG(p.svovf + at);
+                const ulonglong2 y2 = LDCG(reinterpret_cast<const ulonglong2 *>(p.svlist + at * kSvList) + lane);
+                u64 B = kNoKey;
+                u64 x = 2 * lane < cnt ? y2.x : kNoKey;
+                u64 x2 = 2 * lane + 1 < cnt ? y2.y : kNoKey;
+                // (C still holds the previous round's)
+                u64 x3 = kNoKey;
+                if (lane < nsv && sh.pslot[lane] > sh.pslot[s])
+                    x3 = make_key(sh.tm.C[s][lane], (unsigned)sh.pslot[lane]);
+                if (lane == 0)
+                    B = ovf;
+                else if (lane == 1)
                     B = sh.limit == 0xffffffffu ? kNoKey : (u64)sh.limit << 32;
                 B = warp_u64_min(B);
                 u64 top[K];
@@ -2942,9 +2950,9 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             }
             if (l0 == 0) {
                 bookkeeping();
-                // the survivors' smallest cells to other survivors (those to the other
-                // members are among their owners' new cells), a lane each
-                for (int s = warp; s < ns; s += W) {
+                // one CTA: the survivors' smallest cells to other survivors (those to the
+                // other members are among their owners' new cells), a lane each
+                for (int s = warp; ONE && s < ns; s += W) {
                     u64 x = kNoKey;
                     if (lane < ns && sh.tm.sslot[lane] > sh.tm.sslot[s])
                         x = make_key(sh.tm.C[s][lane], (unsigned)sh.tm.sslot[lane]);
@@ -3015,6 +3023,8 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             for (int q = tid; q < rows; q += NT) {
                 const int l = l0 + q;
                 const long long k = row_of(l);
+                unsigned hm = sh.hit[q];
+                sh.hit[q] = 0u;
                 if (!(k < n && live(bitmap, k) && !live(touched, k)))
                     continue;
                 int c = ccnt[l];
@@ -3036,14 +3046,13 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         c = list_count(Cc);
                     }
                     const float *kr = kvs + (size_t)q * KVP;
-#pragma unroll 4
-                    for (int s = 0; s < ns; ++s) {
+                    // (those of merges put off again go)
+                    for (hm &= ns < 32 ? (1u << ns) - 1u : kFull; hm != 0u; hm &= hm - 1u) {
+                        const int s = __ffs(hm) - 1;
                         const unsigned vb = __float_as_uint(kr[s]);
-                        if (vb > (unsigned)(B >> 32))
-                            continue;
                         const long long x = sh.tm.sslot[s];
                         const u64 key = ((u64)vb << 32) | (unsigned)x;
-                        if (x > k && key < B) {
+                        if (key < B) {
                             const u64 out = list_insert(Cc, key);
                             dirty = true;
                             if (c == K)
