@@ -49,7 +49,7 @@
 //      computed and kept back, every CTA looks whether one of its own comes
 //      before a merge of the round, and barrier 3 tells which merges stand.
 //   apply  behind barrier 2 (no CTA still reads the members' old cells): the new
-//      cells D(k, survivor) for every live k, a warp per 32 rows and up to 8
+//      cells D(k, survivor) for every live k, a warp per 32 rows and up to 4
 //      survivors, all loads of an item in flight at once; then logs, caches
 //      (merged columns leave, new cells at or below B enter) and the
 //      survivors' lists: their new cells below a limit go to lists in global
@@ -65,15 +65,20 @@
 // bound sits at the front of the merges is rescanned at once by its owner.  A
 // job's only CTA refreshes emptied rows itself, a warp per row.
 //
-// What bounds it.  A round is a chain of latencies: about 40 us at n = 16384 of
-// which 3 are barrier 1, 6 the selection, 7 the gather and the chain's operands,
-// 5 the merges, 7 the new cells, 6 caches and lists; the memory traffic of a
-// round (some 10 MB) would take under 2 us.  So what counts is merges per
-// round.  Certifying a walk of disjoint entries after the new cells' minima
-// were exchanged (two full barriers and about 13 merges per round) took 46.1 ms for
-// n = 16384 average linkage, 162.8 ms for single and 16.8 ms for n = 1968
-// (complete, one CTA then); selecting up to 64 members by a threshold and
-// merging inside them takes 28.8, 62.4 and 2.7 ms.
+// What bounds it.  A round is a chain of short steps: about 40 us at n = 16384
+// of which 3 are barrier 1, 6 the selection, 6 the gather, 5 the merges, 7 the
+// new cells, 4 caches and lists, 3 publish; the memory traffic of a round (some
+// 10 MB) would take under 2 us.  So what counts is merges per round: certifying
+// a walk of disjoint entries after an exchange of the new cells' minima (two full
+// barriers and about 13 merges per round) took 46.1 ms for n = 16384 average
+// linkage, 162.8 ms for single and 16.8 ms for n = 1968 (complete, on one CTA
+// then); selecting up to 64 members by a threshold and merging inside them takes
+// 25.6, 51 and 2.4 ms.  Next, the instructions themselves: each step's code
+// runs once or twice per round, so most of it is fetched anew every round
+// (n = 2000: 58 % of the SM's instruction cache requests hit, and waiting for
+// instructions was the largest stall after barriers, 3.7 of 11 cycles per
+// instruction outside them).  That is why no loop below is unrolled unless its
+// loads have to be in flight together: it took 5 to 9 % off every grid run.
 //
 // Exact arithmetic: every product and sum of the update uses __fmul_rn /
 // __fadd_rn / __fsub_rn (never contracted into FMA), the coefficient
@@ -443,6 +448,7 @@ __device__ void exchange_requests(int cnt, const int (&rq)[kReqPerCta], int b, S
         sh.wcnt[warp] = inc;
     __syncthreads();
     int base = 0;
+#pragma unroll 1
     for (int w = 0; w < warp; ++w)
         base += sh.wcnt[w];
     const int off0 = base + inc - cnt;
@@ -453,6 +459,7 @@ __device__ void exchange_requests(int cnt, const int (&rq)[kReqPerCta], int b, S
     }
     if ((int)threadIdx.x == b) {
         // this CTA's own requests (list pq) get their positions
+#pragma unroll 1
         for (int q = 0; q < cnt; ++q) {
             const int l = sh.myreq_l[pq][q];
             if (off0 + q < kMaxReq)
@@ -654,6 +661,61 @@ __device__ void warp_row_topk(const MergeParams &p, long long r, u64 (&out)[K], 
     warp_topk_next(L, out, next);
 }
 
+// Eight 16-byte pieces of a packed row (j0, j0 + stride, .. below j1; column of
+// word q: q + base_c), live cells into a sorted list: all loads in flight, one
+// comparison per cell, and one copy of the insertion for the few that pass (a
+// copy per cell made this scan 47 KB of instructions, and fetching them cost
+// more than running them).
+__device__ __forceinline__ void take_batch(const MergeParams &p, long long j0, int stride, long long j1,
+                                           long long base_c, const unsigned *bitmap, u64 (&L)[K], long long &cnt)
+{
+    const float4 *D4 = reinterpret_cast<const float4 *>(p.D);
+    float v[8][4];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const long long j = j0 + (long long)u * stride;
+        const float4 x = j < j1 ? LDCG(D4 + j) : make_float4(-1.0f, -1.0f, -1.0f, -1.0f);
+        v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
+    }
+    const int c0 = (int)((j0 << 2) + base_c);
+    unsigned in = 0u;
+    int had = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        if (v[u][0] >= 0.0f) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int c = c0 + 4 * u * stride + e;
+                const unsigned on = (bitmap[c >> 5] >> (c & 31)) & 1u;
+                had += (int)on;
+                // the whole key: ties on the value stop here
+                if (make_key(v[u][e], (unsigned)c) < L[K - 1])
+                    in |= on << (4 * u + e);
+            }
+        }
+    }
+    cnt += had;
+#pragma unroll 1
+    for (; in != 0u; in &= in - 1u) {
+        const int i = __ffs(in) - 1;
+        float x = v[0][0];
+#pragma unroll
+        for (int q = 1; q < 32; ++q)
+            x = i == q ? v[q >> 2][q & 3] : x;
+        const u64 key = make_key(x, (unsigned)(c0 + 4 * (i >> 2) * stride + (i & 3)));
+        if (key < L[K - 1])
+            list_insert(L, key);
+    }
+}
+
+// block_topk of K-lists, out of line: it is called at the end of every scan.
+template <int NT, bool ONE, int TB>
+__device__ __noinline__ void block_topk_call(u64 a, u64 b, u64 c, u64 d, Shared<NT, ONE> &sh)
+{
+    u64 L[K] = {a, b, c, d};
+    block_topk<NT, ONE, K, TB>(L, sh);
+}
+
 // K smallest keys of row r over live columns, computed by the whole CTA (a
 // refill, or a row whose cache emptied).  Adds the live cells read to
 // `live_cells`.  Result in sh.tko.
@@ -689,36 +751,20 @@ __device__ __noinline__ void block_row_topk(const MergeParams &p, long long r, i
     if (a0 > end)
         a0 = end;
     const long long a1 = a0 + ((end - a0) & ~3LL);
-    if (piece == 0)
-        for (long long q = start + ts; q < a0; q += TB)
+    // (head, then tail)
+#pragma unroll 1
+    for (int part = piece == 0 ? 0 : 1; part < (piece == np - 1 ? 2 : 1); ++part)
+#pragma unroll 1
+        for (long long q = (part ? a1 : start) + ts; q < (part ? end : a0); q += TB)
             take(LDCG(p.D + q), q);
-    if (piece == np - 1)
-        for (long long q = a1 + ts; q < end; q += TB)
-            take(LDCG(p.D + q), q);
-    const float4 *D4 = reinterpret_cast<const float4 *>(p.D);
     const long long part = ((a1 - a0) >> 2) / np;
     const long long jb = (a0 >> 2) + part * piece;
     const long long j1 = piece == np - 1 ? a1 >> 2 : jb + part;
-    for (long long j0 = jb + ts; j0 < j1; j0 += 8 * TB) {
-        float4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const long long j = j0 + (long long)u * TB;
-            v[u] = j < j1 ? LDCG(D4 + j) : make_float4(-1.0f, -1.0f, -1.0f, -1.0f);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (v[u].x >= 0.0f) {
-                const long long q = (j0 + (long long)u * TB) << 2;
-                take(v[u].x, q);
-                take(v[u].y, q + 1);
-                take(v[u].z, q + 2);
-                take(v[u].w, q + 3);
-            }
-        }
-    }
+#pragma unroll 1
+    for (long long j0 = jb + ts; j0 < j1; j0 += 8 * TB)
+        take_batch(p, j0, TB, j1, base_c, bitmap, L, cnt);
     live_cells += cnt;
-    block_topk<NT, ONE, K, TB>(L, sh);
+    block_topk_call<NT, ONE, TB>(L[0], L[1], L[2], L[3], sh);
 }
 // block_row_topk in the row-log layout, column by column: live column c > r
 // holds its current cell in row r of M when c's stamp is not after r's, and
@@ -769,11 +815,11 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
     if (c_a > n)
         c_a = n;
     const long long c_b = c_a + ((n - c_a) & ~3LL);
-    if (piece == 0)
-        for (long long c = r + 1 + ts; c < c_a; c += TB)
-            one(c);
-    if (piece == np - 1)
-        for (long long c = c_b + ts; c < n; c += TB)
+    // (head, then tail)
+#pragma unroll 1
+    for (int end = piece == 0 ? 0 : 1; end < (piece == np - 1 ? 2 : 1); ++end)
+#pragma unroll 1
+        for (long long c = (end ? c_b : r + 1) + ts; c < (end ? n : c_a); c += TB)
             one(c);
     {
         constexpr int U = 2;
@@ -844,11 +890,12 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
                             mn = k;
                     }
                 }
-                u64 M4[K] = {mn, kNoKey, kNoKey, kNoKey};
-                block_topk<NT, ONE, K, TB>(M4, sh);
+                block_topk_call<NT, ONE, TB>(mn, kNoKey, kNoKey, kNoKey, sh);
                 thr = sh.tnext;
                 first = false;
             }
+            // one copy of the insertion for the few cells that pass (see take_batch)
+            unsigned in = 0u;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const long long c = (j0 + (long long)u * TB) << 2;
@@ -856,14 +903,25 @@ __device__ __noinline__ void block_row_topk_cols(const MergeParams &p, long long
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const u64 k = make_key(v[u][e], (unsigned)(c + e));
-                    if (((m4[u] >> e) & 1u) && k <= thr && k < L[K - 1])
-                        list_insert(L, k);
+                    if (k <= thr && k < L[K - 1])
+                        in |= m4[u] & (1u << e) ? 1u << (4 * u + e) : 0u;
                 }
+            }
+#pragma unroll 1
+            for (; in != 0u; in &= in - 1u) {
+                const int i = __ffs(in) - 1;
+                float x = v[0][0];
+#pragma unroll
+                for (int q = 1; q < 4 * U; ++q)
+                    x = i == q ? v[q >> 2][q & 3] : x;
+                const u64 k = make_key(x, (unsigned)(((j0 + (long long)(i >> 2) * TB) << 2) + (i & 3)));
+                if (k < L[K - 1])
+                    list_insert(L, k);
             }
         }
     }
     live_cells += cnt;
-    block_topk<NT, ONE, K, TB>(L, sh);
+    block_topk_call<NT, ONE, TB>(L[0], L[1], L[2], L[3], sh);
     if (tlog && ts == 0)
         tlog[1] += global_ns() - tm0;
 }
@@ -896,30 +954,15 @@ __device__ __noinline__ void warp_row_refresh(const MergeParams &p, long long r,
     if (a0 > end)
         a0 = end;
     const long long a1 = a0 + ((end - a0) & ~3LL);
-    for (long long q = start + lane; q < a0; q += 32)
-        take(LDCG(p.D + q), q);
-    for (long long q = a1 + lane; q < end; q += 32)
-        take(LDCG(p.D + q), q);
-    const float4 *D4 = reinterpret_cast<const float4 *>(p.D);
+#pragma unroll 1
+    for (int part = 0; part < 2; ++part)  // head, tail
+#pragma unroll 1
+        for (long long q = (part ? a1 : start) + lane; q < (part ? end : a0); q += 32)
+            take(LDCG(p.D + q), q);
     const long long j1 = a1 >> 2;
-    for (long long j0 = (a0 >> 2) + lane; j0 < j1; j0 += 8 * 32) {
-        float4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const long long j = j0 + 32 * u;
-            v[u] = j < j1 ? LDCG(D4 + j) : make_float4(-1.0f, -1.0f, -1.0f, -1.0f);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (v[u].x >= 0.0f) {
-                const long long q = (j0 + 32 * u) << 2;
-                take(v[u].x, q);
-                take(v[u].y, q + 1);
-                take(v[u].z, q + 2);
-                take(v[u].w, q + 3);
-            }
-        }
-    }
+#pragma unroll 1
+    for (long long j0 = (a0 >> 2) + lane; j0 < j1; j0 += 8 * 32)
+        take_batch(p, j0, 32, j1, base_c, bitmap, L, cnt);
     live_cells += cnt;
     warp_topk_next(L, out, next);
 }
@@ -1104,6 +1147,7 @@ __device__ __noinline__ void simulate_steps(Team &tm, int &L_out, bool &dep_out)
             for (int h = 0; h < 2; ++h) {
                 const int k = lane + 32 * h;
                 if (lost[h] && lv[h]) {
+#pragma unroll 1
                     for (u64 q = mk[h]; q; q &= q - 1) {
                         const int c = __ffsll((long long)q) - 1;
                         const unsigned x = __float_as_uint(row[h][c]), y = (unsigned)(k << 8 | c);
@@ -1236,6 +1280,7 @@ __device__ __noinline__ void simulate(Team &tm, int linkage)
             sidx[h] = rt[h] >= 0 ? __popcll(ends & ((1ull << rt[h]) - 1ull)) : -1;
         // merges of survivor s: masks of both halves
         unsigned w0 = 0u, w1 = 0u, g0 = 0u, g1 = 0u, g10 = 0u;
+#pragma unroll 1
         for (int s = 0; s < ns; ++s) {
             const unsigned x0 = __ballot_sync(kFull, sidx[0] == s), x1 = __ballot_sync(kFull, sidx[1] == s);
             if (lane == s) {
@@ -1285,6 +1330,7 @@ __device__ __noinline__ void simulate(Team &tm, int linkage)
     // the survivors' cells to one another
     if (lane < ns) {
         const int a = tm.mi(tm.sq[lane]);
+#pragma unroll 1
         for (int s = 0; s < ns; ++s)
             tm.C[s][lane] = tm.S[tm.mi(tm.sq[s])][a];
     }
@@ -1351,6 +1397,7 @@ __device__ __forceinline__ void chain_cells_made(Team &tm, int q0, int nw)
 {
     const int lane = threadIdx.x & 31;
     const int L = tm.L;
+#pragma unroll 1
     for (int q = q0; q < L; q += nw) {
         const int4 rec = tm.rec[q];
         const int i = rec.x & 0xff, j = (rec.x >> 8) & 0xff;
@@ -1380,6 +1427,7 @@ __device__ __forceinline__ void chain_limits(Team &tm, int q0, int nw)
     const int lane = threadIdx.x & 31;
     const int L = tm.L, m = tm.m;
     const unsigned thv = tm.thv;
+#pragma unroll 1
     for (int q = q0; q < L; q += nw) {
         const int4 rq = tm.rec[q];
         unsigned xy = 0xffffffffu, cc = 0xffffffffu, un = 0xffffffffu;
@@ -1545,6 +1593,7 @@ __device__ __noinline__ float chain_cells(const MergeParams &p, const Team &tm, 
         return LDCG(p.D + (k > x ? tm.mbase[a] + k : bk + x));
     };
     int prev = tm.prog[f];
+#pragma unroll 1
     for (int e = 1; e < len; ++e) {
         const int q = tm.prog[f + e];
         const int x = tm.rec[q].x;
@@ -1631,7 +1680,7 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
     const int *rsize = sh.cx.rsize, *rstamp = sh.cx.rstamp;
     const int nblk = rows / 32;
     const unsigned last = L > 0 ? (unsigned)sh.tm.rec[L - 1].y : 0u;
-    constexpr int U = 8;
+    constexpr int U = 4;  // (8: 6 % slower at n = 1968 and 16384, twice the instructions)
     // (fewer survivors at a time when that leaves no warp without an item)
     int ug = U;
     while (ug > 2 && nblk * ((ns + ug / 2 - 1) / (ug / 2)) <= NT / 32)
@@ -1704,6 +1753,7 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
                     if (vb <= last) {
                         const u64 kA = ((u64)vb << 32) | (unsigned)(k < x ? k : x);
                         const unsigned kC = (unsigned)(k < x ? x : k);
+#pragma unroll 1
                         for (int e = s + 1; e < L; ++e) {
                             const int4 rec = sh.tm.rec[e];
                             const u64 eA = ((u64)(unsigned)rec.y << 32) | (unsigned)sh.tm.mem[rec.x & 0xff];
@@ -1749,6 +1799,7 @@ __device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &s
     // a pivot that takes in at least kPub rows' first entries, then the
     // entries up to it in order by counting
     u64 head = kNoKey;
+#pragma unroll 1
     for (int l = tid; l < R; l += NT) {
         const int c = ccnt[l];
         const u64 B = cB[l];
@@ -1773,8 +1824,10 @@ __device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &s
 #pragma unroll
         for (int q = 0; q < kPub; ++q)
             Lst[q] = kNoKey;
+#pragma unroll 1
         for (int l = tid; l < R; l += NT) {
             const int c = ccnt[l];
+#pragma unroll 1
             for (int q = 0; q <= c; ++q) {
                 u64 e;
                 entry_at(l, q, c, e);
@@ -1810,8 +1863,10 @@ __device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &s
     const u64 pivot = find_pivot(count, gmin, kNoKey, sh.ppivot, kPub, 3 * kPub);
     int have = 0;
     if (head <= pivot && head != kNoKey) {
+#pragma unroll 1
         for (int l = tid; l < R; l += NT) {
             const int c = ccnt[l];
+#pragma unroll 1
             for (int q = 0; q <= c; ++q) {
                 u64 e;
                 entry_at(l, q, c, e);
@@ -1834,8 +1889,10 @@ __device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &s
         at = base + at - have;
     }
     if (have > 0) {
+#pragma unroll 1
         for (int l = tid; l < R; l += NT) {
             const int c = ccnt[l];
+#pragma unroll 1
             for (int q = 0; q <= c; ++q) {
                 u64 e;
                 const u64 x = entry_at(l, q, c, e);
@@ -1855,10 +1912,12 @@ __device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &s
     // (at most 3 * kPub threads of 4 rows and K + 1 entries each: they fit)
     static_assert(3 * kPub * 4 * (K + 1) <= kCand, "published entries fit");
     const int N = sh.ncand < kCand ? sh.ncand : kCand;
+#pragma unroll 1
     for (int c0 = (tid >> 5) * 8; c0 < N; c0 += NT / 4) {
         const int c = c0 + (lane >> 2);
         const u64 key = c < N ? sh.ckey[c] : kNoKey;
         int rank = 0;
+#pragma unroll 1
         for (int f = lane & 3; f < N; f += 4)
             rank += sh.ckey[f] < key;
         rank += __shfl_xor_sync(kFull, rank, 1);
@@ -1994,8 +2053,10 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
     // per-phase wall-clock totals of this CTA (thread 0), when timing is on
     auto &ty = sh.ty;
     if (tid == 0) {
+#pragma unroll 1
         for (int q = 0; q < 6; ++q)
             ty.ph[q] = 0;
+#pragma unroll 1
         for (int q = 0; q < 8; ++q)
             ty.xs[q] = 0;
         ty.xscan[0] = ty.xscan[1] = ty.tmark = 0;
@@ -2018,11 +2079,13 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
 
     // ---- setup
     sh.hit[tid] = 0u;
+#pragma unroll 1
     for (long long w = tid; w < nwords; w += NT) {
         const long long live_n = n - w * 32;
         bitmap[w] = live_n >= 32 ? 0xffffffffu : ((1u << live_n) - 1u);
         touched[w] = 0u;
     }
+#pragma unroll 1
     for (int l = tid; l < R; l += NT) {
         rsize[l] = 1;
         if (!ONE) {
@@ -2030,6 +2093,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             rstamp[l] = -1;
         }
     }
+#pragma unroll 1
     for (long long r = (long long)b * NT + tid; r < n; r += (long long)G * NT) {
         STCG(p.size_g + r, 1);
         if (full)
@@ -2061,6 +2125,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
     {
         int bad = 0;
         unsigned mx = 0u;
+#pragma unroll 1
         for (int l = warp; l < R; l += W) {
             const long long r = row_of(l);
             u64 top[K], next = kNoKey;
@@ -2088,6 +2153,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
 
     long long t = 0;   // merges done
     const long long max_rounds = 2 * n + 64;
+#pragma unroll 1
     for (int r = 0;; ++r) {
         const int par = r & 1;
         if (r > max_rounds) {
@@ -2146,6 +2212,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             }
             // keys and column words, entry q of CTA g at [q * G + g]
             constexpr int KW = kPub / 2, CW = kPub / 4;  // 16-byte words of both
+#pragma unroll 1
             for (int w = tid; w < (KW + CW) * G; w += NT) {
                 const int g = w / (KW + CW), part = w % (KW + CW);
                 const uint4 v = LDCG(reinterpret_cast<const uint4 *>(recs + g) + part);
@@ -2170,6 +2237,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             // survivor's row below that round's limit is in its list (those over
             // the list's size: above svovf) or among the cells to other survivors
             const int nsv = sh.nps;
+#pragma unroll 1
             for (int s = warp; s < nsv; s += W) {
                 const size_t at = (size_t)(par ^ 1) * kSurv + s;
                 const int cnt = LDCG(p.svcnt + at);
@@ -2187,9 +2255,8 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 else if (lane == 1)
                     B = sh.limit == 0xffffffffu ? kNoKey : (u64)sh.limit << 32;
                 B = warp_u64_min(B);
-                u64 top[K];
                 int c = 0;
-#pragma unroll
+#pragma unroll 1
                 for (int q = 0; q <= K; ++q) {
                     u64 y = x < x2 ? x : x2;
                     y = x3 < y ? x3 : y;
@@ -2198,7 +2265,8 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     x2 = x2 == y ? kNoKey : x2;
                     x3 = x3 == y ? kNoKey : x3;
                     if (q < K) {
-                        top[q < K ? q : 0] = y < B ? y : kNoKey;
+                        if (lane == 0)
+                            sh.svk[s][q] = y < B ? y : kNoKey;
                         c += y < B;
                     } else {
                         B = y < B ? y : B;
@@ -2206,15 +2274,12 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 }
                 if (lane == 0) {
                     atomicAdd(&sh.svsum, cnt < 8 ? cnt : 8);
-#pragma unroll
-                    for (int q = 0; q < K; ++q)
-                        sh.svk[s][q] = top[q];
                     sh.svB[s] = B;
                     sh.svc[s] = c;
                     const long long row = sh.pslot[s];
                     if (owner_of(row) == b) {
                         const int l = slot_of(row);
-                        cache_store(l, top);
+                        cache_store(l, sh.svk[s]);
                         ccnt[l] = (unsigned char)c;
                         cB[l] = B;
                         if (c <= kSurvivorRefillAt && B != kNoKey)
@@ -2229,6 +2294,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             const int ipar = par ^ 1;
             const int inp = sh.npieces;  // pieces per row of the previous round
             const int nps = sh.nps;
+#pragma unroll 1
             for (int s2 = W - 1 - warp; s2 < ninst; s2 += W) {
                 const int l = sh.inst_slot[s2];
                 const int pos = pend_s[l];
@@ -2269,6 +2335,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         M[q] = kNoKey;
                 sort_list(M);
                 int c = list_count(M);
+#pragma unroll 1
                 for (unsigned w = __ballot_sync(kFull, xr < B); w; w &= w - 1) {
                     const u64 x = __shfl_sync(kFull, xr, __ffs(w) - 1);
                     if (x < B) {
@@ -2291,6 +2358,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             __syncthreads();
         }
         // (the previous round's bits; the selection's barriers follow)
+#pragma unroll 1
         for (int q = tid; q < sh.nptouch; q += NT)
             atomicAnd(&touched[sh.ptouch[q] >> 5], ~(1u << (sh.ptouch[q] & 31)));
         lap(ty.xs[0]);
@@ -2330,6 +2398,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             {
                 u64 head = kNoKey, hard = kNoKey;
                 if (ONE) {
+#pragma unroll 1
                     for (int l = tid; l < R; l += TS) {
                         const int c = ccnt[l];
                         const u64 B = cB[l];
@@ -2339,6 +2408,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         }
                     }
                 } else {
+#pragma unroll 1
                     for (int g = tid; g < G; g += TS) {
                         const u64 x = wkey[g], y = wkey[(kPub - 1) * G + g];  // (a list that is full may go on)
                         head = x < head ? x : head;
@@ -2377,15 +2447,18 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     const bool svw = !ONE && 32 * (warp + 1) == TS;
                     if (head <= pivot && head != kNoKey) {
                         if (ONE) {
+#pragma unroll 1
                             for (int l = tid; l < R; l += TS) {
                                 const int cc = ccnt[l];
                                 const u64 B = cB[l];
                                 const u64 rowbits = (u64)l << kRankBits;
+#pragma unroll 1
                                 for (int q = 0; q < cc; ++q)
                                     have += entry_key(ck[(size_t)q * Rmax + l], rowbits, q) <= pivot;
                                 have += B != kNoKey && entry_key(B, rowbits, cc) <= pivot;
                             }
                         } else {
+#pragma unroll 1
                             for (int g = tid; g < G; g += TS) {
 #pragma unroll
                                 for (int q = 0; q < kPub; ++q) {
@@ -2399,6 +2472,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         const u64 rowbits = (u64)sh.pslot[lane] << kRankBits;
                         const int cc = sh.svc[lane];
                         const u64 B = sh.svB[lane];
+#pragma unroll 1
                         for (int q = 0; q < cc; ++q)
                             svn += entry_key(sh.svk[lane][q], rowbits, q) <= pivot;
                         svn += B != kNoKey && entry_key(B, rowbits, cc) <= pivot;
@@ -2426,10 +2500,12 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     };
                     if (have > 0) {
                         if (ONE) {
+#pragma unroll 1
                             for (int l = tid; l < R; l += TS) {
                                 const int cc = ccnt[l];
                                 const u64 B = cB[l];
                                 const u64 rowbits = (u64)l << kRankBits;
+#pragma unroll 1
                                 for (int q = 0; q < cc; ++q) {
                                     const u64 x = ck[(size_t)q * Rmax + l];
                                     const u64 e = entry_key(x, rowbits, q);
@@ -2441,7 +2517,9 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                                     put(entry_key(B, rowbits, cc), kRowStop | (unsigned)B);
                             }
                         } else {
+#pragma unroll 1
                             for (int g = tid; g < G; g += TS) {
+#pragma unroll 1
                                 for (int q = 0; q < kPub; ++q) {
                                     const u64 e = wkey[q * G + g];
                                     if (e > pivot || e == kNoKey)
@@ -2455,6 +2533,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         const u64 rowbits = (u64)sh.pslot[lane] << kRankBits;
                         const int cc = sh.svc[lane];
                         const u64 B = sh.svB[lane];
+#pragma unroll 1
                         for (int q = 0; q < cc; ++q) {
                             const u64 x = sh.svk[lane][q];
                             const u64 e = entry_key(x, rowbits, q);
@@ -2477,10 +2556,12 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 }
                 const int N = sh.ncand;
                 // key order by counting (entries are distinct), four threads per entry
+#pragma unroll 1
                 for (int c0 = (tid >> 5) * 8; c0 < N; c0 += TS / 4) {
                     const int c = c0 + (lane >> 2);
                     const u64 key = c < N ? sh.ckey[c] : kNoKey;
                     int rank = 0;
+#pragma unroll 1
                     for (int f = lane & 3; f < N; f += 4)
                         rank += sh.ckey[f] < key;
                     rank += __shfl_xor_sync(kFull, rank, 1);
@@ -2496,11 +2577,13 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 // which entries bring a row or column that no earlier one has
                 const int E = N < kEntries ? N : kEntries;
                 // (eight threads per entry)
+#pragma unroll 1
                 for (int c0 = (tid >> 5) * 4; c0 < E; c0 += TS / 8) {
                     const int e = c0 + (lane >> 3);
                     const uint2 w = e < E ? sh.erc[e] : make_uint2(0u, 0u);
                     const unsigned row = w.x, col = w.y & kColMask;
                     int in = 0;
+#pragma unroll 1
                     for (int f = lane & 7; f < e; f += 8) {
                         const uint2 o = sh.erc[f];
                         const unsigned fc = o.y & kColMask;
@@ -2599,6 +2682,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             {
                 // members in slot order, with their sizes, stamps and bounds: eight
                 // threads per member
+#pragma unroll 1
                 for (int a0 = (tid >> 5) * 4; a0 < m; a0 += TS / 8) {
                     const int a = a0 + (lane >> 3), part = lane & 7;
                     const int x = a < m ? sh.umem[a] : -1;
@@ -2611,10 +2695,12 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                             st = LDCG(p.stamp + x);
                     }
                     int rank = 0;
+#pragma unroll 1
                     for (int q = part; q < m; q += 8)
                         rank += sh.umem[q] < x;
                     u64 A = kNoKey;
                     unsigned C = 0u, ex = 0xffu;
+#pragma unroll 1
                     for (int e = part; e < ne; e += 8) {
                         const uint2 w = sh.erc[e];
                         if ((w.y & kRowStop) && w.x == (unsigned)x) {
@@ -2655,6 +2741,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             bad = count_s(bad != 0);
             {
                 // the entries by member (eight threads per entry)
+#pragma unroll 1
                 for (int c0 = (tid >> 5) * 4; c0 < ne; c0 += TS / 8) {
                     const int e = c0 + (lane >> 3);
                     const uint2 w = e < ne ? sh.erc[e] : make_uint2(0u, kRowStop);
@@ -2662,6 +2749,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     if (!(w.y & kRowStop)) {
                         const int row = (int)w.x, col = (int)(w.y & kColMask);
                         at = 0u;
+#pragma unroll 1
                         for (int a = lane & 7; a < m; a += 8) {
                             const int x = sh.tm.mem[a];
                             at |= x == row ? (unsigned)a : x == col ? (unsigned)a << 8 : 0u;
@@ -2700,6 +2788,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 const int linkage = p.linkage;
                 const bool chain = linkage != 0 && linkage != 5;
                 constexpr int ALL = kTeam * kTeam / 2, U = (ALL + TA - 1) / TA > 8 ? 8 : (ALL + TA - 1) / TA;
+#pragma unroll 1
                 for (int e0 = tid; e0 < ALL; e0 += U * TA) {
                     float v[U];
 #pragma unroll
@@ -2729,6 +2818,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 if (full) {
                     // the lines of the members' rows that the merges will read
                     const int nblk = R / 32;
+#pragma unroll 1
                     for (int e = tid; e < m * nblk; e += TA) {
                         const long long k = row_of((e / m) * 32);
                         const float *line = p.D + sh.tm.mbase[e % m] + k;
@@ -2743,6 +2833,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     // per member row (columns above it): which cells are at or below
                     // the bound, and the smallest of them
                     const unsigned thv = sh.tm.thv;
+#pragma unroll 1
                     for (int a = warp; a < m; a += WA) {
                         const unsigned v0 = __float_as_uint(sh.tm.S[a][lane]);
                         const unsigned v1 = __float_as_uint(sh.tm.S[a][lane + 32]);
@@ -2774,6 +2865,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 // step 2)
                 if (grid_wait(p, p.bar + kBar2, epoch2, sh, sync_a)) {
                     const int L = sh.tm.L;
+#pragma unroll 1
                     for (int q = tid; q < 2 * L; q += TA) {
                         const int x = sh.tm.mem[q < L ? sh.tm.mi(q) : sh.tm.mj(q - L)];
                         atomicOr(&touched[x >> 5], 1u << (x & 31));
@@ -2805,6 +2897,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             // CTA would wait for it.
             const int nexec = sh.nexec;
             const int np = scan_pieces(G, nexec, early);
+#pragma unroll 1
             for (int w = G - 1 - b; w < nexec * np; w += G) {
                 const int s2 = w / np, piece = w % np;
                 const long long rr = sh.exec_row[s2];
@@ -2835,7 +2928,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
 
         // ---- apply the L merges to every live row k outside them, a chunk of
         // rows at a time; per chunk (1) the new cells D(k, survivor) of
-        // Section 4 step 3, a warp per 32 rows and 8 survivors, stored and kept
+        // Section 4 step 3, a warp per 32 rows and 4 survivors, stored and kept
         // in kvs, (2) per survivor the smallest of them above it, NT / kSurv
         // threads each, and the rows' caches, a thread each
         auto bookkeeping = [&]() {
@@ -2847,6 +2940,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     STCG(p.bar + kViol + (par ^ 1), 0u);
             }
             if (b == 0) {
+#pragma unroll 1
                 for (int q = tid; q < L; q += NT) {
                     STCG(p.merges + 2 * (t + q), (int32_t)sh.tm.mem[sh.tm.mi(q)]);
                     STCG(p.merges + 2 * (t + q) + 1, (int32_t)sh.tm.mem[sh.tm.mj(q)]);
@@ -2855,6 +2949,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 if (tid < ns)
                     STCG(p.size_g + sh.tm.sslot[tid], sh.tm.rec[sh.tm.sq[tid]].z + sh.tm.rec[sh.tm.sq[tid]].w);
             }
+#pragma unroll 1
             for (int q = tid; q < 2 * L; q += NT) {
                 const int x = sh.tm.mem[q < L ? sh.tm.mi(q) : sh.tm.mj(q - L)];
                 if (owner_of(x) == b) {
@@ -2889,6 +2984,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     sh.npieces = sh.viol < sh.tm.L ? 0 : scan_pieces(G, sh.nexec, early);
             }
             // slots to clear from `touched` after the next round
+#pragma unroll 1
             for (int a = tid; a < m; a += NT)
                 sh.ptouch[a] = sh.tm.mem[a];
             if (tid == 0)
@@ -2900,6 +2996,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
 #pragma unroll
         for (int q = 0; q < P; ++q)
             ps[q] = kNoKey;
+#pragma unroll 1
         for (int l0 = 0; l0 < R; l0 += CH) {
             const int rows = R - l0 < CH ? R - l0 : CH;
             bool wait = tie;
@@ -2923,6 +3020,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 }
                 const int V = sh.viol;
                 if (V >= L) {
+#pragma unroll 1
                     for (int it = warp; it < rows / 32 * ns; it += W) {
                         const int blk = it / ns, s = it % ns;
                         const int l = l0 + blk * 32 + lane;
@@ -2934,6 +3032,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     break;
                 }
                 // the merges from V on wait for another round
+#pragma unroll 1
                 for (int q = V + tid; q < L; q += NT) {
                     const int x = sh.tm.mem[sh.tm.mi(q)], y = sh.tm.mem[sh.tm.mj(q)];
                     atomicAnd(&touched[x >> 5], ~(1u << (x & 31)));
@@ -2952,6 +3051,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 bookkeeping();
                 // one CTA: the survivors' smallest cells to other survivors (those to the
                 // other members are among their owners' new cells), a lane each
+#pragma unroll 1
                 for (int s = warp; ONE && s < ns; s += W) {
                     u64 x = kNoKey;
                     if (lane < ns && sh.tm.sslot[lane] > sh.tm.sslot[s])
@@ -2969,6 +3069,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     }
                 }
                 if (b == 0) {
+#pragma unroll 1
                     for (int e = tid; e < ns * ns; e += NT) {
                         const int x = e / ns, y = e % ns;
                         if (x < y) {  // (the later last merge has the larger index)
@@ -2988,6 +3089,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 // survivor, so a row's words of the round go out together (by
                 // rows they would be one sector each)
                 const int sq = lane < ns ? sh.tm.sq[lane] : 0;
+#pragma unroll 1
                 for (int q = warp; q < rows; q += W) {
                     if (lane < ns && ((sh.okm[q >> 5] >> (q & 31)) & 1u))
                         STCG(p.TL + row_of(l0 + q) * p.pitch + t + sq, kvs[(size_t)q * KVP + lane]);
@@ -3020,6 +3122,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     }
                 }
             }
+#pragma unroll 1
             for (int q = tid; q < rows; q += NT) {
                 const int l = l0 + q;
                 const long long k = row_of(l);
@@ -3047,6 +3150,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     }
                     const float *kr = kvs + (size_t)q * KVP;
                     // (those of merges put off again go)
+#pragma unroll 1
                     for (hm &= ns < 32 ? (1u << ns) - 1u : kFull; hm != 0u; hm &= hm - 1u) {
                         const int s = __ffs(hm) - 1;
                         const unsigned vb = __float_as_uint(kr[s]);
@@ -3132,6 +3236,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
         {
             const int nresc = sh.nresc;
             if (ONE) {
+#pragma unroll 1
                 for (int q = warp; q < nresc; q += W) {
                     const int l = rlist[q];
                     u64 top[K], next;
@@ -3143,6 +3248,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     }
                 }
             } else {
+#pragma unroll 1
                 for (int q = 0; q < nresc; ++q) {
                     const int l = rlist[q];
                     if (full)
@@ -3197,8 +3303,10 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             if (p.timing) {
                 ty.ph[1] += ty.xs[5] + ty.xs[0] + ty.xs[1] + ty.xs[2] + ty.xs[3];
                 ty.ph[5] += ty.xs[4] + ty.xs[6] + ty.xs[7];
+#pragma unroll 1
                 for (int q = 0; q < 6; ++q)
                     atomicAdd(St + 8 + q, ty.ph[q]);
+#pragma unroll 1
                 for (int q = 0; q < 8; ++q)
                     atomicAdd(St + 16 + q, ty.xs[q]);
             }
@@ -3257,6 +3365,7 @@ __global__ void __launch_bounds__(NT, MINB) batch_kernel(BatchParams bp)
         p.skip_arrive_cta = -1;
         p.timing = 0;
         // the slot keeps the previous job's words: clear the ones that must start at zero
+#pragma unroll 1
         for (size_t q = threadIdx.x; q < (L.total - L.zero) / 4; q += NT)
             reinterpret_cast<int *>(ws + L.zero)[q] = 0;
         __syncthreads();
@@ -3285,6 +3394,7 @@ __global__ void __launch_bounds__(256) expand_kernel(const float *__restrict__ P
         return;
     const int tx = threadIdx.x, ty = threadIdx.y;
     int bad = 0;
+#pragma unroll 1
     for (int yy = ty; yy < 32; yy += 8) {
         const long long r = tr * 32 + yy, c = tc * 32 + tx;
         float v = 0.0f;
@@ -3300,6 +3410,7 @@ __global__ void __launch_bounds__(256) expand_kernel(const float *__restrict__ P
         tile[yy][tx] = v;
     }
     __syncthreads();
+#pragma unroll 1
     for (int yy = ty; yy < 32; yy += 8) {
         const long long c = tc * 32 + yy, r = tr * 32 + tx;
         if (c > r && c < n)
@@ -3417,6 +3528,7 @@ int merge_chunk_rows(long long n, int G, int nt)
     // the registers allow, else whatever fits at all
     const long long sm = 228 * 1024, cta = 227 * 1024, fixed = (long long)static_smem(nt, G);
     const long long share = sm / (kThreads / nt) - 1024 - fixed;
+#pragma unroll 1
     for (int c = most; c >= 32 && 2 * c >= most; c = (c / 2) & ~31)
         if ((long long)smem_for(n, G, c) <= share)
             return c;
