@@ -73,7 +73,7 @@
 // barriers and about 13 merges per round) took 46.1 ms for n = 16384 average
 // linkage, 162.8 ms for single and 16.8 ms for n = 1968 (complete, on one CTA
 // then); selecting up to 64 members by a threshold and merging inside them takes
-// 25.6, 51 and 2.4 ms.  Next, the instructions themselves: each step's code
+// 25.2, 49.5 and 2.4 ms.  Next, the instructions themselves: each step's code
 // runs once or twice per round, so most of it is fetched anew every round
 // (n = 2000: 58 % of the SM's instruction cache requests hit, and waiting for
 // instructions was the largest stall after barriers, 3.7 of 11 cycles per
@@ -161,17 +161,6 @@ __device__ __forceinline__ long long row_base(const MergeParams &p, long long r)
     return p.full ? r * p.pitch : tri_off(r, p.n) - r - 1;
 }
 
-
-// Cell {x, y} read directly (the cells between members of a round's chain),
-// the slots' stamps sx, sy given.  Row-log layout: the cell is current in the
-// row of M whose slot was stamped later (both rows hold the input value
-// while neither slot has merged).
-__device__ __forceinline__ float member_cell(const MergeParams &p, long long x, int sx, long long y, int sy)
-{
-    if (!p.full)
-        return LDCG(p.D + pair_idx(x, y, p.n));
-    return sx >= sy ? LDCG(p.D + x * p.pitch + y) : LDCG(p.D + y * p.pitch + x);
-}
 
 __device__ __forceinline__ u64 make_key(float v, unsigned c)
 {
@@ -583,9 +572,11 @@ __device__ bool grid_wait(const MergeParams &p, const unsigned *bar, unsigned ep
 }
 
 // Live-column test against the CTA's copy of the liveness bitmap.
+// (slots fit 24 bits: 32-bit indices are half the instructions)
 __device__ __forceinline__ bool live(const unsigned *bitmap, long long c)
 {
-    return (bitmap[c >> 5] >> (c & 31)) & 1u;
+    const unsigned i = (unsigned)c;
+    return (bitmap[i >> 5] >> (i & 31u)) & 1u;
 }
 
 // Adds one input cell to a per-lane list during the initial scan: checks it
@@ -1670,7 +1661,7 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
     const int tid = threadIdx.x, lane = tid & 31;
     const int b = sh.cx.b, G = ONE ? 1 : sh.cx.G;
     auto rows_at = [&](int l) -> long long {
-        return ONE ? (long long)l : (long long)((long long)b + (long long)G * (l >> 5)) * kRowBlock + (l & 31);
+        return (long long)(ONE ? l : (b + G * (l >> 5)) * kRowBlock + (l & 31));
     };
     constexpr int KVP = kSurv + 1;
     const long long n = p.n;
@@ -1786,7 +1777,7 @@ __device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &s
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = sh.cx.b, G = ONE ? 1 : sh.cx.G;
     auto rows_at = [&](int l) -> long long {
-        return ONE ? (long long)l : (long long)((long long)b + (long long)G * (l >> 5)) * kRowBlock + (l & 31);
+        return (long long)(ONE ? l : (b + G * (l >> 5)) * kRowBlock + (l & 31));
     };
     constexpr int W = NT / 32;
     const int R = sh.cx.R;
@@ -1794,7 +1785,7 @@ __device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &s
     const u64 *ck = sh.cx.ck, *cB = sh.cx.cB;
     const unsigned char *ccnt = sh.cx.ccnt;
     const int *pend_t = sh.cx.pend_t;
-    auto slot_of = [&](long long r) -> int { return (int)(((r / kRowBlock) / G) * kRowBlock + (r & 31)); };
+    auto slot_of = [&](long long r) -> int { return (int)(((unsigned)r / kRowBlock / (unsigned)G) * kRowBlock + ((unsigned)r & 31u)); };
     RecA *rec = p.recA + (size_t)(rr & 1) * G + b;
     // a pivot that takes in at least kPub rows' first entries, then the
     // entries up to it in order by counting
@@ -2023,12 +2014,11 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
     unsigned char *const &ccnt = sh.cx.ccnt;
 
     auto row_of = [&](int l) -> long long {
-        return ONE ? (long long)l
-                   : (long long)((long long)b + (long long)G * (l >> 5)) * kRowBlock + (l & 31);
+        return (long long)(ONE ? l : (b + G * (l >> 5)) * kRowBlock + (l & 31));
     };
-    auto owner_of = [&](long long r) -> int { return ONE ? 0 : (int)((r / kRowBlock) % G); };
+    auto owner_of = [&](long long r) -> int { return ONE ? 0 : (int)((unsigned)r / kRowBlock % (unsigned)G); };
     auto slot_of = [&](long long r) -> int {
-        return ONE ? (int)r : (int)(((r / kRowBlock) / G) * kRowBlock + (r & 31));
+        return ONE ? (int)r : (int)(((unsigned)r / kRowBlock / (unsigned)G) * kRowBlock + ((unsigned)r & 31u));
     };
     auto cache_load = [&](u64 (&L)[K], int l) {
 #pragma unroll
@@ -2797,7 +2787,14 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         const int a = e & (kTeam - 1), c = (a + (e / kTeam) + 1) & (kTeam - 1);
                         v[u] = 0.0f;
                         if (e < ALL && a < m && c < m)
-                            v[u] = member_cell(p, sh.tm.mem[a], sh.tm.mst[a], sh.tm.mem[c], sh.tm.mst[c]);
+                            {
+                            // row-log layout: the cell is current in the row of M
+                            // whose slot was stamped later (both rows hold the input
+                            // value while neither has merged)
+                            const int x = sh.tm.mem[a], y = sh.tm.mem[c];
+                            const bool of_a = full ? sh.tm.mst[a] >= sh.tm.mst[c] : x < y;
+                            v[u] = LDCG(p.D + (of_a ? sh.tm.mbase[a] + y : sh.tm.mbase[c] + x));
+                        }
                     }
                     if (chain && warp == 0 && e0 == tid)
                         chain_select(sh.tm);
@@ -3494,19 +3491,20 @@ size_t smem_for(long long n, int G, int chunk)
 
 // CTAs for n objects when the caller names no number.  One up to 416 objects: a
 // block of 32 rows per CTA and grid barriers are slower there (complete, ms,
-// one CTA / grid: n = 300 0.69 / 0.82, n = 400 0.96 / 1.01, n = 512 1.24 / 1.07,
-// n = 1000 3.30 / 1.64, n = 2048 12.6 / 2.8).  Centroid linkage makes few merges
-// per round and none side by side, so the barriers weigh more: 16.7 / 21.5 at
-// n = 1000, 36.6 / 35.7 at 1600, 54.4 / 46.0 at 2048.  Above, one CTA per block
-// up to 64 of them, then one per two blocks (complete: n = 3500 64 CTAs 4.64,
-// 96 4.57; average: n = 5003 80 CTAs 6.42, 152 6.49; n = 8191 96 10.9, 128 10.3),
-// at most one per SM.  Single linkage (the merges of a round are worked out one
-// by one, and every CTA repeats them) runs better on fewer CTAs with the same
-// most blocks per CTA (n = 16384: 128 35.8, 152 36.4; the others 25.5 and 25.0).
+// one CTA / grid: n = 300 0.61 / 0.69, n = 400 0.86 / 0.87, n = 512 1.14 / 0.91,
+// n = 1000 3.13 / 1.39, n = 2048 12.2 / 2.4).  Centroid linkage makes few merges
+// per round and none side by side, so the barriers weigh more: 15.2 / 16.7 at
+// n = 1000, 23.3 / 22.3 at 1300, 49.8 / 36.2 at 2048.  Above, one CTA per block
+// up to 64 of them, then one per two blocks, at most one per SM (complete: n = 3500
+// 64 CTAs 4.11, 96 3.99; n = 4096 64 CTAs 4.81, 128 4.53; average: n = 5003 80 CTAs
+// 5.67, 152 5.55; n = 6500 96 7.66, 128 7.18): the last few percent would take
+// twice the SMs.  Single linkage (the merges of a round are worked out one by one,
+// and every CTA repeats them) runs better on fewer CTAs with the same most blocks
+// per CTA (n = 16384: 128 31.9, 152 32.4; Ward 23.5 and 22.0).
 int default_grid(long long n, int linkage, int num_sms)
 {
     const long long nb = (n + kRowBlock - 1) / kRowBlock;
-    if (n <= (linkage == LW_CENTROID ? 1536 : 416))
+    if (n <= (linkage == LW_CENTROID ? 1152 : 416))
         return 1;
     long long G = nb <= 64 ? nb : nb / 2 > 64 ? nb / 2 : 64;
     if (G > num_sms)
