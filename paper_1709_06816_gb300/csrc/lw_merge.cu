@@ -78,7 +78,8 @@
 // (n = 2000: 58 % of the SM's instruction cache requests hit, and waiting for
 // instructions was the largest stall after barriers, 3.7 of 11 cycles per
 // instruction outside them).  That is why no loop below is unrolled unless its
-// loads have to be in flight together: it took 5 to 9 % off every grid run.
+// loads have to be in flight together: it took 5 to 9 % off every grid run (72 %
+// of the requests hit since, and the stall is 1.5 cycles per instruction).
 //
 // Exact arithmetic: every product and sum of the update uses __fmul_rn /
 // __fadd_rn / __fsub_rn (never contracted into FMA), the coefficient
@@ -416,7 +417,7 @@ struct Shared {
     } ty;
 };
 
-// After barrier A: the list of rows to refill in this round -- every CTA's
+// After the main barrier: the list of rows to refill in this round -- every CTA's
 // requests in CTA order (deterministic, the same in every CTA), cut at
 // kMaxReq.  Thread t holds CTA t's request count and rows.  Sets
 // sh.exec_row and sh.nexec; thread b gives this CTA's own requests (list
