@@ -2344,7 +2344,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     pend_t[l] = -1;
                 }
             }
-            if (tid == TA)
+            if (tid == TA && inp != 0)
                 ty.installs += ninst;
             __syncthreads();
         }
@@ -2978,8 +2978,10 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 sh.nps = ns;
                 if (!ONE)
                     // (a scan beside merges that were put off again may have left
-                    // their columns out: its list is dropped)
-                    sh.npieces = sh.viol < sh.tm.L ? 0 : scan_pieces(G, sh.nexec, early);
+                    // their columns out: its list is dropped.  Only a round on
+                    // condition puts any off; others may take more merges than
+                    // viol's start, kSurv)
+                    sh.npieces = tie && sh.viol < sh.tm.L ? 0 : scan_pieces(G, sh.nexec, early);
             }
             // slots to clear from `touched` after the next round
 #pragma unroll 1
