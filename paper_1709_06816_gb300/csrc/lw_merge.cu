@@ -666,7 +666,7 @@ __device__ __forceinline__ void take_batch(const MergeParams &p, long long j0, i
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         const long long j = j0 + (long long)u * stride;
-        const float4 x = j < j1 ? LDCG(D4 + j) : make_float4(-1.0f, -1.0f, -1.0f, -1.0f);
+        const float4 x = j < j1 ? LDCG(D4 + j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
     }
     const int c0 = (int)((j0 << 2) + base_c);
@@ -674,7 +674,8 @@ __device__ __forceinline__ void take_batch(const MergeParams &p, long long j0, i
     int had = 0;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        if (v[u][0] >= 0.0f) {
+        // (the index, not the value: a cell may be NaN once the recurrence overflowed)
+        if (j0 + (long long)u * stride < j1) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int c = c0 + 4 * u * stride + e;
