@@ -25,7 +25,7 @@ constexpr int kRankBits = 4;             // an entry's rank in its row
 constexpr unsigned kRankMask = 15u;
 constexpr int kBar2 = 32;                // words of the second and third barrier counter and of
 constexpr int kBar3 = 48;                // the first conditional merge that must wait (two, by
-constexpr int kViol = 8;                 // round parity; kSurv less it, 0: none)
+constexpr int kViol = 8;                 // round parity; kTeam less it, 0: none)
 constexpr int kRedoBelow = 16;           // a chain cut below this many merges, and below half its
 constexpr int kRedoGap = 4;              // length (and a bit), is walked step by step instead
 constexpr int kTieGain = 3;              // merges a round must gain to take them on condition

@@ -18,7 +18,8 @@
 //
 // Rounds.  A grid barrier costs about a microsecond on GB300, and a merge by
 // itself less, so a round takes as many consecutive merges of the sequential
-// iteration as it can prove from one exchange (up to 32).  The merges are
+// iteration as it can prove from one exchange (up to 63, into at most 32 merged
+// clusters).  The merges are
 // exactly those of the step-by-step algorithm (same pairs, same order, same
 // rounded values); only the bookkeeping differs.  One round:
 //
@@ -43,11 +44,13 @@
 //      and the limits checked side by side (the chain); where cells made by the
 //      round's own merges cut it short, and for single and centroid linkage,
 //      one warp takes the merges step by step.
-//   on condition  the bounds for outside cells may end a chain that the cells
-//      themselves would not (many equal values).  When that costs kTieGain
-//      merges or more, the merges are taken on condition: the new cells are
-//      computed and kept back, every CTA looks whether one of its own comes
-//      before a merge of the round, and barrier 3 tells which merges stand.
+//   on condition  the bounds for outside cells may end a round that the cells
+//      themselves would not (equal values; inversions; values small against the
+//      largest, for single linkage).  When that costs kTieGain merges of a chain,
+//      or half as many steps as were proved (see simulate), the merges are taken
+//      on condition: the new cells are computed and kept back, every CTA looks
+//      whether one of its own comes before a merge of the round, and barrier 3
+//      tells which merges stand (settle).
 //   apply  behind barrier 2 (no CTA still reads the members' old cells): the new
 //      cells D(k, survivor) for every live k, a warp per 32 rows and up to 4
 //      survivors, all loads of an item in flight at once; then logs, caches
@@ -333,8 +336,13 @@ struct Team {
     unsigned char step[kEntries];
     unsigned char ce[kSurv];     // entry of merge q
     unsigned char ex[kTeam];     // entry that ends a member's row (0xff: none)
-    int tie;                     // the merges wait for a look at the cells outside
     int redo;                    // the chain broke off early: step by step instead
+    // merges on condition (tie): they wait for a look at the cells outside, those
+    // from `sure` on (cmax: their largest height); taken step by step (steps):
+    // how many at most the next time (reach)
+    int tie, sure, steps, reach;
+    unsigned cmax;
+    unsigned char cons[kTeam];   // merge that takes in the cluster of merge q (L: none)
     float X[kSurv][kTeam + 1];
     float C[kSurv][kSurv + 1];
     unsigned lim[kSurv];
@@ -1047,8 +1055,13 @@ __device__ __forceinline__ unsigned merged_bound(int lab, int lbb, float fi, flo
 // its time: everything is computed for all 64 members without branches, and
 // what rarely happens (a lost minimum with other cells below the bound, a new
 // cell below it, equal values at a bound) sits behind votes.
+template <bool B>
+struct Flag {
+    static constexpr bool value = B;
+};
+
 template <int LK>
-__device__ __noinline__ void simulate_steps(Team &tm, int &L_out, bool &dep_out)
+__device__ __noinline__ void simulate_steps(Team &tm, int reach, int per, int &L_out, int &sure_out)
 {
     const int lane = threadIdx.x & 31;
     const int m = tm.m;
@@ -1072,159 +1085,188 @@ __device__ __noinline__ void simulate_steps(Team &tm, int &L_out, bool &dep_out)
         tm.res[a] = 0;
     }
     u64 merged = 0ull;
-    bool dep = false;
-    int L = 0;
+    int L = 0, sure = -1;
     __syncwarp();
-    while (L < kTeam - 1) {
-        const bool sec = nv[1] < nv[0] || (nv[1] == nv[0] && nc[1] < nc[0]);
-        const unsigned v1 = sec ? nv[1] : nv[0], c1 = sec ? nc[1] : nc[0];
-        const unsigned hb = __reduce_min_sync(kFull, v1);
-        const unsigned lbmin = __reduce_min_sync(kFull, lbv[0] < lbv[1] ? lbv[0] : lbv[1]);
-        const unsigned code = __reduce_min_sync(kFull, v1 == hb ? c1 : kNone);
-        if (code == kNone)
-            break;
-        const int i = (int)(code >> 8), j = (int)(code & 0xffu);
-        if (hb >= lbmin) {
-            // equal values: whole keys against the bounds that are keys (those
-            // of merged clusters are values)
-            const u64 kA = ((u64)hb << 32) | (unsigned)tm.mem[i];
-            const unsigned kC = (unsigned)tm.mem[j];
-            bool ok = kA < tm.thA || (kA == tm.thA && kC < tm.thC);
+    // `most` merges at most; false: a merge was not proved, but nothing known comes
+    // before it
+    auto run = [&](auto cond, int most) -> bool {
+        while (L < most) {
+            const bool sec = nv[1] < nv[0] || (nv[1] == nv[0] && nc[1] < nc[0]);
+            const unsigned v1 = sec ? nv[1] : nv[0], c1 = sec ? nc[1] : nc[0];
+            const unsigned hb = __reduce_min_sync(kFull, v1);
+            const unsigned lbmin = __reduce_min_sync(kFull, lbv[0] < lbv[1] ? lbv[0] : lbv[1]);
+            const unsigned code = __reduce_min_sync(kFull, v1 == hb ? c1 : kNone);
+            if (code == kNone)
+                return true;
+            const int i = (int)(code >> 8), j = (int)(code & 0xffu);
+            if (hb >= lbmin) {
+                // equal values: whole keys against the bounds that are keys (those
+                // of merged clusters are values; on condition thv, so that the bound of
+                // the cells not listed is still asked)
+                const u64 kA = ((u64)hb << 32) | (unsigned)tm.mem[i];
+                const unsigned kC = (unsigned)tm.mem[j];
+                bool ok = kA < tm.thA || (kA == tm.thA && kC < tm.thC), proved = true;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int a = lane + 32 * h;
+                    if (lv[h]) {
+                        if ((merged >> a) & 1ull)
+                            proved = proved && hb < lbv[h];
+                        else
+                            ok = ok && (kA < tm.lbA[a] || (kA == tm.lbA[a] && kC < tm.lbC[a]));
+                    }
+                }
+                if (!__all_sync(kFull, ok))
+                    return true;
+                if (!decltype(cond)::value && !__all_sync(kFull, proved))
+                    return false;
+            }
+            float ca[2], cb[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int a = lane + 32 * h;
-                if (lv[h]) {
-                    if ((merged >> a) & 1ull)
-                        ok = ok && hb < lbv[h];
-                    else
-                        ok = ok && (kA < tm.lbA[a] || (kA == tm.lbA[a] && kC < tm.lbC[a]));
-                }
+                ca[h] = row[h][i];
+                cb[h] = row[h][j];
             }
-            if (!__all_sync(kFull, ok))
-                break;
-        }
-        float ca[2], cb[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            ca[h] = row[h][i];
-            cb[h] = row[h][j];
-        }
-        const int2 si = tm.sl[i], sj = tm.sl[j];
-        const float hgt = __uint_as_float(hb);
-        const float fi = (float)si.x, fj = (float)sj.x, fs = (float)(si.x + sj.x);
-        const float4 co = merge_coefs<LK>(si.x, sj.x, hgt);
-        const u64 bi = 1ull << i, bj = 1ull << j;
-        bool low[2], lost[2];
-        float v[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int k = lane + 32 * h;
-            v[h] = LK == 3 ? ward_cell(fi, fj, fs, fk[h], hgt, ca[h], cb[h])
-                           : lw_sum(co.x, co.y, co.z, co.w, ca[h], cb[h]);
-            row[h][i] = v[h];
-            tm.S[i][k] = v[h];
-            lv[h] = lv[h] && k != j;
-            low[h] = lv[h] && k != i && __float_as_uint(v[h]) <= thv;
-            const unsigned c = nc[h] & 0xffu;
-            lost[h] = (c == (unsigned)i || c == (unsigned)j) && k != i;  // (a column above k)
-            mk[h] &= ~(bi | bj);
-            nv[h] = lost[h] || k == j ? kNone : nv[h];
-            nc[h] = lost[h] || k == j ? kNone : nc[h];
-        }
-        const unsigned nbits = merged_bound<LK>(si.y, sj.y, fi, fs, hgt, tm.dmax);
-        merged |= bi;
-        const unsigned more = __ballot_sync(kFull, (lost[0] && mk[0] != 0ull && lv[0]) || (lost[1] && mk[1] != 0ull && lv[1]));
-        const unsigned l0 = __ballot_sync(kFull, low[0]), l1 = __ballot_sync(kFull, low[1]);
-        if (more) {
+            const int2 si = tm.sl[i], sj = tm.sl[j];
+            const float hgt = __uint_as_float(hb);
+            const float fi = (float)si.x, fj = (float)sj.x, fs = (float)(si.x + sj.x);
+            const float4 co = merge_coefs<LK>(si.x, sj.x, hgt);
+            const u64 bi = 1ull << i, bj = 1ull << j;
+            bool low[2], lost[2];
+            float v[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int k = lane + 32 * h;
-                if (lost[h] && lv[h]) {
+                if constexpr (decltype(cond)::value)
+                    tm.X[L - sure][k] = ca[h];  // (steps_undo puts it back)
+                v[h] = LK == 3 ? ward_cell(fi, fj, fs, fk[h], hgt, ca[h], cb[h])
+                               : lw_sum(co.x, co.y, co.z, co.w, ca[h], cb[h]);
+                row[h][i] = v[h];
+                tm.S[i][k] = v[h];
+                lv[h] = lv[h] && k != j;
+                low[h] = lv[h] && k != i && __float_as_uint(v[h]) <= thv;
+                const unsigned c = nc[h] & 0xffu;
+                lost[h] = (c == (unsigned)i || c == (unsigned)j) && k != i;  // (a column above k)
+                mk[h] &= ~(bi | bj);
+                nv[h] = lost[h] || k == j ? kNone : nv[h];
+                nc[h] = lost[h] || k == j ? kNone : nc[h];
+            }
+            const unsigned nbits = decltype(cond)::value ? thv : merged_bound<LK>(si.y, sj.y, fi, fs, hgt, tm.dmax);
+            merged |= bi;
+            const unsigned more = __ballot_sync(kFull, (lost[0] && mk[0] != 0ull && lv[0]) || (lost[1] && mk[1] != 0ull && lv[1]));
+            const unsigned l0 = __ballot_sync(kFull, low[0]), l1 = __ballot_sync(kFull, low[1]);
+            if (more) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int k = lane + 32 * h;
+                    if (lost[h] && lv[h]) {
 #pragma unroll 1
-                    for (u64 q = mk[h]; q; q &= q - 1) {
-                        const int c = __ffsll((long long)q) - 1;
-                        const unsigned x = __float_as_uint(row[h][c]), y = (unsigned)(k << 8 | c);
+                        for (u64 q = mk[h]; q; q &= q - 1) {
+                            const int c = __ffsll((long long)q) - 1;
+                            const unsigned x = __float_as_uint(row[h][c]), y = (unsigned)(k << 8 | c);
+                            if (x < nv[h] || (x == nv[h] && y < nc[h])) {
+                                nv[h] = x;
+                                nc[h] = y;
+                            }
+                        }
+                    }
+                }
+            }
+            unsigned ri = kNone, rc = kNone;
+            u64 rm = 0ull;
+            if (l0 | l1) {
+                // new cells at or below the bound: those of rows k < i, and row i's
+                unsigned w[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int k = lane + 32 * h;
+                    const unsigned x = __float_as_uint(v[h]), y = (unsigned)(k << 8 | i);
+                    if (low[h] && k < i) {
+                        mk[h] |= bi;
                         if (x < nv[h] || (x == nv[h] && y < nc[h])) {
                             nv[h] = x;
                             nc[h] = y;
                         }
                     }
+                    w[h] = low[h] && k > i ? x : kNone;
                 }
+                rm = (((u64)l1 << 32) | l0) & ~((bi << 1) - 1ull);
+                ri = __reduce_min_sync(kFull, w[0] < w[1] ? w[0] : w[1]);
+                const unsigned k0 = w[0] == ri ? (unsigned)lane : 64u, k1 = w[1] == ri ? (unsigned)lane + 32u : 64u;
+                const unsigned kk = __reduce_min_sync(kFull, k0 < k1 ? k0 : k1);
+                rc = rm ? ((unsigned)i << 8 | kk) : kNone;
             }
-        }
-        unsigned ri = kNone, rc = kNone;
-        u64 rm = 0ull;
-        if (l0 | l1) {
-            // new cells at or below the bound: those of rows k < i, and row i's
-            unsigned w[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int k = lane + 32 * h;
-                const unsigned x = __float_as_uint(v[h]), y = (unsigned)(k << 8 | i);
-                if (low[h] && k < i) {
-                    mk[h] |= bi;
-                    if (x < nv[h] || (x == nv[h] && y < nc[h])) {
-                        nv[h] = x;
-                        nc[h] = y;
-                    }
+                if (k == i) {
+                    mk[h] = rm;
+                    nv[h] = ri;
+                    nc[h] = rc;
+                    lbv[h] = nbits;
+                    fk[h] = fs;
                 }
-                w[h] = low[h] && k > i ? x : kNone;
+                if (k == j) {
+                    mk[h] = 0ull;
+                    lbv[h] = kNone;
+                }
             }
-            rm = (((u64)l1 << 32) | l0) & ~((bi << 1) - 1ull);
-            ri = __reduce_min_sync(kFull, w[0] < w[1] ? w[0] : w[1]);
-            const unsigned k0 = w[0] == ri ? (unsigned)lane : 64u, k1 = w[1] == ri ? (unsigned)lane + 32u : 64u;
-            const unsigned kk = __reduce_min_sync(kFull, k0 < k1 ? k0 : k1);
-            rc = rm ? ((unsigned)i << 8 | kk) : kNone;
+            const int qi = tm.res[i], qj = tm.res[j];
+            __syncwarp();
+            if (lane == 0) {
+                tm.rec[L] = make_int4(i | j << 8 | qi << 16 | qj << 24, (int)hb, si.x, sj.x);
+                if (LK != 3)
+                    tm.co[L] = co;
+                tm.res[i] = L + 1;
+                tm.sl[i] = make_int2(si.x + sj.x, (int)nbits);
+            }
+            ++L;
+            __syncwarp();
         }
+        return true;
+    };
+    if (!run(Flag<false>(), kTeam - 1)) {
+        // from here on condition: the merged clusters' cells will be looked at
+        sure = L;
+        if (per * reach >= L) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                lbv[h] = lv[h] && ((merged >> (lane + 32 * h)) & 1ull) ? thv : lbv[h];
+            run(Flag<true>(), min(L + reach, kTeam - 1));
+        }
+    }
+    L_out = L;
+    sure_out = sure < 0 ? L : sure;
+}
+
+// Takes back merges V .. L - 1 of simulate_steps (all on condition): the cells
+// between members are again those after V merges.
+__device__ __forceinline__ void steps_undo(Team &tm, int L, int V, int sure)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int e = L - 1; e >= V; --e) {
+        const int i = tm.mi(e);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int k = lane + 32 * h;
-            if (k == i) {
-                mk[h] = rm;
-                nv[h] = ri;
-                nc[h] = rc;
-                lbv[h] = nbits;
-                fk[h] = fs;
-            }
-            if (k == j) {
-                mk[h] = 0ull;
-                lbv[h] = kNone;
-            }
+            const float x = tm.X[e - sure][k];
+            tm.S[k][i] = x;
+            tm.S[i][k] = x;
         }
-        const int qi = tm.res[i], qj = tm.res[j];
-        dep = dep || (qi | qj) != 0;
-        __syncwarp();
-        if (lane == 0) {
-            tm.rec[L] = make_int4(i | j << 8 | qi << 16 | qj << 24, (int)hb, si.x, sj.x);
-            if (LK != 3)
-                tm.co[L] = co;
-            tm.res[i] = L + 1;
-            tm.sl[i] = make_int2(si.x + sj.x, (int)nbits);
-        }
-        ++L;
         __syncwarp();
     }
-    L_out = L;
-    dep_out = dep;
 }
 
-// The round's merges by simulate_steps (warp 0, the members' cells in S and
-// their minima ready), and those that lead to each survivor, in order.  For
-// single and centroid linkage, whose merges mostly take part in one another,
-// and where the chain (below) breaks off early for that reason.
-__device__ __noinline__ void simulate(Team &tm, int linkage)
+// The first L merges of simulate_steps (their cells between members in S): those
+// that lead to each survivor, in order, and the survivors' cells to one another.
+__device__ __noinline__ void steps_program(Team &tm, int L)
 {
     const int lane = threadIdx.x & 31;
-    int L;
-    bool dep;
-    switch (linkage) {
-    case 0: simulate_steps<0>(tm, L, dep); break;
-    case 1: simulate_steps<1>(tm, L, dep); break;
-    case 2: simulate_steps<2>(tm, L, dep); break;
-    case 3: simulate_steps<3>(tm, L, dep); break;
-    case 4: simulate_steps<4>(tm, L, dep); break;
-    default: simulate_steps<5>(tm, L, dep); break;
-    }
+    const bool dep = __any_sync(kFull, (lane < L && ((unsigned)tm.rec[lane].x >> 16) != 0u) ||
+                                           (lane + 32 < L && ((unsigned)tm.rec[lane + 32].x >> 16) != 0u));
+    tm.cons[lane] = (unsigned char)L;
+    tm.cons[lane + 32] = (unsigned char)L;
     int ns = L;
     if (!dep) {
         // every merge joins two clusters of the round before: its own survivor
@@ -1245,10 +1287,14 @@ __device__ __noinline__ void simulate(Team &tm, int linkage)
             if (q < L) {
                 const int x = tm.rec[q].x;
                 const int si = (x >> 16) & 0xff, sj = (x >> 24) & 0xff;
-                if (si)
+                if (si) {
                     tm.root[si - 1] = q;  // (merge q consumes that result)
-                if (sj)
+                    tm.cons[si - 1] = (unsigned char)q;
+                }
+                if (sj) {
                     tm.root[sj - 1] = q;
+                    tm.cons[sj - 1] = (unsigned char)q;
+                }
             }
         }
         __syncwarp();
@@ -1317,10 +1363,8 @@ __device__ __noinline__ void simulate(Team &tm, int linkage)
         tm.sfirst[ns] = L;
         tm.L = L;
         tm.ns = ns;
-        tm.tie = 0;
     }
     __syncwarp();
-    // the survivors' cells to one another
     if (lane < ns) {
         const int a = tm.mi(tm.sq[lane]);
 #pragma unroll 1
@@ -1328,6 +1372,49 @@ __device__ __noinline__ void simulate(Team &tm, int linkage)
             tm.C[s][lane] = tm.S[tm.mi(tm.sq[s])][a];
     }
     __syncwarp();
+}
+
+// The round's merges by simulate_steps (warp 0, the members' cells in S and
+// their minima ready).  For single and centroid linkage, whose merges mostly
+// take part in one another, and where the chain (below) breaks off early for
+// that reason.  The bounds of the cells outside are weak there (single: a margin
+// of the matrix's largest value; centroid: up to a quarter of the height; zeros
+// and equal values anywhere), so the merges go on past them, on condition,
+// `reach` of them: twice as many as stood the last time (and 2).  That has to be
+// half of the proved ones (the look takes some 7 us of a round's 35), or all
+// where the cells outside are computed twice for it (twice: a CTA with several
+// chunks of rows).
+__device__ __noinline__ void simulate(Team &tm, int linkage, bool twice)
+{
+    const int lane = threadIdx.x & 31;
+    const int reach = tm.reach, per = twice ? 1 : 2;
+    int L, sure;
+    switch (linkage) {
+    case 0: simulate_steps<0>(tm, reach, per, L, sure); break;
+    case 1: simulate_steps<1>(tm, reach, per, L, sure); break;
+    case 2: simulate_steps<2>(tm, reach, per, L, sure); break;
+    case 3: simulate_steps<3>(tm, reach, per, L, sure); break;
+    case 4: simulate_steps<4>(tm, reach, per, L, sure); break;
+    default: simulate_steps<5>(tm, reach, per, L, sure); break;
+    }
+    const bool tie = L > sure && per * (L - sure) >= sure;
+    if (!tie) {
+        steps_undo(tm, L, sure, sure);
+        L = sure;
+    }
+    unsigned top = 0u;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (lane + 32 * h >= sure && lane + 32 * h < L)
+            top = max(top, (unsigned)tm.rec[lane + 32 * h].y);
+    top = __reduce_max_sync(kFull, top);
+    if (lane == 0) {
+        tm.tie = tie;
+        tm.sure = sure;
+        tm.steps = 1;
+        tm.cmax = top;
+    }
+    steps_program(tm, L);
 }
 
 // ---- the round's merges where they follow the entries (complete, group and
@@ -1518,6 +1605,7 @@ __device__ __forceinline__ void chain_accept(Team &tm, bool allow)
         tm.prog[lane] = lane;
         tm.sfirst[lane] = lane;
         tm.sq[lane] = lane;
+        tm.cons[lane] = (unsigned char)La;
         tm.sslot[lane] = tm.mem[tm.mi(lane)];
     }
     if (lane == 0) {
@@ -1525,6 +1613,9 @@ __device__ __forceinline__ void chain_accept(Team &tm, bool allow)
         tm.L = La;
         tm.ns = La;
         tm.tie = tie;
+        tm.sure = sure;
+        tm.steps = 0;
+        tm.cmax = La > 0 ? (unsigned)tm.rec[La - 1].y : 0u;
         // a cell made between members comes first: many merges are still known
         tm.redo = most < L && ((made_first >> most) & 1u) && most < kRedoBelow && 2 * most < L + kRedoGap;
     }
@@ -1566,13 +1657,34 @@ __device__ __noinline__ void chain_phase(Team &tm, int linkage, bool allow)
     sync_a();
 }
 
+// Merges on condition: a cell v of row k that merge q made, and that is there
+// until merge cons[q] takes its cluster in.  Does it come before one of the
+// merges meanwhile that no bound proved?  The first such goes to *viol.
+__device__ __noinline__ void outside_check(const Team &tm, int q, unsigned vb, unsigned k, int *viol)
+{
+    const unsigned x = (unsigned)tm.mem[tm.mi(q)];
+    const u64 kA = ((u64)vb << 32) | min(k, x);
+    const unsigned kC = max(k, x);
+    const int last = min((int)tm.cons[q], tm.L - 1);
+#pragma unroll 1
+    for (int e = max(q + 1, tm.sure); e <= last; ++e) {
+        const int4 rec = tm.rec[e];
+        const u64 eA = ((u64)(unsigned)rec.y << 32) | (unsigned)tm.mem[rec.x & 0xff];
+        if (eA > kA || (eA == kA && (unsigned)tm.mem[(rec.x >> 8) & 0xff] > kC)) {
+            atomicMin(viol, e);
+            break;
+        }
+    }
+}
+
 // Merges f + 1 .. f + len - 1 of a survivor's program for row k, whose first
-// merge gave v: the new cell after the last one.  An operand is a cell in
+// merge gave v: the new cell after the last one (CHECK: each is checked; a copy of
+// its own, the call would cost the others registers).  An operand is a cell in
 // memory or the result of an earlier merge of the program, mostly of the one
 // just before.
-template <bool ONE>
+template <bool ONE, bool CHECK>
 __device__ __noinline__ float chain_cells(const MergeParams &p, const Team &tm, int f, int len, float v, float nk,
-                                          long long k, int sk, bool ok)
+                                          long long k, int sk, bool ok, int *viol)
 {
     float tmp[kTeam];
     const bool full = !ONE && p.full;
@@ -1596,6 +1708,8 @@ __device__ __noinline__ float chain_cells(const MergeParams &p, const Team &tm, 
         const float a = si < 0 ? load(x & 0xff) : si == prev ? v : tmp[si];
         const float b = sj < 0 ? load((x >> 8) & 0xff) : sj == prev ? v : tmp[sj];
         v = merge_cell(tm, p.linkage, q, a, b, nk);
+        if (CHECK && ok && __float_as_uint(v) <= tm.cmax)
+            outside_check(tm, q, __float_as_uint(v), (unsigned)k, viol);
         prev = q;
     }
     return v;
@@ -1652,13 +1766,15 @@ __device__ __forceinline__ u64 find_pivot(F &&count, u64 least, u64 top, u64 gue
 
 // The new cells D(k, survivor) of Section 4 step 3 for the rows l0 .. l0 + rows
 // of a CTA outside the round's merges: into kvs (kvs[q * (kSurv + 1) + s]:
-// chunk row q, survivor s) and, unless the merges wait (tie), into memory.  A
-// warp takes 32 rows and 8 survivors at a time from a counter (team B comes in
-// when its scans are done): 16 loads in flight per thread; the rows of a warp
-// are consecutive, so row cells are read and written in whole lines.
+// chunk row q, survivor s) and into memory (kStore); with merges on condition
+// each is compared with the later merges and goes to kvs only (kKeep: the CTA's
+// rows are one chunk) or nowhere (kCheck).  A warp takes 32 rows and up to 4
+// survivors at a time from a counter (team B comes in when its scans are
+// done): 8 loads in flight per thread; the rows of a warp are consecutive, so
+// row cells are read and written in whole lines.
+constexpr int kStore = 0, kKeep = 1, kCheck = 2;
 template <int NT, bool ONE>
-__device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> &sh, int l0, int rows, int ns, int L,
-                                       bool tie)
+__device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> &sh, int l0, int rows, int ns, int mode)
 {
     const int tid = threadIdx.x, lane = tid & 31;
     const int b = sh.cx.b, G = ONE ? 1 : sh.cx.G;
@@ -1672,7 +1788,7 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
     float *kvs = sh.cx.kvs;
     const int *rsize = sh.cx.rsize, *rstamp = sh.cx.rstamp;
     const int nblk = rows / 32;
-    const unsigned last = L > 0 ? (unsigned)sh.tm.rec[L - 1].y : 0u;
+    int *const viol = mode != kStore ? &sh.viol : nullptr;
     constexpr int U = 4;  // (8: 6 % slower at n = 1968 and 16384, twice the instructions)
     // (fewer survivors at a time when that leaves no warp without an item)
     int ug = U;
@@ -1733,29 +1849,18 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
             const int f = sh.tm.sfirst[s], len = sh.tm.sfirst[s + 1] - f;
             const int q = sh.tm.prog[f];
             float v = merge_cell(sh.tm, p.linkage, q, va[u], vb[u], nk);
+            if (viol && ok && __float_as_uint(v) <= sh.tm.cmax)
+                outside_check(sh.tm, q, __float_as_uint(v), (unsigned)k, viol);
             if (len > 1)
-                v = chain_cells<ONE>(p, sh.tm, f, len, v, nk, k, sk, ok);
-            if (ok) {
+                v = viol ? chain_cells<ONE, true>(p, sh.tm, f, len, v, nk, k, sk, ok, viol)
+                         : chain_cells<ONE, false>(p, sh.tm, f, len, v, nk, k, sk, ok, viol);
+            if (ok && mode != kCheck) {
                 const long long x = sh.tm.sslot[s];
                 kvs[(size_t)(blk * 32 + lane) * KVP + s] = v;
                 if (x > k && __float_as_uint(v) <= bhi)
                     hm |= 1u << s;
-                if (tie) {
-                    // does it come before a later merge of the round?  (s = q)
-                    const unsigned vb = __float_as_uint(v);
-                    if (vb <= last) {
-                        const u64 kA = ((u64)vb << 32) | (unsigned)(k < x ? k : x);
-                        const unsigned kC = (unsigned)(k < x ? x : k);
-#pragma unroll 1
-                        for (int e = s + 1; e < L; ++e) {
-                            const int4 rec = sh.tm.rec[e];
-                            const u64 eA = ((u64)(unsigned)rec.y << 32) | (unsigned)sh.tm.mem[rec.x & 0xff];
-                            if (eA > kA || (eA == kA && (unsigned)sh.tm.mem[(rec.x >> 8) & 0xff] > kC)) {
-                                atomicMin(&sh.viol, e);
-                                break;
-                            }
-                        }
-                    }
+                if (mode == kKeep) {
+                    // (written when every merge stands)
                 } else if (full) {
                     // row x is rewritten whole; row k keeps its stale copy
                     // and the new value goes to k's log (below)
@@ -1768,6 +1873,97 @@ __device__ __forceinline__ void new_cells(const MergeParams &p, Shared<NT, ONE> 
         if (hm != 0u)
             atomicOr(&sh.hit[blk * 32 + lane], hm);
     }
+}
+
+// Merges taken on condition (the whole CTA, out of line: rounds without such
+// merges do not pay for it): the new cells first; every CTA looks whether one
+// of its own comes before a merge of the round that no bound proved, and
+// barrier 3 tells the first such, V.  Merges from V on wait for another round.
+// Returns 1 if the new cells are in kvs and in memory already, -1 if a wait ran
+// out.
+template <int NT, bool ONE>
+__device__ __noinline__ int settle(const MergeParams &p, Shared<NT, ONE> &sh, int par, unsigned &epoch3)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = sh.cx.b, G = ONE ? 1 : sh.cx.G;
+    auto row_of = [&](int l) -> long long {
+        return (long long)(ONE ? l : (b + G * (l >> 5)) * kRowBlock + (l & 31));
+    };
+    constexpr int W = NT / 32, KVP = kSurv + 1;
+    Team &tm = sh.tm;
+    const int R = sh.cx.R, CH = p.chunk;
+    unsigned *touched = sh.cx.touched;
+    const bool full = !ONE && p.full, one_chunk = sh.cx.Rmax <= CH;
+    const int L = tm.L, ns = tm.ns;
+#pragma unroll 1
+    for (int l0 = 0; l0 < R; l0 += CH) {
+        new_cells(p, sh, l0, R - l0 < CH ? R - l0 : CH, ns, one_chunk ? kKeep : kCheck);
+        __syncthreads();
+        if (l0 + CH < R) {
+            if (tid == 0)
+                sh.item = 0;
+            __syncthreads();
+        }
+    }
+    if (!ONE) {
+        if (tid == 0 && sh.viol < L)
+            atomicMax(p.bar + kViol + par, (unsigned)(kTeam - sh.viol));
+        grid_arrive(p, p.bar + kBar3, epoch3);
+        if (!grid_wait(p, p.bar + kBar3, epoch3, sh))
+            return -1;
+        if (tid == 0)
+            sh.viol = kTeam - ld_relaxed_s32(reinterpret_cast<const int *>(p.bar + kViol + par));
+        __syncthreads();
+    }
+    const int V = sh.viol < L ? sh.viol : L;
+    if (V == L && one_chunk) {
+#pragma unroll 1
+        for (int it = warp; it < R / 32 * ns; it += W) {
+            const int blk = it / ns, s = it % ns;
+            const int l = blk * 32 + lane;
+            const long long k = row_of(l), x = tm.sslot[s];
+            if ((sh.okm[blk] >> lane) & 1u)
+                STCG(full ? p.D + x * p.pitch + k : p.D + (k > x ? row_base(p, x) + k : row_base(p, k) + x),
+                     sh.cx.kvs[(size_t)l * KVP + s]);
+        }
+        if (tid == 0 && tm.steps)
+            tm.reach = min(max(2 * (V - tm.sure) + 2, 4), kSurv);
+        return 1;
+    }
+    sh.hit[tid] = 0u;
+    if (V < L) {
+#pragma unroll 1
+        for (int q = V + tid; q < L; q += NT) {
+            const int x = tm.mem[tm.mi(q)], y = tm.mem[tm.mj(q)];
+            atomicAnd(&touched[x >> 5], ~(1u << (x & 31)));
+            atomicAnd(&touched[y >> 5], ~(1u << (y & 31)));
+        }
+        __syncthreads();
+        // (a slot may take part in merges of both sides)
+#pragma unroll 1
+        for (int q = tid; q < V; q += NT) {
+            const int x = tm.mem[tm.mi(q)], y = tm.mem[tm.mj(q)];
+            atomicOr(&touched[x >> 5], 1u << (x & 31));
+            atomicOr(&touched[y >> 5], 1u << (y & 31));
+        }
+        if (tm.steps) {
+            if (warp == 0) {
+                steps_undo(tm, L, V, tm.sure);
+                steps_program(tm, V);
+            }
+        } else if (tid == 0) {
+            tm.sfirst[V] = V;
+            tm.L = V;
+            tm.ns = V;
+        }
+    }
+    if (tid == 0) {
+        sh.item = 0;
+        if (tm.steps)
+            tm.reach = min(max(2 * (V - tm.sure) + 2, 4), kSurv);
+    }
+    __syncthreads();
+    return 0;
 }
 
 // The record for round rr: this CTA's kPub smallest entries (cached keys and
@@ -2105,6 +2301,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
         sh.nptouch = 0;
         sh.nresc = 0;
         sh.tm.dmax = 0u;
+        sh.tm.reach = 4;
         sh.pivot = 0ull;
         sh.ppivot = 0ull;
         sh.limit = sh.width = 0u;
@@ -2290,11 +2487,6 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
             for (int s2 = W - 1 - warp; s2 < ninst; s2 += W) {
                 const int l = sh.inst_slot[s2];
                 const int pos = pend_s[l];
-                if (inp == 0) {
-                    if (lane == 0)
-                        pend_t[l] = -1;  // no list: the row may ask again
-                    continue;
-                }
                 const long long row = row_of(l);
                 // (one key per lane, kPartWords lanes per piece, then the K smallest
                 // of them; B, a lower bound of the row's other cells)
@@ -2345,7 +2537,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     pend_t[l] = -1;
                 }
             }
-            if (tid == TA && inp != 0)
+            if (tid == TA)
                 ty.installs += ninst;
             __syncthreads();
         }
@@ -2855,7 +3047,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     }
                     sync_a();
                     if (warp == 0)
-                        simulate(sh.tm, linkage);
+                        simulate(sh.tm, linkage, Rmax > CH);
                 }
                 sync_a();
                 lap(ty.xs[3]);
@@ -2863,18 +3055,21 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 // slots they take part in are marked, and slot j retires (Section 4
                 // step 2)
                 if (grid_wait(p, p.bar + kBar2, epoch2, sh, sync_a)) {
+                    // (on condition: j retires when the merge stands, with the
+                    // bookkeeping, so that the scans beside it leave no column out)
                     const int L = sh.tm.L;
+                    const bool tie = sh.tm.tie != 0;
 #pragma unroll 1
                     for (int q = tid; q < 2 * L; q += TA) {
                         const int x = sh.tm.mem[q < L ? sh.tm.mi(q) : sh.tm.mj(q - L)];
                         atomicOr(&touched[x >> 5], 1u << (x & 31));
-                        if (q >= L)
+                        if (q >= L && !tie)
                             atomicAnd(&bitmap[x >> 5], ~(1u << (x & 31)));
                     }
                 }
                 if (tid == 0) {
                     sh.item = 0;
-                    sh.viol = kSurv;
+                    sh.viol = kTeam;
                 }
                 if constexpr (ONE)
                     __syncthreads();
@@ -2951,6 +3146,8 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
 #pragma unroll 1
             for (int q = tid; q < 2 * L; q += NT) {
                 const int x = sh.tm.mem[q < L ? sh.tm.mi(q) : sh.tm.mj(q - L)];
+                if (tie && q >= L)
+                    atomicAnd(&bitmap[x >> 5], ~(1u << (x & 31)));
                 if (owner_of(x) == b) {
                     const int l = slot_of(x);
                     ccnt[l] = 0;
@@ -2978,11 +3175,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                 sh.ninst = 0;
                 sh.nps = ns;
                 if (!ONE)
-                    // (a scan beside merges that were put off again may have left
-                    // their columns out: its list is dropped.  Only a round on
-                    // condition puts any off; others may take more merges than
-                    // viol's start, kSurv)
-                    sh.npieces = tie && sh.viol < sh.tm.L ? 0 : scan_pieces(G, sh.nexec, early);
+                    sh.npieces = scan_pieces(G, sh.nexec, early);
             }
             // slots to clear from `touched` after the next round
 #pragma unroll 1
@@ -2997,57 +3190,23 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
 #pragma unroll
         for (int q = 0; q < P; ++q)
             ps[q] = kNoKey;
+        bool kept = false;  // the new cells are in kvs and in memory already
+        if (tie) {
+            const int k = settle<NT, ONE>(p, sh, par, epoch3);
+            if (k < 0)
+                return;
+            kept = k != 0;
+            L = sh.tm.L;
+            ns = sh.tm.ns;
+        }
 #pragma unroll 1
         for (int l0 = 0; l0 < R; l0 += CH) {
             const int rows = R - l0 < CH ? R - l0 : CH;
-            bool wait = tie;
-            while (true) {
-                new_cells(p, sh, l0, rows, ns, L, wait);
-                __syncthreads();
-                lap(ty.xs[4]);
-                if (!wait)
-                    break;
-                // the merges taken on condition: has any CTA found a cell that comes
-                // before one of them?
-                if (!ONE) {
-                    if (tid == 0 && sh.viol < L)
-                        atomicMax(p.bar + kViol + par, (unsigned)(kSurv - sh.viol));
-                    grid_arrive(p, p.bar + kBar3, epoch3);
-                    if (!grid_wait(p, p.bar + kBar3, epoch3, sh))
-                        return;
-                    if (tid == 0)
-                        sh.viol = kSurv - ld_relaxed_s32(reinterpret_cast<const int *>(p.bar + kViol + par));
-                    __syncthreads();
-                }
-                const int V = sh.viol;
-                if (V >= L) {
-#pragma unroll 1
-                    for (int it = warp; it < rows / 32 * ns; it += W) {
-                        const int blk = it / ns, s = it % ns;
-                        const int l = l0 + blk * 32 + lane;
-                        const long long k = row_of(l), x = sh.tm.sslot[s];
-                        if ((sh.okm[blk] >> lane) & 1u)
-                            STCG(full ? p.D + x * p.pitch + k : p.D + (k > x ? row_base(p, x) + k : row_base(p, k) + x),
-                                 kvs[(size_t)(blk * 32 + lane) * KVP + s]);
-                    }
-                    break;
-                }
-                // the merges from V on wait for another round
-#pragma unroll 1
-                for (int q = V + tid; q < L; q += NT) {
-                    const int x = sh.tm.mem[sh.tm.mi(q)], y = sh.tm.mem[sh.tm.mj(q)];
-                    atomicAnd(&touched[x >> 5], ~(1u << (x & 31)));
-                    atomicAnd(&touched[y >> 5], ~(1u << (y & 31)));
-                    atomicOr(&bitmap[y >> 5], 1u << (y & 31));
-                }
-                L = ns = V;
-                wait = false;
-                if (tid == 0) {
-                    sh.tm.sfirst[V] = V;
-                    sh.item = 0;
-                }
+            if (!kept) {
+                new_cells(p, sh, l0, rows, ns, kStore);
                 __syncthreads();
             }
+            lap(ty.xs[4]);
             if (l0 == 0) {
                 bookkeeping();
                 // one CTA: the survivors' smallest cells to other survivors (those to the
@@ -3150,9 +3309,8 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         c = list_count(Cc);
                     }
                     const float *kr = kvs + (size_t)q * KVP;
-                    // (those of merges put off again go)
 #pragma unroll 1
-                    for (hm &= ns < 32 ? (1u << ns) - 1u : kFull; hm != 0u; hm &= hm - 1u) {
+                    for (; hm != 0u; hm &= hm - 1u) {
                         const int s = __ffs(hm) - 1;
                         const unsigned vb = __float_as_uint(kr[s]);
                         const long long x = sh.tm.sslot[s];
