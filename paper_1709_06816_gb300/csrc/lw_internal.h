@@ -20,7 +20,7 @@ constexpr int kCand = 512;               // most entries up to a round's pivot
 constexpr int kHeadsHi = 64;             // most lists whose heads the pivot takes in
 constexpr int kPieces = 4;               // most pieces a refill row is scanned in
 constexpr int kPartWords = 8;            // words of a piece: its smallest keys, the bound of the others
-constexpr int kSvList = 64;             // listed new cells per survivor
+constexpr int kSvList = 64;              // places for listed new cells per survivor
 constexpr int kRankBits = 4;             // an entry's rank in its row
 constexpr unsigned kRankMask = 15u;
 constexpr int kBar2 = 32;                // words of the second and third barrier counter and of
@@ -92,9 +92,8 @@ struct MergeParams {
     int *size_g;                   // [n] cluster sizes
     int chunk;                     // rows per chunk of the apply pass (set at launch)
     RecA *recA;                    // [2][G] published entries and refill requests
-    int *svcnt;                    // [2][kSurv] new cells of a survivor below the limit,
-    unsigned long long *svovf;     // the least of them that is not listed [2][kSurv],
-    unsigned long long *svlist;    // and the listed ones [2][kSurv][kSvList], by round parity
+    unsigned long long *svlist;    // [2][kSurv][kSvList] survivors' new cells below the limit, by
+    unsigned long long *svovf;     // round parity, and [2][kSurv] the least that is not listed
     unsigned long long *parts;     // [2][kMaxReq][kPieces][kPartWords] refill lists (top-K of a row's pieces)
     unsigned int *bar;             // grid barrier counters, words 0 and kBar2 (zero at launch)
     int *status;                   // [4] status word [0]; barrier that gave up [1]
@@ -138,7 +137,7 @@ __host__ __device__ inline WorkspaceLayout workspace_layout(long long n, int G)
     size_t off = 0;
     L.size = off;   off = up(off + sizeof(int) * (size_t)n);
     L.recA = off;   off = up(off + sizeof(RecA) * 2 * (size_t)G);
-    L.sv = off;     off = up(off + 2 * kSurv * (size_t)(16 + 8 * kSvList));
+    L.sv = off;     off = up(off + 2 * kSurv * (size_t)(8 * (kSvList + 1)));
     L.parts = off;  off = up(off + 8 * kPartWords * (size_t)kMaxReq * kPieces * 2);
     L.zero = off;
     L.bar = off;    off = up(off + 256);
@@ -155,7 +154,6 @@ __host__ __device__ inline void bind_workspace(MergeParams &p, char *ws, const W
     p.recA = reinterpret_cast<RecA *>(ws + L.recA);
     p.svlist = reinterpret_cast<unsigned long long *>(ws + L.sv);
     p.svovf = p.svlist + 2 * kSurv * kSvList;
-    p.svcnt = reinterpret_cast<int *>(p.svovf + 2 * kSurv);
     p.parts = reinterpret_cast<unsigned long long *>(ws + L.parts);
     p.bar = reinterpret_cast<unsigned int *>(ws + L.bar);
     p.status = reinterpret_cast<int *>(ws + L.status);

@@ -26,8 +26,8 @@
 namespace {
 
 // Largest n this entry point accepts and the scratch that serves it
-// (workspace_layout): cluster sizes 4n B; per CTA two records of 144 B; 64 KB of
-// refill lists; 34 KB of survivors' lists; barrier, status and counter words.
+// (workspace_layout): cluster sizes 4n B; per CTA two records of 144 B; 128 KB of
+// refill lists; 33 KB of survivors' lists; barrier, status and counter words.
 // At n = 16384 on a 256-CTA grid that is about 305 KB; the array holds 2 MB,
 // and every call checks its layout against that size.
 constexpr long long kNoAllocMaxN = LW_NOALLOC_MAX_N;
