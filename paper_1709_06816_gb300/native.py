@@ -191,24 +191,19 @@ def lw_get_stats(ctx: int) -> dict:
     s = lib.lw_get_stats(ctx, a, 33)
     if s != 0:
         raise LwError(s, "lw_get_stats")
+    # (walk_steps: entries that the rounds selected their members from)
     out = {"rounds": a[0], "idle_rounds": a[1], "updated": a[2], "grid": a[3],
            "refills": a[4], "refill_cells": a[5], "installs": a[6], "walk_steps": a[7],
            "rescans": a[14], "rescan_cells": a[15]}
     if any(a[8:14]):
+        # the counters of lw_get_stats [8..13] and [16..25] by what they hold
+        # ([12], [24] and those from [26] on are 0)
         G = max(1, a[3])
-        names = ("barrier", "walk", "pass1", "refill", "certify", "pass2")
-        out["phase_ms"] = {nm: a[8 + q] / G / 1e6 for q, nm in enumerate(names)}
-        sub = ("records", "walk_installs", "chain", "minima", "certify", "bookkeeping", "pass2",
-               "rescans", "scan_log", "scan_matrix", "walk_only")
-        out["subphase_ms"] = {nm: a[16 + q] / G / 1e6 for q, nm in enumerate(sub)}
-        if a[28] > 0:
-            out["barrier_detail"] = {
-                "barriers": a[28],
-                "last_arriver_wait_us": a[27] / a[28] / 1e3,
-                "b_last_serving_refill": a[30] / max(1, a[29]),
-                "a_last_serving_refill": a[31] / max(1, a[28] - a[29]),
-                "last_is_cta0": a[32] / a[28],
-            }
+        names = {8: "barrier", 9: "merges", 10: "to_new_cells", 11: "gather_wait", 13: "apply"}
+        out["phase_ms"] = {nm: a[q] / G / 1e6 for q, nm in names.items()}
+        sub = {16: "lists", 17: "selection", 18: "member_cells", 19: "merges", 20: "new_cells",
+               21: "records", 22: "caches", 23: "rescans", 25: "refill_scans"}
+        out["subphase_ms"] = {nm: a[q] / G / 1e6 for q, nm in sub.items()}
     return out
 
 
