@@ -3,7 +3,9 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 struct lw_ctx;
 
@@ -40,6 +42,110 @@ constexpr uint64_t kNoKey = ~0ull;
 constexpr unsigned kColMask = 0x3fffffffu;
 constexpr unsigned kRowStop = 0x80000000u;   // the row's cache ends here (cells beyond unknown)
 constexpr unsigned kHardStop = 0x40000000u;  // the CTA published no entries beyond this one
+
+// ---- the update formula and the bounds of the cells it makes.  Host code too, for
+// the test of the bounds: compiled there without contraction of products and sums.
+#ifdef __CUDA_ARCH__
+#define LW_ON(device, host) device
+#else
+#define LW_ON(device, host) host
+#endif
+__host__ __device__ __forceinline__ float mul_rn(float a, float b) { return LW_ON(__fmul_rn(a, b), a * b); }
+__host__ __device__ __forceinline__ float add_rn(float a, float b) { return LW_ON(__fadd_rn(a, b), a + b); }
+__host__ __device__ __forceinline__ float sub_rn(float a, float b) { return LW_ON(__fsub_rn(a, b), a - b); }
+__host__ __device__ __forceinline__ float div_rn(float a, float b) { return LW_ON(__fdiv_rn(a, b), a / b); }
+__host__ __device__ __forceinline__ float div_fast(float a, float b) { return LW_ON(__fdividef(a, b), a / b); }
+__host__ __device__ __forceinline__ float ll_rn(long long a) { return LW_ON(__ll2float_rn(a), (float)a); }
+__host__ __device__ __forceinline__ unsigned bits_of(float a)
+{
+    unsigned u;
+    memcpy(&u, &a, sizeof u);
+    return LW_ON(__float_as_uint(a), u);
+}
+__host__ __device__ __forceinline__ float value_of(unsigned u)
+{
+    float a;
+    memcpy(&a, &u, sizeof a);
+    return LW_ON(__uint_as_float(u), a);
+}
+#undef LW_ON
+
+// The update of Section 4 step 3 from coefficients: the four terms (bh is the
+// third) added in printed order, every operation rounded once.
+__host__ __device__ __forceinline__ float lw_sum(float ai, float aj, float bh, float ga, float dki, float dkj)
+{
+    float s = mul_rn(ai, dki);
+    s = add_rn(s, mul_rn(aj, dkj));
+    s = add_rn(s, bh);
+    return add_rn(s, mul_rn(ga, fabsf(sub_rn(dki, dkj))));
+}
+
+// Ward's cell (coefficients depend on the third cluster's size fk).
+__host__ __device__ __forceinline__ float ward_cell(float fi, float fj, float fs, float fk, float h, float a, float b)
+{
+    const float T = add_rn(fs, fk);  // (integers below 2^24: exact)
+    const float x = div_rn(add_rn(fi, fk), T), y = div_rn(add_rn(fj, fk), T);
+    const float z = -div_rn(fk, T);
+    return lw_sum(x, y, mul_rn(z, h), 0.0f, a, b);
+}
+
+// Table 1 coefficients of a merge of sizes ni, nj at height h: a_i, a_j, b
+// times h, g (LK 3, Ward: per cell, see ward_cell).  Centroid: exact integers,
+// each converted to float once, one division.
+template <int LK>
+__host__ __device__ __forceinline__ float4 merge_coefs(int ni, int nj, float h)
+{
+    float4 co = make_float4(0.5f, 0.5f, mul_rn(0.0f, h), 0.0f);
+    if (LK == 0)
+        co.w = -0.5f;
+    if (LK == 1)
+        co.w = 0.5f;
+    if (LK == 2 || LK == 5) {
+        const float fs = (float)(ni + nj);
+        co.x = div_rn((float)ni, fs);
+        co.y = div_rn((float)nj, fs);
+    }
+    if (LK == 5)
+        co.z = mul_rn(-div_rn(ll_rn((long long)ni * nj), ll_rn((long long)(ni + nj) * (ni + nj))), h);
+    return co;
+}
+
+// A lower bound (value bits) of the cells between a merged cluster and others,
+// from the bounds la, lb of its two parts' cells (both above the height h): the
+// update formula is monotone in both distances, so it is evaluated at the
+// bounds, less a margin for its roundings.  Per linkage, rounding errors in
+// units of 2^-24: complete: s + |d|/2 >= max(a, b) up to 3 relative, and >=
+// min(a, b) without error (rounding is monotone, and so for weighted); single:
+// the terms reach the larger distance, 2.5 of the largest value in the matrix;
+// weighted: 1 relative; average, centroid: 4 relative; Ward: the weighted mean
+// of a and b is a bound for every size of the third cluster (the formula rises
+// from it with that size while a, b >= h), at most 12 relative.  The margins
+// taken (2e-6 = 33, 8e-6 = 134 units) leave room for the bound's own roundings.
+// Values too small for a relative margin, or not finite, give bound 0: the
+// round then ends where it would need it.
+template <int LK>
+__host__ __device__ __forceinline__ unsigned merged_bound(int lab, int lbb, float fi, float fs, float h, unsigned dmax)
+{
+    const float la = value_of((unsigned)lab), lb = value_of((unsigned)lbb);
+    float r;
+    if (LK == 0)
+        r = fminf(la, lb) - 2.0e-6f * value_of(dmax);
+    else if (LK == 1)
+        r = fmaxf(fminf(la, lb), fmaxf(la, lb) * (1.0f - 2.0e-6f));
+    else if (LK == 4)
+        r = fmaxf(fminf(la, lb), (0.5f * la + 0.5f * lb) * (1.0f - 2.0e-6f));
+    else {
+        const float w = div_fast(fi, fs);
+        r = w * la + (1.0f - w) * lb;
+        if (LK == 5)
+            r = r - w * (1.0f - w) * h;
+        r = r * (1.0f - 8.0e-6f);
+    }
+    if ((lab & lbb) == -1)
+        return 0xffffffffu;  // no such cells
+    // (a NaN fails both comparisons)
+    return r > 1.0e-30f && r < 3.0e38f ? bits_of(r) : 0u;
+}
 
 // Status words written by the kernel (values match lw_status).
 enum : int { kOk = 0, kErrInput = 2, kErrInternal = 4, kErrTimeout = 5, kErrBounds = 6 };

@@ -295,16 +295,6 @@ __device__ __forceinline__ void sort_list(u64 (&L)[K])
     cswap(L[1], L[2]);
 }
 
-// The update of Section 4 step 3 from coefficients: the four terms (bh is the
-// third) added in printed order, every operation rounded once.
-__device__ __forceinline__ float lw_sum(float ai, float aj, float bh, float ga, float dki, float dkj)
-{
-    float s = __fmul_rn(ai, dki);
-    s = __fadd_rn(s, __fmul_rn(aj, dkj));
-    s = __fadd_rn(s, bh);
-    return __fadd_rn(s, __fmul_rn(ga, fabsf(__fsub_rn(dki, dkj))));
-}
-
 // A round's members and merges (static shared memory).
 struct Team {
     // the members (slots in ascending order), size and bound of the cells
@@ -967,36 +957,6 @@ __device__ __noinline__ void warp_row_refresh(const MergeParams &p, long long r,
     live_cells += cnt;
     warp_topk_next(L, out, next);
 }
-// Ward's cell (coefficients depend on the third cluster's size fk).
-__device__ __forceinline__ float ward_cell(float fi, float fj, float fs, float fk, float h, float a, float b)
-{
-    const float T = __fadd_rn(fs, fk);  // (integers below 2^24: exact)
-    const float x = __fdiv_rn(__fadd_rn(fi, fk), T), y = __fdiv_rn(__fadd_rn(fj, fk), T);
-    const float z = -__fdiv_rn(fk, T);
-    return lw_sum(x, y, __fmul_rn(z, h), 0.0f, a, b);
-}
-
-// Table 1 coefficients of a merge of sizes ni, nj at height h: a_i, a_j, b
-// times h, g (LK 3, Ward: per cell, see ward_cell).  Centroid: exact integers,
-// each converted to float once, one division.
-template <int LK>
-__device__ __forceinline__ float4 merge_coefs(int ni, int nj, float h)
-{
-    float4 co = make_float4(0.5f, 0.5f, __fmul_rn(0.0f, h), 0.0f);
-    if (LK == 0)
-        co.w = -0.5f;
-    if (LK == 1)
-        co.w = 0.5f;
-    if (LK == 2 || LK == 5) {
-        const float fs = (float)(ni + nj);
-        co.x = __fdiv_rn((float)ni, fs);
-        co.y = __fdiv_rn((float)nj, fs);
-    }
-    if (LK == 5)
-        co.z = __fmul_rn(-__fdiv_rn(__ll2float_rn((long long)ni * nj), __ll2float_rn((long long)(ni + nj) * (ni + nj))),
-                         h);
-    return co;
-}
 
 // Merge q for a row of size nk: the new cell from its two cells.
 __device__ __forceinline__ float merge_cell(const Team &tm, int linkage, int q, float a, float b, float nk)
@@ -1007,43 +967,6 @@ __device__ __forceinline__ float merge_cell(const Team &tm, int linkage, int q, 
     }
     const float4 co = tm.co[q];
     return lw_sum(co.x, co.y, co.z, co.w, a, b);
-}
-
-// A lower bound (value bits) of the cells between a merged cluster and others,
-// from the bounds la, lb of its two parts' cells (both above the height h): the
-// update formula is monotone in both distances, so it is evaluated at the
-// bounds, less a margin for its roundings.  Per linkage, rounding errors in
-// units of 2^-24: complete: s + |d|/2 >= max(a, b) up to 3 relative, and >=
-// min(a, b) without error (rounding is monotone, and so for weighted); single:
-// the terms reach the larger distance, 2.5 of the largest value in the matrix;
-// weighted: 1 relative; average, centroid: 4 relative; Ward: the weighted mean
-// of a and b is a bound for every size of the third cluster (the formula rises
-// from it with that size while a, b >= h), at most 12 relative.  The margins
-// taken (2e-6 = 33, 8e-6 = 134 units) leave room for the bound's own roundings.
-// Values too small for a relative margin, or not finite, give bound 0: the
-// round then ends where it would need it.
-template <int LK>
-__device__ __forceinline__ unsigned merged_bound(int lab, int lbb, float fi, float fs, float h, unsigned dmax)
-{
-    const float la = __int_as_float(lab), lb = __int_as_float(lbb);
-    float r;
-    if (LK == 0)
-        r = fminf(la, lb) - 2.0e-6f * __uint_as_float(dmax);
-    else if (LK == 1)
-        r = fmaxf(fminf(la, lb), fmaxf(la, lb) * (1.0f - 2.0e-6f));
-    else if (LK == 4)
-        r = fmaxf(fminf(la, lb), (0.5f * la + 0.5f * lb) * (1.0f - 2.0e-6f));
-    else {
-        const float w = __fdividef(fi, fs);
-        r = w * la + (1.0f - w) * lb;
-        if (LK == 5)
-            r = r - w * (1.0f - w) * h;
-        r = r * (1.0f - 8.0e-6f);
-    }
-    if ((lab & lbb) == -1)
-        return 0xffffffffu;  // no such cells
-    // (a NaN fails both comparisons)
-    return r > 1.0e-30f && r < 3.0e38f ? __float_as_uint(r) : 0u;
 }
 
 // The step-by-step iteration among a round's members, as far as no other cell
