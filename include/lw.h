@@ -289,7 +289,8 @@ void lw_batch_destroy(lw_batch *batch);
  * lw_set_batch_classes -- how one-CTA batch jobs are grouped: class q takes
  * the jobs with n_hi[q-1] < n <= n_hi[q] (n_hi ascending, count <= 16) and
  * runs them with CTAs of cta_threads[q] threads (128, 256 or 512: smaller
- * CTAs let several jobs share an SM).  Each class is its own persistent
+ * CTAs let several jobs share an SM; a limit above what such a CTA's shared
+ * memory holds counts as that much).  Each class is its own persistent
  * launch; the classes run side by side as branches of the batch's CUDA
  * graph.  count = 0 restores the default (one class of 512-thread CTAs).
  * The autotuner of the Python package measures and sets this table.

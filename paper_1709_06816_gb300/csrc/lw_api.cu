@@ -707,6 +707,15 @@ lw_status lw_batch_create(lw_ctx *ctx, const lw_job *jobs, int32_t njobs, lw_bat
         lw_batch::Class k;
         k.n_hi = c.first < cap ? c.first : cap;
         k.nt = c.second;
+        // jobs that no CTA of this size holds go to the next class or over the
+        // device (asked for the largest job the class would get: the search for
+        // the limit takes a dozen occupancy queries)
+        long long top = 2;
+        for (int q = 0; q < njobs; ++q)
+            if (jobs[q].n <= k.n_hi && jobs[q].n > top)
+                top = jobs[q].n;
+        if (lw::batch_ctas_per_sm(top, k.nt) < 1)
+            k.n_hi = batch_auto_split(k.nt);
         if (b->classes.empty() || k.n_hi > b->classes.back().n_hi)
             b->classes.push_back(k);
     }
@@ -774,6 +783,7 @@ lw_status lw_batch_create(lw_ctx *ctx, const lw_job *jobs, int32_t njobs, lw_bat
             table[q].merges = J.merges_out;
             table[q].heights = J.heights_out;
         }
+        // (this also sets the kernel's shared-memory limit for the launch below)
         const int per_sm = lw::batch_ctas_per_sm(c.n_max < 2 ? 2 : c.n_max, c.nt);
         if (per_sm < 1) {
             set_err(ctx, "batch jobs of n=%lld do not fit one CTA of %d threads", c.n_max, c.nt);
