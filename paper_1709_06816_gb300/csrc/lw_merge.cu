@@ -467,9 +467,8 @@ __device__ void exchange_requests(int cnt, const int (&rq)[kReqPerCta], int b, S
     __syncthreads();
 }
 
-// KK smallest keys over every thread's sorted list; result in sh.tko (all threads).
 // Barrier of the threads that work together: the whole CTA (TB == NT), or
-// its last TB threads (named barrier 1) while warp 0 does something else.
+// its last TB threads (named barrier 1).
 template <int NT, int TB>
 __device__ __forceinline__ void team_sync()
 {
@@ -1983,88 +1982,88 @@ __device__ __forceinline__ void publish(const MergeParams &p, Shared<NT, ONE> &s
             STCG(&rec->col[tid], col);
         }
     } else {
-    {
-        const u64 x = warp_u64_min(head);
-        if (lane == 0)
-            sh.wmin[warp][0] = x;
-    }
-    if (tid == 0)
-        sh.ncand = 0;
-    __syncthreads();
-    const u64 gmin = warp_u64_min(lane < W ? sh.wmin[lane][0] : kNoKey);
-    auto count = [&](u64 x) -> int { return __syncthreads_count(head <= x && head != kNoKey); };
-    const u64 pivot = find_pivot(count, gmin, kNoKey, sh.ppivot, kPub, 3 * kPub);
-    int have = 0;
-    if (head <= pivot && head != kNoKey) {
-#pragma unroll 1
-        for (int l = tid; l < R; l += NT) {
-            const int c = ccnt[l];
-#pragma unroll 1
-            for (int q = 0; q <= c; ++q) {
-                u64 e;
-                entry_at(l, q, c, e);
-                have += e <= pivot && e != kNoKey;
-            }
+        {
+            const u64 x = warp_u64_min(head);
+            if (lane == 0)
+                sh.wmin[warp][0] = x;
         }
-    }
-    int at = have;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_up_sync(kFull, at, off);
-        if (lane >= off)
-            at += o;
-    }
-    {
-        int base = 0;
-        if (lane == 31 && at > 0)
-            base = atomicAdd(&sh.ncand, at);
-        base = __shfl_sync(kFull, base, 31);
-        at = base + at - have;
-    }
-    if (have > 0) {
+        if (tid == 0)
+            sh.ncand = 0;
+        __syncthreads();
+        const u64 gmin = warp_u64_min(lane < W ? sh.wmin[lane][0] : kNoKey);
+        auto count = [&](u64 x) -> int { return __syncthreads_count(head <= x && head != kNoKey); };
+        const u64 pivot = find_pivot(count, gmin, kNoKey, sh.ppivot, kPub, 3 * kPub);
+        int have = 0;
+        if (head <= pivot && head != kNoKey) {
 #pragma unroll 1
-        for (int l = tid; l < R; l += NT) {
-            const int c = ccnt[l];
+            for (int l = tid; l < R; l += NT) {
+                const int c = ccnt[l];
 #pragma unroll 1
-            for (int q = 0; q <= c; ++q) {
-                u64 e;
-                const u64 x = entry_at(l, q, c, e);
-                if (e == kNoKey || e > pivot)
-                    break;
-                if (at < kCand) {
-                    sh.ckey[at] = e;
-                    sh.ccol[at] = q < c ? (unsigned)x : kRowStop | (unsigned)x;
+                for (int q = 0; q <= c; ++q) {
+                    u64 e;
+                    entry_at(l, q, c, e);
+                    have += e <= pivot && e != kNoKey;
                 }
-                ++at;
             }
         }
-    }
-    __syncthreads();
-    if (tid == 0)
-        sh.ppivot = pivot;
-    // (at most 3 * kPub threads of 4 rows and K + 1 entries each: they fit)
-    static_assert(3 * kPub * 4 * (K + 1) <= kCand, "published entries fit");
-    const int N = sh.ncand < kCand ? sh.ncand : kCand;
-#pragma unroll 1
-    for (int c0 = (tid >> 5) * 8; c0 < N; c0 += NT / 4) {
-        const int c = c0 + (lane >> 2);
-        const u64 key = c < N ? sh.ckey[c] : kNoKey;
-        int rank = 0;
-#pragma unroll 1
-        for (int f = lane & 3; f < N; f += 4)
-            rank += sh.ckey[f] < key;
-        rank += __shfl_xor_sync(kFull, rank, 1);
-        rank += __shfl_xor_sync(kFull, rank, 2);
-        if (c < N && (lane & 3) == 0 && rank < kPub) {
-            STCG(&rec->key[rank], key);
-            // (more entries may follow the last: none is published)
-            STCG(&rec->col[rank], sh.ccol[c] | (rank == kPub - 1 ? kHardStop : 0u));
+        int at = have;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(kFull, at, off);
+            if (lane >= off)
+                at += o;
         }
-    }
-    if (tid >= N && tid < kPub) {
-        STCG(&rec->key[tid], kNoKey);
-        STCG(&rec->col[tid], 0u);
-    }
+        {
+            int base = 0;
+            if (lane == 31 && at > 0)
+                base = atomicAdd(&sh.ncand, at);
+            base = __shfl_sync(kFull, base, 31);
+            at = base + at - have;
+        }
+        if (have > 0) {
+#pragma unroll 1
+            for (int l = tid; l < R; l += NT) {
+                const int c = ccnt[l];
+#pragma unroll 1
+                for (int q = 0; q <= c; ++q) {
+                    u64 e;
+                    const u64 x = entry_at(l, q, c, e);
+                    if (e == kNoKey || e > pivot)
+                        break;
+                    if (at < kCand) {
+                        sh.ckey[at] = e;
+                        sh.ccol[at] = q < c ? (unsigned)x : kRowStop | (unsigned)x;
+                    }
+                    ++at;
+                }
+            }
+        }
+        __syncthreads();
+        if (tid == 0)
+            sh.ppivot = pivot;
+        // (at most 3 * kPub threads of 4 rows and K + 1 entries each: they fit)
+        static_assert(3 * kPub * 4 * (K + 1) <= kCand, "published entries fit");
+        const int N = sh.ncand < kCand ? sh.ncand : kCand;
+#pragma unroll 1
+        for (int c0 = (tid >> 5) * 8; c0 < N; c0 += NT / 4) {
+            const int c = c0 + (lane >> 2);
+            const u64 key = c < N ? sh.ckey[c] : kNoKey;
+            int rank = 0;
+#pragma unroll 1
+            for (int f = lane & 3; f < N; f += 4)
+                rank += sh.ckey[f] < key;
+            rank += __shfl_xor_sync(kFull, rank, 1);
+            rank += __shfl_xor_sync(kFull, rank, 2);
+            if (c < N && (lane & 3) == 0 && rank < kPub) {
+                STCG(&rec->key[rank], key);
+                // (more entries may follow the last: none is published)
+                STCG(&rec->col[rank], sh.ccol[c] | (rank == kPub - 1 ? kHardStop : 0u));
+            }
+        }
+        if (tid >= N && tid < kPub) {
+            STCG(&rec->key[tid], kNoKey);
+            STCG(&rec->col[tid], 0u);
+        }
     }
     if (tid == 0) {
         const int par = (rr - 1) & 1;
@@ -2786,21 +2785,21 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         sh.tm.thA = A;
                         sh.tm.thC = C;
                         const unsigned tv = (unsigned)(A >> 32);
-                    sh.tm.thv = tv;
-                    if (!ONE) {
-                        // survivors' cells below a limit above the bound are listed;
-                        // its distance follows the lists' lengths
-                        const unsigned v0 = E > 0 ? (unsigned)(sh.ekey[0] >> 32) : tv;
-                        unsigned w = sh.width;
-                        if (w == 0u)
-                            w = tv > v0 && tv < 0x7f800000u ? 8u * min(tv - v0, 0x100000u) : 0u;
-                        else if (nps > 0 && sh.svsum < 4 * nps)
-                            w += w / 2;
-                        else if (nps > 0 && sh.svsum > 6 * nps)
-                            w -= w / 4;
-                        sh.width = w = min(max(w, 64u), 0x4000000u);
-                        sh.limit = tv < 0x7f000000u ? min(tv + w, 0x7f800000u) : 0xffffffffu;
-                    }
+                        sh.tm.thv = tv;
+                        if (!ONE) {
+                            // survivors' cells below a limit above the bound are listed;
+                            // its distance follows the lists' lengths
+                            const unsigned v0 = E > 0 ? (unsigned)(sh.ekey[0] >> 32) : tv;
+                            unsigned w = sh.width;
+                            if (w == 0u)
+                                w = tv > v0 && tv < 0x7f800000u ? 8u * min(tv - v0, 0x100000u) : 0u;
+                            else if (nps > 0 && sh.svsum < 4 * nps)
+                                w += w / 2;
+                            else if (nps > 0 && sh.svsum > 6 * nps)
+                                w -= w / 4;
+                            sh.width = w = min(max(w, 64u), 0x4000000u);
+                            sh.limit = tv < 0x7f000000u ? min(tv + w, 0x7f800000u) : 0xffffffffu;
+                        }
                         ty.walk += stop;
                     }
                 }
@@ -2924,8 +2923,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                         const int e = e0 + u * TA;
                         const int a = e & (kTeam - 1), c = (a + (e / kTeam) + 1) & (kTeam - 1);
                         v[u] = 0.0f;
-                        if (e < ALL && a < m && c < m)
-                            {
+                        if (e < ALL && a < m && c < m) {
                             // row-log layout: the cell is current in the row of M
                             // whose slot was stamped later (both rows hold the input
                             // value while neither has merged)
@@ -3022,38 +3020,38 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                                  : "memory");
                 lap(ty.ph[3]);
             } else if constexpr (!ONE) {
-            constexpr int TB = NT - TA;
-            // ---- the refills asked for in the previous round, served now by
-            // team B (row s of the list by CTA G - 1 - s mod G: rows are
-            // owned in blocks of 32 from CTA 0 up, so the last CTAs own a block
-            // fewer and take the scans first): the K smallest keys of the row
-            // over live columns.  Other CTAs may already be writing this
-            // round's merges: the columns those touch are dropped when the
-            // owner installs the list and replays the round.
-            // A row is cut in pieces when there are CTAs for them: a whole row
-            // scanned by one CTA outlasts the steps beside it, and every other
-            // CTA would wait for it.
-            const int nexec = sh.nexec;
-            const int np = scan_pieces(G, nexec, early);
+                constexpr int TB = NT - TA;
+                // ---- the refills asked for in the previous round, served now by
+                // team B (row s of the list by CTA G - 1 - s mod G: rows are
+                // owned in blocks of 32 from CTA 0 up, so the last CTAs own a block
+                // fewer and take the scans first): the K smallest keys of the row
+                // over live columns.  Other CTAs may already be writing this
+                // round's merges: the columns those touch are dropped when the
+                // owner installs the list and replays the round.
+                // A row is cut in pieces when there are CTAs for them: a whole row
+                // scanned by one CTA outlasts the steps beside it, and every other
+                // CTA would wait for it.
+                const int nexec = sh.nexec;
+                const int np = scan_pieces(G, nexec, early);
 #pragma unroll 1
-            for (int w = G - 1 - b; w < nexec * np; w += G) {
-                const int s2 = w / np, piece = w % np;
-                const long long rr = sh.exec_row[s2];
-                if (rr < 0 || rr >= n - 1)
-                    continue;  // the same for every thread of the team
-                if (full)
-                    block_row_topk_cols<NT, ONE, TB>(p, rr, piece, np, (int)t, bitmap, sh, st_fill_cells,
-                                                     p.timing ? ty.xscan : nullptr);
-                else
-                    block_row_topk<NT, ONE, TB>(p, rr, piece, np, bitmap, sh, st_fill_cells);
-                if (tid - TA < K + 1)
-                    STCG(p.parts + (((size_t)par * kMaxReq + s2) * kPieces + piece) * kPartWords + (tid - TA),
-                         tid - TA < K ? sh.tko[tid - TA] : sh.tnext);
-            }
-            if (tid == TA)
-                ty.fills += nexec;
-            // (team A does not wait: it begins with the new cells)
-            asm volatile("barrier.cta.sync.aligned 4, %0;" ::"n"(NT) : "memory");
+                for (int w = G - 1 - b; w < nexec * np; w += G) {
+                    const int s2 = w / np, piece = w % np;
+                    const long long rr = sh.exec_row[s2];
+                    if (rr < 0 || rr >= n - 1)
+                        continue;  // the same for every thread of the team
+                    if (full)
+                        block_row_topk_cols<NT, ONE, TB>(p, rr, piece, np, (int)t, bitmap, sh, st_fill_cells,
+                                                         p.timing ? ty.xscan : nullptr);
+                    else
+                        block_row_topk<NT, ONE, TB>(p, rr, piece, np, bitmap, sh, st_fill_cells);
+                    if (tid - TA < K + 1)
+                        STCG(p.parts + (((size_t)par * kMaxReq + s2) * kPieces + piece) * kPartWords + (tid - TA),
+                             tid - TA < K ? sh.tko[tid - TA] : sh.tnext);
+                }
+                if (tid == TA)
+                    ty.fills += nexec;
+                // (team A does not wait: it begins with the new cells)
+                asm volatile("barrier.cta.sync.aligned 4, %0;" ::"n"(NT) : "memory");
             }
         }
         if (sh.flag != 0)
