@@ -3592,23 +3592,28 @@ size_t smem_for(long long n, int G, int chunk)
 }  // namespace
 
 // CTAs for n objects when the caller names no number.  One up to 416 objects: a
-// block of 32 rows per CTA and grid barriers are slower there (complete, ms,
-// one CTA / grid: n = 300 0.61 / 0.69, n = 400 0.86 / 0.87, n = 512 1.14 / 0.91,
-// n = 1000 3.13 / 1.39, n = 2048 12.2 / 2.4).  Centroid linkage makes few merges
-// per round and none side by side, so the barriers weigh more: 15.2 / 16.7 at
-// n = 1000, 23.3 / 22.3 at 1300, 49.8 / 36.2 at 2048.  Above, one CTA per block
-// up to 64 of them, then one per two blocks, at most one per SM (complete: n = 3500
-// 64 CTAs 4.11, 96 3.99; n = 4096 64 CTAs 4.81, 128 4.53; average: n = 5003 80 CTAs
-// 5.67, 152 5.55; n = 6500 96 7.66, 128 7.18): the last few percent would take
+// block of 32 rows per CTA and grid barriers are no faster there (complete, ms,
+// one CTA / grid: n = 300 0.62 / 0.70, n = 400 0.83 / 0.77, n = 512 1.07 / 1.01,
+// n = 1000 3.04 / 1.44, n = 2048 12.0 / 2.5).  Centroid linkage makes few merges
+// per round, so a grid's barriers weigh more: n = 400 2.9 / 3.8, n = 600 5.8 / 5.4,
+// n = 1000 10.3 / 8.1, n = 1152 13.6 / 9.5, n = 2048 32.1 / 15.6; up to 1152 objects
+// it stays on one SM, where a grid would take 19 to 36 of them for 7 to 30 % of the
+// time.  Above, one CTA per block up to 64 of them, then one per two blocks
+// (rounded up: with n = 5003, 157 blocks, 78 CTAs leave three blocks to one of
+// them; complete 5.70, average 5.83, packed 5.61, on 79 CTAs 5.64, 5.71, 5.51;
+// n = 7001, 109 / 110 CTAs, 7.82 / 7.64), at most one per SM (complete: n = 3500
+// 64 CTAs 4.06, 96 3.97; n = 4096 64 CTAs 4.73, 128 4.47; average: n = 5003 79 CTAs
+// 5.71, 152 5.63; n = 6500 102 7.21, 128 7.17): the last percent would take
 // twice the SMs.  Single linkage (the merges of a round are worked out one by one,
-// and every CTA repeats them) runs better on fewer CTAs with the same most blocks
-// per CTA (n = 16384: 128 31.9, 152 32.4; Ward 23.5 and 22.0).
+// and every CTA repeats them) is as fast on fewer CTAs with the same most blocks
+// per CTA and takes those (n = 16384, 128 / 152 CTAs: distances on a 1/1024 grid
+// 52.7 / 53.4, continuous 27.8 / 27.6; Ward 23.0 / 21.5).
 int default_grid(long long n, int linkage, int num_sms)
 {
     const long long nb = (n + kRowBlock - 1) / kRowBlock;
     if (n <= (linkage == LW_CENTROID ? 1152 : 416))
         return 1;
-    long long G = nb <= 64 ? nb : nb / 2 > 64 ? nb / 2 : 64;
+    long long G = nb <= 64 ? nb : nb > 128 ? (nb + 1) / 2 : 64;
     if (G > num_sms)
         G = num_sms;
     if (linkage == LW_SINGLE) {
