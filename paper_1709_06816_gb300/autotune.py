@@ -1,9 +1,9 @@
 """Autotuner of the batch path: which CTA size serves which job sizes.
 
 A one-CTA batch job runs on a CTA of 128, 256 or 512 threads.  Smaller CTAs
-let several jobs share an SM (registers allow 4, 2 or 1 per SM) but give each
-job fewer threads, and the shared memory a job needs grows with n, so the
-best choice depends on n and on the device.  ``tune_batch_classes`` measures,
+let several jobs share an SM (registers allow 4, 2 or 1 per SM; shared memory
+3, 2 or 1 at n = 64 and one of any size from n = 1024 on) but give each job
+fewer threads, so the best choice depends on n and on the device.  ``tune_batch_classes`` measures,
 for each size bucket, the merges per second of a full-device batch of
 synthetic jobs at every CTA size that fits, keeps the fastest, merges
 neighbouring buckets with the same choice into classes and caches the table
@@ -37,14 +37,14 @@ def _cache_path(torch, device: int, shipped: bool = False) -> str:
                         f"batch_{name}_{props.multi_processor_count}.json")
 
 
-def _measure(ctx, torch, device, n_lo, n_hi, nt, jobs_per_cta=2, seed=11):
-    """Merges/s of one full-device batch of jobs with n in (n_lo, n_hi] on CTAs of nt threads."""
+def _measure(ctx, torch, device, n_lo, n_hi, nt, jobs_per_sm=8, seed=11):
+    """Merges/s of one full-device batch of jobs with n in (n_lo, n_hi] on CTAs of nt threads
+    (the same jobs for every CTA size; one CTA of any size holds n = 2048)."""
     import synth
 
     ctx.set_batch_classes([(n_hi, nt)])
     sms = torch.cuda.get_device_properties(device).multi_processor_count
-    per_sm = {128: 4, 256: 2, 512: 1}[nt]
-    count = sms * per_sm * jobs_per_cta
+    count = sms * jobs_per_sm
     rng = np.random.default_rng(seed)
     bank = []
     for q in range(8):
@@ -57,7 +57,7 @@ def _measure(ctx, torch, device, n_lo, n_hi, nt, jobs_per_cta=2, seed=11):
     try:
         plan = native.lw_batch_create(ctx.handle, table)
     except native.LwError:
-        return None  # this CTA size cannot hold jobs of this size
+        return None  # no room for the plan
     try:
         best = None
         for rep in range(3):
@@ -112,7 +112,8 @@ def tune_batch_classes(device: int = 0, force: bool = False, verbose: bool = Fal
             classes[-1] = (hi, nt)
         else:
             classes.append((hi, nt))
-    # jobs above the last bucket keep the one-CTA default (512 threads)
+    # jobs above the last bucket keep the one-CTA default (512 threads), as far as
+    # one CTA holds them
     if classes[-1][1] != 512:
         classes.append((4096, 512))
     else:
