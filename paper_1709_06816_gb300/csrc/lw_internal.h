@@ -28,10 +28,28 @@ constexpr unsigned kRankMask = 15u;
 constexpr int kBar2 = 32;                // words of the second and third barrier counter and of
 constexpr int kBar3 = 48;                // the first conditional merge that must wait (two, by
 constexpr int kViol = 8;                 // round parity; kTeam less it, 0: none)
-constexpr int kRedoBelow = 16;           // a chain cut below this many merges, and below half its
-constexpr int kRedoGap = 4;              // length (and a bit), is walked step by step instead
-constexpr int kTieGain = 3;              // merges a round must gain to take them on condition
-constexpr long long kRefillEarlyN = 24576;  // up to this n a row asks for a refill at one key left, above it at none
+// A chain cut below kRedoBelow merges, and below half its length (and kRedoGap), is
+// walked step by step instead.  Never (0) / 16 / always (64), ms: n = 4000, points four
+// at a time, complete 59.5 / 17.5 / 17.5; n = 8192 average on a 1/1024 grid 13.9 / 11.9 /
+// 11.9; n = 16384 average 27.9 / 24.5 / 24.5; elsewhere within 1 %.
+constexpr int kRedoBelow = 16;
+constexpr int kRedoGap = 4;
+// Merges that a round of the chain must gain to take them on condition: kTieGain, and
+// one for every kTiePart that bounds prove (the look costs a barrier that also waits
+// for the scans beside it, more so in long rounds).  ms, n = 65536 conformer-like
+// complete / n = 4000 integers complete / n = 5000 on a 1/64 grid complete: any 3 merges
+// 146.2 / 26.5 / 6.22, any 8 141.7 / 36.5, any 14 141.1 / 39.4; 2 and half of the
+// proved ones 141.4 / 24.1 / 6.31, 2 and a quarter 142.1 / 24.0 / 6.22.
+constexpr int kTieGain = 2;
+constexpr int kTiePart = 4;
+// Up to this n a row asks for a refill at one key left; above it at none, and the
+// scans start before the selection, in more pieces, with prefetches.  Early saves rounds, late saves scans; ms, early / late: conformer-like, complete,
+// n = 8192 9.0 / 9.8, 16384 21.8 / 21.5, 20480 30.2 / 28.2, 24576 40.2 / 34.7, 28000
+// 49.8 / 40.9, 65536 234 / 146; on a 1/1024 grid, 20480 complete 30.2 / 31.5, average
+// 32.7 / 34.8, single 69.2 / 72.3, 24576 39.8 / 38.0, 41.5 / 41.9, 87.7 / 91.0, 28000
+// 48.8 / 44.0, 49.7 / 48.1, 104 / 108.  The line lies where the grids' gain ends;
+// continuous distances would have it at 16384.
+constexpr long long kRefillEarlyN = 24576;
 constexpr int kSurvivorRefillAt = 1;     // the same for a survivor row right after its merge
 constexpr int kMaxReq = 256;             // refill requests served per round
 constexpr int kReqPerCta = 8;            // refill requests one CTA may make per round
@@ -307,7 +325,9 @@ size_t merge_smem_bytes(long long n, int G, int nt);
 // Rows per chunk of the apply pass (its new cells are kept in shared memory).
 int merge_chunk_rows(long long n, int G, int nt);
 // CTA sizes the kernels are built for: 128, 256 or 512 threads (4, 2 or 1
-// CTAs per SM by registers).
+// CTAs per SM by registers; with their static shared memory of some 50 KB a
+// one-CTA job leaves room for 3, 2 and 1 at n = 64, for 2, 2 and 1 from 256 to 512
+// and for 1 of any size from 1024 on).
 // True if a grid of G CTAs of nt threads for n objects fits co-resident on
 // the current device.
 bool merge_config_ok(long long n, int G, int num_sms, int nt = kThreads);

@@ -46,11 +46,11 @@
 //      one warp takes the merges step by step.
 //   on condition  the bounds for outside cells may end a round that the cells
 //      themselves would not (equal values; inversions; values small against the
-//      largest, for single linkage).  When that costs kTieGain merges of a chain,
-//      or half as many steps as were proved (see simulate), the merges are taken
-//      on condition: the new cells are computed and kept back, every CTA looks
-//      whether one of its own comes before a merge of the round, and barrier 3
-//      tells which merges stand (settle).
+//      largest, for single linkage).  When that costs a quarter as many merges of a
+//      chain as were proved (kTieGain, kTiePart), or half as many steps (see
+//      simulate), the merges are taken on condition: the new cells are computed
+//      and kept back, every CTA looks whether one of its own comes before a merge
+//      of the round, and barrier 3 tells which merges stand (settle).
 //   apply  behind barrier 2 (no CTA still reads the members' old cells): the new
 //      cells D(k, survivor) for every live k, a warp per 32 rows and up to 4
 //      survivors, all loads of an item in flight at once; then logs, caches
@@ -1521,7 +1521,7 @@ __device__ __forceinline__ void chain_accept(Team &tm, bool allow)
     const unsigned bad = __ballot_sync(kFull, in && e >= min(un, own)) | made_first;
     const unsigned out = __ballot_sync(kFull, in && hb >= z) | bad;
     const int most = bad ? __ffs(bad) - 1 : L, sure = out ? __ffs(out) - 1 : L;
-    const bool tie = allow && most >= sure + kTieGain;
+    const bool tie = allow && most >= sure + kTieGain && kTiePart * (most - sure) >= sure;
     const int La = tie ? most : sure;
     if (lane < La) {
         tm.prog[lane] = lane;
