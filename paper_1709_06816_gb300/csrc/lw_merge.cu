@@ -3650,16 +3650,24 @@ size_t merge_smem_bytes(long long n, int G, int nt)
 
 namespace {
 
-int fit_per_sm(const void *fn, int nt, int G, size_t smem)
+// Lets a kernel's launches have all the dynamic shared memory that a CTA can have;
+// false if smem bytes are more than that.  Always the same value: the attribute
+// belongs to the function, and another thread may be between setting it for a
+// smaller job and launching that.
+bool allow_smem(const void *fn, int nt, int G, size_t smem)
 {
     int dev = 0, limit = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-        return 0;
-    if (smem + static_smem(nt, G) > (size_t)limit)
-        return 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+        return false;
+    const long long most = (long long)limit - (long long)static_smem(nt, G);
+    return (long long)smem <= most &&
+           cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess;
+}
+
+int fit_per_sm(const void *fn, int nt, int G, size_t smem)
+{
+    if (!allow_smem(fn, nt, G, smem))
         return 0;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, nt, smem) != cudaSuccess)
@@ -3697,9 +3705,10 @@ cudaError_t launch_merge(const MergeParams &p, int nt, cudaStream_t stream)
 {
     const size_t smem = merge_smem_bytes(p.n, p.G, nt);
     const void *fn = merge_fn(nt, p.G);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess)
-        return e;
+    if (!allow_smem(fn, nt, p.G, smem)) {
+        const cudaError_t e = cudaGetLastError();
+        return e != cudaSuccess ? e : cudaErrorInvalidValue;
+    }
     MergeParams q = p;
     q.chunk = merge_chunk_rows(p.n, p.G, nt);
     void *args[] = {&q};
