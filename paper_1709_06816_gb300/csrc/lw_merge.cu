@@ -47,10 +47,10 @@
 //   on condition  the bounds for outside cells may end a round that the cells
 //      themselves would not (equal values; inversions; values small against the
 //      largest, for single linkage).  When that costs a quarter as many merges of a
-//      chain as were proved (kTieGain, kTiePart), or half as many steps (see
-//      simulate), the merges are taken on condition: the new cells are computed
-//      and kept back, every CTA looks whether one of its own comes before a merge
-//      of the round, and barrier 3 tells which merges stand (settle).
+//      chain as were proved (kTieGain, kTiePart), or as many steps (see simulate),
+//      the merges are taken on condition: the new cells are computed and kept
+//      back, every CTA looks whether one of its own comes before a merge of the
+//      round, and barrier 3 tells which merges stand (settle).
 //   apply  behind barrier 2 (no CTA still reads the members' old cells): the new
 //      cells D(k, survivor) for every live k, a warp per 32 rows and up to 4
 //      survivors, all loads of an item in flight at once; then logs, caches
@@ -82,7 +82,7 @@
 // instructions was the largest stall after barriers, 3.7 of 11 cycles per
 // instruction outside them).  That is why no loop below is unrolled unless its
 // loads have to be in flight together: it took 5 to 9 % off every grid run (72 %
-// of the requests hit since, and the stall is 1.5 cycles per instruction).
+// of the requests hit since, and the stall is 1.4 cycles per instruction).
 //
 // Exact arithmetic: every product and sum of the update uses __fmul_rn /
 // __fadd_rn / __fsub_rn (never contracted into FMA), the coefficient
@@ -983,7 +983,7 @@ struct Flag {
 };
 
 template <int LK>
-__device__ __noinline__ void simulate_steps(Team &tm, int reach, int per, int &L_out, int &sure_out)
+__device__ __noinline__ void simulate_steps(Team &tm, int reach, int &L_out, int &sure_out)
 {
     const int lane = threadIdx.x & 31;
     const int m = tm.m;
@@ -1150,7 +1150,7 @@ __device__ __noinline__ void simulate_steps(Team &tm, int reach, int per, int &L
     if (!run(Flag<false>(), kTeam - 1)) {
         // from here on condition: the merged clusters' cells will be looked at
         sure = L;
-        if (per * reach >= L) {
+        if (reach >= L) {
 #pragma unroll
             for (int h = 0; h < 2; ++h)
                 lbv[h] = lv[h] && ((merged >> (lane + 32 * h)) & 1ull) ? thv : lbv[h];
@@ -1302,24 +1302,26 @@ __device__ __noinline__ void steps_program(Team &tm, int L)
 // that reason.  The bounds of the cells outside are weak there (single: a margin
 // of the matrix's largest value; centroid: up to a quarter of the height; zeros
 // and equal values anywhere), so the merges go on past them, on condition,
-// `reach` of them: twice as many as stood the last time (and 2).  That has to be
-// half of the proved ones (the look takes some 7 us of a round's 35), or all
-// where the cells outside are computed twice for it (twice: a CTA with several
-// chunks of rows).
-__device__ __noinline__ void simulate(Team &tm, int linkage, bool twice)
+// `reach` of them: twice as many as stood the last time (and 2).  They have to be
+// as many as the proved ones: the steps take a warp's time, the look some 7 us of a
+// round's 35, and some are put off again.  Single linkage, ms, ended at the bounds /
+// half as many / as many: n = 5500 on a 1/1024 grid 14.1 / 15.2 / 14.5, n = 16384
+// 55.6 / 52.9 / 50.0, n = 9000 conformer-like 42.1 / 13.5 / 14.7, n = 4000 points four
+// at a time 58.0 / 16.9 / 16.9; n = 3000 centroid 56.5 / 22.2 / 22.2.
+__device__ __noinline__ void simulate(Team &tm, int linkage)
 {
     const int lane = threadIdx.x & 31;
-    const int reach = tm.reach, per = twice ? 1 : 2;
+    const int reach = tm.reach;
     int L, sure;
     switch (linkage) {
-    case 0: simulate_steps<0>(tm, reach, per, L, sure); break;
-    case 1: simulate_steps<1>(tm, reach, per, L, sure); break;
-    case 2: simulate_steps<2>(tm, reach, per, L, sure); break;
-    case 3: simulate_steps<3>(tm, reach, per, L, sure); break;
-    case 4: simulate_steps<4>(tm, reach, per, L, sure); break;
-    default: simulate_steps<5>(tm, reach, per, L, sure); break;
+    case 0: simulate_steps<0>(tm, reach, L, sure); break;
+    case 1: simulate_steps<1>(tm, reach, L, sure); break;
+    case 2: simulate_steps<2>(tm, reach, L, sure); break;
+    case 3: simulate_steps<3>(tm, reach, L, sure); break;
+    case 4: simulate_steps<4>(tm, reach, L, sure); break;
+    default: simulate_steps<5>(tm, reach, L, sure); break;
     }
-    const bool tie = L > sure && per * (L - sure) >= sure;
+    const bool tie = L > sure && L - sure >= sure;
     if (!tie) {
         steps_undo(tm, L, sure, sure);
         L = sure;
@@ -2989,7 +2991,7 @@ __device__ void merge_job(const MergeParams &p, const int b, unsigned char *smem
                     }
                     sync_a();
                     if (warp == 0)
-                        simulate(sh.tm, linkage, Rmax > CH);
+                        simulate(sh.tm, linkage);
                 }
                 sync_a();
                 lap(ty.xs[3]);
