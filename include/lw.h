@@ -85,9 +85,9 @@ typedef struct lw_ctx lw_ctx;
  *   out          receives the handle (host pointer, must not be NULL).
  *   cuda_stream  a cudaStream_t on that device to issue all work on, or NULL
  *                for a stream owned by the context.
- * The context owns its device workspace (row-minimum keys 8n B, cluster
- * sizes 4n B, per-CTA exchange records, barrier words) and reuses it across
- * calls; it grows on demand.  Returns LW_ERR_INVALID_ARG for a bad device,
+ * The context owns its device workspace (cluster sizes 4n B, per-CTA exchange
+ * records, lists of 161 KB, barrier words) and the working layout of multi-CTA
+ * runs (LW_OPT_LAYOUT), and reuses them across calls; they grow on demand.  Returns LW_ERR_INVALID_ARG for a bad device,
  * LW_ERR_CUDA if the device cannot be used.
  */
 lw_status lw_create(lw_ctx **out, int device, void *cuda_stream);
@@ -164,7 +164,12 @@ lw_status lw_get_stats(lw_ctx *ctx, int64_t *stats, int count);
 /*
  * lw_set_option -- knobs of the context (value 0 = automatic / default):
  *   LW_OPT_GRID       CTAs of the persistent grid, 1..SM count (clamped to
- *                     what fits co-resident);
+ *                     what fits co-resident).  0: 1 up to 416 objects (1152 for
+ *                     centroid linkage), one per 32 objects up to 64, then one
+ *                     per 64 objects up to the SM count.  A 512-thread CTA fills
+ *                     an SM: contexts that run side by side share the device
+ *                     better with 1 (n = 2048, 64 contexts: 852 runs a second by
+ *                     default, 1037 with 1; a run by itself 2.5 ms and 12 ms);
  *   LW_OPT_TIMEOUT_MS bound of every device wait in milliseconds (default
  *                     5000);
  *   LW_OPT_TEST_SKIP_ARRIVE  failure-detection test hook: CTA `value` of a
@@ -183,9 +188,10 @@ lw_status lw_get_stats(lw_ctx *ctx, int64_t *stats, int count);
  *                     (default) or 1 the row-log layout -- a symmetric n x n
  *                     copy whose rows are rewritten whole, an n x n log of
  *                     each row's cells to later-merged slots and a stamp per
- *                     slot (8n^2 bytes held by the context, used when they
- *                     fit in half the free device memory, else the packed
- *                     triangle), so that every merge moves contiguous words;
+ *                     slot (8n^2 bytes held by the context, 134 MB at n = 4096,
+ *                     used when they fit in half the free device memory, else
+ *                     the packed triangle), so that every merge moves contiguous
+ *                     words;
  *                     2 the packed triangle (dist itself, no extra memory).
  *                     One-CTA runs always use the packed triangle.  Results
  *                     are the same either way;

@@ -76,7 +76,7 @@
 // barriers and about 13 merges per round) took 46.1 ms for n = 16384 average
 // linkage, 162.8 ms for single and 16.8 ms for n = 1968 (complete, on one CTA
 // then); selecting up to 64 members by a threshold and merging inside them takes
-// 25.2, 49.5 and 2.4 ms.  Next, the instructions themselves: each step's code
+// 24.7, 50.0 and 2.3 ms.  Next, the instructions themselves: each step's code
 // runs once or twice per round, so most of it is fetched anew every round
 // (n = 2000: 58 % of the SM's instruction cache requests hit, and waiting for
 // instructions was the largest stall after barriers, 3.7 of 11 cycles per

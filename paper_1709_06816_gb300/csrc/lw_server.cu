@@ -17,11 +17,13 @@
 // barrier for CTAs that another grid, or a one-CTA job, keeps off the device.
 // A request still in the queue can be cancelled.
 //
-// Large requests run with a modest grid (one CTA per 1024 objects): a merge
-// of the persistent kernel is bound by barrier and memory latency far more
-// than by the number of CTAs, so several large jobs side by side finish
-// sooner than the same jobs one after another over the whole device
-// (cooperative launches on different lanes run concurrently).
+// Requests run on one CTA up to 2048 objects and on one per 1024 above.  That is
+// a rule for a loaded server: a round is bound by latency, so many requests side
+// by side on few SMs each get more work through than the same ones after one
+// another on many (a burst of 48 mixed requests of up to 32768 objects: 186 ms;
+// one CTA per 768, 512 and 256 objects 204, 217 and 317).  A request that is
+// alone on the device takes longer for it (n = 2048: 12 ms on one CTA, 2.5 on 64).
+// (Cooperative launches on different lanes run concurrently.)
 
 #include "../../include/lw.h"
 #include "lw_internal.h"
@@ -151,8 +153,8 @@ struct lw_server {
     }
 
     // One CTA for up to 2048 objects (256 threads up to 512 objects, so that
-    // two small requests share an SM, else 512 -- the batch autotuner's
-    // finding on GB300); above that, 512-thread CTAs, one per 1024 objects.
+    // two small requests share an SM, else 512, as in the batch path's table);
+    // above that, 512-thread CTAs, one per 1024 objects.
     int grid_for(int64_t n) const
     {
         if (n <= 2048)
